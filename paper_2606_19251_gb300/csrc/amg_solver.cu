@@ -33,6 +33,7 @@
 
 #include "ctx.cuh"
 #include "wavefront.cuh"
+#include "tail.cuh"
 #include "setup_device.h"
 
 using namespace amg;
@@ -1461,6 +1462,91 @@ static void launch_coarse(amg_ctx *c, const T *b, T *u, cudaStream_t s) {
     }
 }
 
+// ---------------------------------------------------------------------------
+// the V-cycle's coarse tail as one dense operator (tail.cuh)
+// ---------------------------------------------------------------------------
+// The tail of the smoother in use (none with Chebyshev or without a level
+// that fits).
+static DevTail *tail_of(amg_ctx *c) {
+    if (c->smoother == AMG_SMOOTHER_CHEB) return nullptr;
+    DevTail *t = &c->tail[c->smoother == AMG_SMOOTHER_GNN ? 1 : 0];
+    return t->level >= 0 ? t : nullptr;
+}
+
+// First level of the tail: at most kTailRows rows, at least one smoothed
+// level in it, its level vectors within a CTA's shared memory and the
+// coarsest solves of its columns affordable; -1 if there is none.
+static int tail_level(const amg_ctx *c) {
+    const int nlev = static_cast<int>(c->host.size());
+    const double nL = c->host.back().A.n_rows;
+    size_t rows = nL;
+    int best = -1;
+    for (int l = nlev - 2; l >= 0 && nlev - l <= kTailMaxLevels; --l) {
+        const int n = c->host[l].A.n_rows;
+        rows += n;
+        if (n > kTailRows || 3 * rows * kTailCols * sizeof(double) > kTailSmem || n * nL * nL > kTailCoarseWork) break;
+        best = l;
+    }
+    return best;
+}
+
+template <class T>
+static int build_tail(amg_ctx *c, int sm, cudaStream_t s) {
+    DevTail &t = c->tail[sm];
+    const int nlev = static_cast<int>(c->lev.size());
+    TailArgs<T> a{};
+    a.nlev = nlev - t.level;
+    a.nu1 = c->opt.nu1;
+    a.nu2 = c->opt.nu2;
+    a.pinv = sm;
+    a.ld = t.ld;
+    a.Linv = c->Linv;
+    a.LinvT = c->LinvT;
+    a.B = static_cast<T *>(t.B);
+    int off = 0;
+    for (int k = 0; k < a.nlev; ++k) {
+        const DevLevel &L = c->lev[t.level + k];
+        TailLevel<T> &D = a.lev[k];
+        D.n = L.n;
+        D.off = off;
+        off += 3 * L.n * kTailCols;
+        if (k == a.nlev - 1) break;
+        D.A = {L.A.rp, L.A.col, mvals<T>(L.A)};
+        D.P = {L.P.rp, L.P.col, mvals<T>(L.P)};
+        D.R = {L.R.rp, L.R.col, mvals<T>(L.R)};
+        D.m = sm ? qvals<T>(L) : jvals<T>(L);
+    }
+    using V = typename std::conditional<std::is_same<T, float>::value, FloatPair, double>::type;
+    const size_t smem = static_cast<size_t>(off) * sizeof(V);
+    CK(cudaFuncSetAttribute(k_tail_build<T, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kTailSmem)));
+    k_tail_build<T, V><<<(c->lev[t.level].n + kTailCols - 1) / kTailCols, kTailThreads, smem, s>>>(a); AMG_COUNT();
+    CKL("V-cycle tail");
+    t.ok = true;
+    return AMG_OK;
+}
+
+// Make the tail of the smoother in use current before V-cycles on s.  The
+// smoother's values change with the coefficients; B is re-formed at the next
+// V-cycle that needs it (or with host-given coefficients, in that call).
+static int ensure_tail(amg_ctx *c, cudaStream_t s) {
+    c->use_tail = true;
+    DevTail *t = tail_of(c);
+    if (!t || t->ok) return AMG_OK;
+    const int sm = c->smoother == AMG_SMOOTHER_GNN ? 1 : 0;
+    return c->opt.precision == AMG_FP64 ? build_tail<double>(c, sm, s) : build_tail<float>(c, sm, s);
+}
+
+template <class T>
+static void launch_tail(const DevTail &t, int n, const T *b, T *e, cudaStream_t s) {
+    const T *B = static_cast<const T *>(t.B);
+    const dim3 g((n + kBlock / 32 - 1) / (kBlock / 32));
+    const int loads = (t.ld * static_cast<int>(sizeof(T)) + 511) / 512;   // 16-byte loads per lane and row
+    if (loads <= 2) launch_pdl(k_tail_apply<T, 2>, g, dim3(kBlock), 0, s, n, t.ld, B, b, e);
+    else if (loads <= 4) launch_pdl(k_tail_apply<T, 4>, g, dim3(kBlock), 0, s, n, t.ld, B, b, e);
+    else if (loads <= 8) launch_pdl(k_tail_apply<T, 8>, g, dim3(kBlock), 0, s, n, t.ld, B, b, e);
+    else launch_pdl(k_tail_apply<T, 16>, g, dim3(kBlock), 0, s, n, t.ld, B, b, e);
+}
+
 // Smoothing on a latency-optimised level: every pseudo-inverse sweep is one
 // pass with M A (ping-pong between cur and alt); the first sweep from zero
 // also keeps w = M b.  Jacobi fuses its first two sweeps from zero.
@@ -1515,6 +1601,10 @@ static T *vcycle_level(amg_ctx *c, int l, cudaStream_t s) {
     const int nlev = static_cast<int>(c->lev.size());
     if (l == nlev - 1) {
         launch_coarse<T>(c, b, u, s);
+        return u;
+    }
+    if (c->use_tail && tail_of(c) && tail_of(c)->level == l) {
+        launch_tail<T>(*tail_of(c), L.n, b, u, s);
         return u;
     }
     T *bc = reinterpret_cast<T *>(c->lev[l + 1].vb);
@@ -1692,7 +1782,8 @@ static int ensure_graph(amg_ctx *c) {
 template <class T>
 static int solve_staged(amg_ctx *c, cudaStream_t s, double tol, int *n_vc, double *hist) {
     const int max_iter = c->opt.max_iter;
-    int rc = ensure_graph<T>(c);
+    int rc = ensure_tail(c, s);
+    if (!rc) rc = ensure_graph<T>(c);
     if (rc) return rc;
     enqueue_init<T>(c, s, tol, max_iter);
     CKL("solve init launch");
@@ -1708,7 +1799,8 @@ static int solve_staged(amg_ctx *c, cudaStream_t s, double tol, int *n_vc, doubl
         // from the current iterate (Sec. 3.3 fallback)
         c->smoother = AMG_SMOOTHER_JACOBI;
         c->last_rerouted = 1;
-        rc = ensure_graph<T>(c);
+        rc = ensure_tail(c, s);
+        if (!rc) rc = ensure_graph<T>(c);
         if (rc) return rc;
         launch_pdl(k_state_continue, dim3(1), dim3(1), 0, s, c->state);
         const SolveGraph &GJ = c->sgraph[AMG_SMOOTHER_JACOBI + 3 * c->opt.outer];
@@ -1749,6 +1841,7 @@ static void free_device(amg_ctx *c) {
     c->lev.clear();
     c->nL = 0;
     c->have_q = false;
+    for (DevTail &t : c->tail) t = DevTail{};
 }
 
 static void layout_mat(Planner &pl, DevMat &m, const HostCSR &h) {
@@ -1857,6 +1950,16 @@ static void layout(amg_ctx *c, Planner &pl) {
     c->Ldense = pl.take<double>(static_cast<size_t>(nL) * nL);
     c->Linv = pl.take<double>(static_cast<size_t>(nL) * nL);
     c->LinvT = pl.take<double>(static_cast<size_t>(nL) * nL);
+    const int tl = tail_level(c);
+    for (DevTail &t : c->tail) {
+        t = DevTail{};
+        if (tl < 0) continue;
+        const int n = c->host[tl].A.n_rows;
+        const size_t tb = c->opt.precision == AMG_FP64 ? sizeof(double) : sizeof(float);
+        t.level = tl;
+        t.ld = static_cast<int>((n * tb + 511) / 512 * 512 / tb);
+        t.B = pl.take<char>(tb * n * t.ld);
+    }
     const int n0 = c->host[0].A.n_rows;
     c->ell_ptr = pl.take<int>(c->h_ell_ptr.size());
     c->ell_row = pl.take<int>(c->h_ell_row.size());
@@ -1995,6 +2098,8 @@ static int upload(amg_ctx *c) {
     CK(cudaFuncSetAttribute(k_coarse<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 8 * kMaxCoarseDense));
     k_tri_inverse<<<grid_for(nL), kBlock, 0, s>>>(nL, c->Ldense, c->Linv, c->LinvT); AMG_COUNT();
     CKL("hierarchy setup kernels");
+    c->smoother = AMG_SMOOTHER_JACOBI;
+    if ((prc = ensure_tail(c, s))) return prc;
     int flag = 0;
     std::vector<int> wide(nlev, 0);
     CK(cudaMemcpyAsync(&flag, c->dflag, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -2243,8 +2348,12 @@ int amg_set_jacobi(amg_ctx *c, double omega) {
             k_jacobi_vals<<<grid_for(L.n), kBlock, 0, c->stream>>>(L.n, L.diag, omega, L.j64, L.j32); AMG_COUNT();
         }
         CKL("jacobi values");
-        CK(cudaStreamSynchronize(c->stream));
+        c->tail[0].ok = false;
         c->jac_omega = omega;
+        c->smoother = AMG_SMOOTHER_JACOBI;
+        const int rc = ensure_tail(c, c->stream);
+        if (rc) return rc;
+        CK(cudaStreamSynchronize(c->stream));
     }
     c->smoother = AMG_SMOOTHER_JACOBI;
     return AMG_OK;
@@ -2379,6 +2488,7 @@ int set_coeffs_device(amg_ctx *c, const double *coef, int n_rows, cudaStream_t s
         c->q_nodes = false;
         c->q64_stale = false;
     }
+    c->tail[1].ok = false;
     CKL("assemble pseudo-inverse");
     // the solve kernels fetch matrix values ahead of their grid-dependency
     // wait: finish writing them before any of those kernels is launched
@@ -2399,6 +2509,7 @@ int amg_set_coeffs(amg_ctx *c, const double *coef, int n_rows) {
         return ctx_fail(c, "need one coefficient row per smoothed level"), AMG_ERR_ARG;
     CK(cudaSetDevice(c->opt.device));
     int rc = set_coeffs_device(c, coef, n_rows, c->stream);
+    if (!rc) rc = ensure_tail(c, c->stream);
     if (rc) return rc;
     CK(cudaStreamSynchronize(c->stream));
     return AMG_OK;
@@ -2447,7 +2558,11 @@ int amg_set_node_coeffs(amg_ctx *c, const double *coef, long long n_values) {
     c->have_q = true;
     c->q_nodes = true;   // the wavefront chains read the stored values
     c->q64_stale = false;
+    c->tail[1].ok = false;
     c->smoother = AMG_SMOOTHER_GNN;
+    const int rc = ensure_tail(c, s);
+    if (rc) return rc;
+    CK(cudaStreamSynchronize(s));
     return AMG_OK;
 }
 
@@ -2538,6 +2653,20 @@ int amg_solve_device(amg_ctx *c, const double *d_b, double *d_x, double rtol, vo
     return rc;
 }
 
+// As ensure_tail for a caller's stream.  A V-cycle being captured steps
+// through the levels instead: its replays follow later coefficient changes,
+// which rewrite the levels' values in place but re-form the tail's operator
+// only at the next V-cycle call.
+static int ensure_vcycle_tail(amg_ctx *c, cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        c->use_tail = false;
+        return AMG_OK;
+    }
+    return ensure_tail(c, s);
+}
+
 int amg_vcycle_device(amg_ctx *c, const double *d_r, double *d_e, void *stream) {
     if (!c) return AMG_ERR_ARG;
     c->err.clear();
@@ -2546,6 +2675,8 @@ int amg_vcycle_device(amg_ctx *c, const double *d_r, double *d_e, void *stream) 
     if (rc) return rc;
     CK(cudaSetDevice(c->opt.device));
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    rc = ensure_vcycle_tail(c, s);
+    if (rc) return rc;
     const int n0 = c->lev[0].n;
     if (c->opt.precision == AMG_FP64) {
         CK(cudaMemcpyAsync(c->lev[0].vb, d_r, sizeof(double) * n0, cudaMemcpyDeviceToDevice, s));
@@ -2785,6 +2916,8 @@ double vcycle_bytes_level(const amg_ctx *c, int l, int tb) {
     const DevLevel &L = c->lev[l];
     const int nlev = static_cast<int>(c->lev.size());
     if (l == nlev - 1) return 8.0 * c->nL * c->nL + 2.0 * tb * c->nL;
+    if (tail_of(const_cast<amg_ctx *>(c)) && tail_of(const_cast<amg_ctx *>(c))->level == l)
+        return 1.0 * tb * L.n * L.n + 2.0 * tb * L.n;   // the coarse tail's dense operator
     const bool cheb = (c->smoother == AMG_SMOOTHER_CHEB);
     const int nu1 = cheb ? (c->opt.nu1 > 0 ? 1 : 0) : c->opt.nu1;
     const int nu2 = cheb ? (c->opt.nu2 > 0 ? 1 : 0) : c->opt.nu2;
@@ -2909,6 +3042,10 @@ int amg_kernel_launch(amg_ctx *c, int which, int level, int reps, void *stream, 
         return ctx_fail(c, "bad level or repetition count"), AMG_ERR_ARG;
     CK(cudaSetDevice(c->opt.device));
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (which == AMG_K_VCYCLE && (c->smoother != AMG_SMOOTHER_GNN || c->have_q)) {
+        const int rc = ensure_vcycle_tail(c, s);
+        if (rc) return rc;
+    }
     if (c->opt.precision == AMG_FP64) return kernel_launch<double>(c, which, level, reps, s, bytes);
     return kernel_launch<float>(c, which, level, reps, s, bytes);
 }

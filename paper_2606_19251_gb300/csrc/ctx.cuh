@@ -59,6 +59,14 @@ struct WfPlan {
     std::vector<int> lohi;                     // 2 x nblk
 };
 
+// Dense operator of the V-cycle's coarse tail (tail.cuh) for one smoother.
+struct DevTail {
+    int level = -1;                            // first level of the tail, or -1
+    int ld = 0;                                // row stride of B (entries)
+    void *B = nullptr;                         // in the V-cycle precision
+    bool ok = false;                           // B belongs to the smoother's current values
+};
+
 enum : int { kRunning = 1, kStalled = 2 };
 
 struct SolveState {
@@ -134,6 +142,8 @@ struct amg_ctx {
     bool q_nodes = false;                      // Q^-1 from per-node coefficients (stored values only)
     bool q64_stale = false;                    // only the FP32 Q^-1 was assembled (coefficients kept in wcoef)
     std::vector<amg::WfPlan> wfplan;           // per level
+    amg::DevTail tail[2];                      // per smoother (Jacobi, pseudo-inverse)
+    bool use_tail = false;                     // the V-cycle being enqueued applies the tail's dense operator
 };
 
 namespace amg {

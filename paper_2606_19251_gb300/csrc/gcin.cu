@@ -1351,6 +1351,7 @@ int gnn_predict_coeffs(amg_ctx *c, double *c_out) {
     g_launches.fetch_add(g->exec_kernels);
     c->have_q = true;
     c->q_nodes = false;
+    c->tail[1].ok = false;                         // re-formed by the next V-cycle
     c->q64_stale = c->opt.precision != AMG_FP64;   // the graph assembled the FP32 values only
     c->smoother = AMG_SMOOTHER_GNN;
     int dflag = 0;
