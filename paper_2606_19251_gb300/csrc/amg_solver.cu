@@ -1735,6 +1735,56 @@ static void free_graph(SolveGraph &G) {
     G = SolveGraph{};
 }
 
+static void free_vgraph(VcycleGraph &G) {
+    if (G.exec) cudaGraphExecDestroy(G.exec);
+    G = VcycleGraph{};
+}
+
+// One V-cycle on lev[0].vb for amg_vcycle_device; returns the result's
+// buffer.  A caller's Krylov loop repeats it, and as single launches it is
+// bound by the host (1.35 us each on a Grace core, against 0.6 to 0.9 us per
+// dependent kernel of a graph and 1 us for launching one): from the second
+// call on it is one graph launch (9k rows: 50.6 -> 34.4 us a call; 280k rows,
+// bound by the device, 137.4 -> 135.3).  The first call launches the kernels, so a
+// V-cycle that is not repeated pays for no capture; so does a caller's own
+// capture (use_tail is off), and a capture that fails leaves the kernels.
+template <class T>
+static T *vcycle_repeat(amg_ctx *c, cudaStream_t s) {
+    VcycleGraph &G = c->vgraph[c->smoother];
+    if (G.version != c->hier_version || G.q_nodes != static_cast<int>(c->q_nodes)) {
+        free_vgraph(G);
+        G.version = c->hier_version;
+        G.q_nodes = static_cast<int>(c->q_nodes);
+    }
+    if (!c->use_tail || c->opt.fused_sweeps) return vcycle_level<T>(c, 0, s);
+    if (!G.exec) {
+        if (++G.calls != 2) return vcycle_level<T>(c, 0, s);
+        // another stream of this thread may be under capture: ours must not disturb it
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        const long long before = g_launches.load();
+        cudaGraph_t g = nullptr;
+        cudaError_t e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeRelaxed);
+        if (e == cudaSuccess) {
+            G.e = vcycle_level<T>(c, 0, c->stream);
+            e = cudaStreamEndCapture(c->stream, &g);
+        }
+        G.kernels = g_launches.load() - before;
+        g_launches.fetch_sub(G.kernels);
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&G.exec, g, 0);
+        if (g) cudaGraphDestroy(g);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            G.exec = nullptr;
+            return vcycle_level<T>(c, 0, s);
+        }
+    }
+    if (cudaGraphLaunch(G.exec, s) != cudaSuccess) return vcycle_level<T>(c, 0, s);
+    g_launches.fetch_add(G.kernels);
+    return static_cast<T *>(G.e);
+}
+
 // Build (once per hierarchy and smoother) the whole-solve graph.
 template <class T>
 static int ensure_graph(amg_ctx *c) {
@@ -1835,6 +1885,7 @@ static void free_device(amg_ctx *c) {
     c->ell_val = nullptr;
     train_bufs_free(c);
     for (auto &G : c->sgraph) free_graph(G);
+    for (auto &G : c->vgraph) free_vgraph(G);
     if (c->arena) cudaFree(c->arena);
     c->arena = nullptr;
     c->arena_bytes = 0;
@@ -2381,6 +2432,7 @@ int amg_set_chebyshev(amg_ctx *c, int degree) {
     }
     if (degree != c->cheb_degree) {   // the captured graphs hold the polynomial's steps
         for (int o = 0; o < 2; ++o) free_graph(c->sgraph[AMG_SMOOTHER_CHEB + 3 * o]);
+        free_vgraph(c->vgraph[AMG_SMOOTHER_CHEB]);
         c->cheb_degree = degree;
     }
     c->smoother = AMG_SMOOTHER_CHEB;
@@ -2680,11 +2732,11 @@ int amg_vcycle_device(amg_ctx *c, const double *d_r, double *d_e, void *stream) 
     const int n0 = c->lev[0].n;
     if (c->opt.precision == AMG_FP64) {
         CK(cudaMemcpyAsync(c->lev[0].vb, d_r, sizeof(double) * n0, cudaMemcpyDeviceToDevice, s));
-        double *e = vcycle_level<double>(c, 0, s);
+        double *e = vcycle_repeat<double>(c, s);
         CK(cudaMemcpyAsync(d_e, e, sizeof(double) * n0, cudaMemcpyDeviceToDevice, s));
     } else {
         launch_pdl(k_convert<double, float>, dim3(grid_for(n0)), dim3(kBlock), 0, s, n0, d_r, reinterpret_cast<float *>(c->lev[0].vb));
-        float *e = vcycle_level<float>(c, 0, s);
+        float *e = vcycle_repeat<float>(c, s);
         launch_pdl(k_convert<float, double>, dim3(grid_for(n0)), dim3(kBlock), 0, s, n0, e, d_e);
     }
     CKL("vcycle");

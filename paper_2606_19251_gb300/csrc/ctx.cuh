@@ -95,6 +95,17 @@ struct SolveGraph {
     int q_nodes = -1;    // the pseudo-inverse source the captured chains use
 };
 
+// One V-cycle of amg_vcycle_device as a CUDA graph, captured at the second
+// call with the same hierarchy and smoother.
+struct VcycleGraph {
+    cudaGraphExec_t exec = nullptr;
+    long long version = -1;
+    int q_nodes = -1;
+    int calls = 0;
+    void *e = nullptr;          // the buffer that holds the result
+    long long kernels = 0;
+};
+
 struct GcinEngine;
 void gcin_engine_free(GcinEngine *e);
 
@@ -127,6 +138,7 @@ struct amg_ctx {
     long long hier_version = 0;                // bumped by every hierarchy upload
     void *train = nullptr;                     // training (adjoint) buffers, created on demand
     amg::SolveGraph sgraph[6];                 // per smoother + 3 x outer iteration
+    amg::VcycleGraph vgraph[3];                // per smoother
     int cheb_degree = 3;
     long long cheb_version = -1;               // hierarchy version the Chebyshev intervals belong to
     double *pcg = nullptr;                     // conjugate gradients: r, r_prev, z, p, q (n_0 each)
