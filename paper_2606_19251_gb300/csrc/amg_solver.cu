@@ -264,30 +264,6 @@ __global__ void k_dinv_vals(int n, const double *__restrict__ diag, double *__re
     d32[i] = static_cast<float>(v);
 }
 
-// (M A) values from the pair list in FP32, for the FP32 V-cycle (GB300's FP64
-// pipe is narrow; the FP32 V-cycle needs only the FP32 product)
-__global__ void k_assemble_ma32(int nnz, const int *__restrict__ pp, const int *__restrict__ pq_p,
-                                const int *__restrict__ pq_q, const float *__restrict__ q32,
-                                const float *__restrict__ a32, float *__restrict__ ma32) {
-    const int e = blockIdx.x * kBlock + threadIdx.x;
-    if (e >= nnz) return;
-    float acc = 0.f;
-    for (int t = pp[e]; t < pp[e + 1]; ++t) acc = fmaf(q32[pq_p[t]], a32[pq_q[t]], acc);
-    ma32[e] = acc;
-}
-
-// (M A) values from the pair list (FP64), with the V-cycle-precision copy
-__global__ void k_assemble_ma(int nnz, const int *__restrict__ pp, const int *__restrict__ pq_p,
-                              const int *__restrict__ pq_q, const double *__restrict__ q64,
-                              const double *__restrict__ a64, double *__restrict__ ma64, float *__restrict__ ma32) {
-    const int e = blockIdx.x * kBlock + threadIdx.x;
-    if (e >= nnz) return;
-    double acc = 0.0;
-    for (int t = pp[e]; t < pp[e + 1]; ++t) acc = fma(q64[pq_p[t]], a64[pq_q[t]], acc);
-    ma64[e] = acc;
-    ma32[e] = static_cast<float>(acc);
-}
-
 // u = (omega/a_ii) b  (first Jacobi sweep from u = 0)
 template <class T>
 __global__ void k_scale(int n, const T *__restrict__ jac, const T *__restrict__ b, T *__restrict__ u) {
@@ -782,25 +758,10 @@ __global__ void k_pinv_basis(int n, const int *__restrict__ rp, const int *__res
     }
 }
 
-// Q^-1 values on A's pattern from c = (d0, d1, d2, o1, o2) (Sec. 3.1):
-// q_ii = (d0 + d1 x + d2 x^2) bw, q_ij = (o1 x + o2 x^2) bw, in FP64 with the
-// polynomial evaluated as d0 + d1 x + (d2 x) x, uncontracted.
-__global__ void k_assemble_q(int nnz, const unsigned char *__restrict__ isd, const double *__restrict__ bx,
-                             const double *__restrict__ bw, double c0, double c1, double c2, double c3, double c4,
-                             double *__restrict__ q64, float *__restrict__ q32) {
-    const int p = blockIdx.x * kBlock + threadIdx.x;
-    if (p >= nnz) return;
-    const double x = bx[p];
-    const double f = isd[p] ? __dadd_rn(__dadd_rn(c0, __dmul_rn(c1, x)), __dmul_rn(__dmul_rn(c2, x), x))
-                            : __dadd_rn(__dmul_rn(c3, x), __dmul_rn(__dmul_rn(c4, x), x));
-    const double q = __dmul_rn(f, bw[p]);
-    q64[p] = q;
-    q32[p] = static_cast<float>(q);
-}
-
 // Q^-1 values with one coefficient row per node (cn: n x 5): the diagonal of
 // row i from node i's (d0, d1, d2), an off-diagonal entry (i, j) from the mean
-// of nodes i's and j's (o1, o2) (a symmetric Q^-1); arithmetic as k_assemble_q.
+// of nodes i's and j's (o1, o2) (a symmetric Q^-1); the polynomial as d0 + d1 x + (d2 x) x,
+// uncontracted.
 __global__ void k_assemble_q_nodes(int n, const int *__restrict__ rp, const int *__restrict__ col,
                                    const unsigned char *__restrict__ isd, const double *__restrict__ bx,
                                    const double *__restrict__ bw, const double *__restrict__ cn,
@@ -827,8 +788,8 @@ __global__ void k_assemble_q_nodes(int n, const int *__restrict__ rp, const int 
 // Every smoothed level's Q^-1 (and then M A) in one launch each, with the
 // coefficients read from device memory (the FP32 network output, widened to
 // FP64 exactly as the host path does): a thread finds its level from the
-// cumulative entry offsets; the arithmetic per entry is k_assemble_q's (and
-// k_assemble_ma / k_assemble_ma32's).
+// cumulative entry offsets.  q_ii = (d0 + d1 x + d2 x^2) bw, q_ij = (o1 x +
+// o2 x^2) bw, the polynomial as d0 + d1 x + (d2 x) x, uncontracted.
 constexpr int kAsmMaxLevels = 32;
 struct AsmQ {
     int nlev;
@@ -840,6 +801,36 @@ struct AsmQ {
     float *q32[kAsmMaxLevels];
     int row[kAsmMaxLevels];                   // coefficient row of the level
 };
+
+// Coefficient rows given by the host, as a kernel argument.
+struct AsmCoef {
+    double c[kAsmMaxLevels][5];
+};
+
+// Q^-1 of every level in L from host coefficients, in FP64 with the FP32
+// copy, and the wavefront chains' coefficient rows (one launch for all
+// levels: per level they were 2 to 3 launches and a host copy, and
+// amg_loss_grad sets new coefficients in every call).
+__global__ void k_assemble_q_host(AsmQ L, const __grid_constant__ AsmCoef C, const double *__restrict__ scal,
+                                  float *__restrict__ wcoef) {
+    const long long p = static_cast<long long>(blockIdx.x) * kBlock + threadIdx.x;
+    if (p < L.nlev) {
+        const int l = L.row[p];
+        for (int k = 0; k < 5; ++k) wcoef[8 * l + k] = static_cast<float>(C.c[p][k]);
+        wcoef[8 * l + 5] = static_cast<float>(1.0 / scal[l]);
+    }
+    if (p >= L.start[L.nlev]) return;
+    int l = 0;
+    while (p >= L.start[l + 1]) ++l;
+    const long long e = p - L.start[l];
+    const double *c = C.c[l];
+    const double x = L.bx[l][e];
+    const double f = L.isd[l][e] ? __dadd_rn(__dadd_rn(c[0], __dmul_rn(c[1], x)), __dmul_rn(__dmul_rn(c[2], x), x))
+                                 : __dadd_rn(__dmul_rn(c[3], x), __dmul_rn(__dmul_rn(c[4], x), x));
+    const double q = __dmul_rn(f, L.bw[l][e]);
+    L.q64[l][e] = q;
+    L.q32[l][e] = static_cast<float>(q);
+}
 
 // mode 0: the FP32 V-cycle's values only, in FP32 from the FP32 basis (the
 // FP64 values are assembled when something asks for them); mode 1: both from
@@ -888,7 +879,9 @@ __global__ void k_wf_coef(int nlev, const float *__restrict__ dc, const double *
     wcoef[8 * l + 5] = static_cast<float>(1.0 / scal[l]);
 }
 
-// fp64 != 0: FP64 products with the FP32 copy (FP64 V-cycle); else FP32 only
+// (M A) values from the pair lists.  fp64 != 0: FP64 products with the FP32
+// copy (FP64 V-cycle); else FP32 only (GB300's FP64 pipe is narrow; the FP32
+// V-cycle needs only the FP32 product)
 __global__ void k_assemble_ma_all(AsmMA M, int fp64) {
     const long long p = static_cast<long long>(blockIdx.x) * kBlock + threadIdx.x;
     if (p >= M.start[M.nlev]) return;
@@ -1453,10 +1446,48 @@ __global__ void __launch_bounds__(32) k_coarse_warp(int n, const double *__restr
     if (i < n) u[i] = static_cast<T>(x);
 }
 
+// Coarsest solve for 33 to 64 rows (the default coarsening stops at 64): a
+// warp per row and each lane's factor entries in registers before the
+// grid-dependency wait, so that only b's loads and two warp sums follow it.
+// The sums run in k_coarse's order (the same bits).
+template <class T>
+__global__ void __launch_bounds__(1024) k_coarse_64(int n, const double *__restrict__ Linv,
+                                                    const double *__restrict__ LinvT, const T *__restrict__ b,
+                                                    T *__restrict__ u) {
+    __shared__ double sb[64], sy[64];
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    double m[2][2], mt[2][2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int i = warp + 32 * h, j = lane + 32 * k;
+            m[h][k] = (i < n && j <= i) ? Linv[i * n + j] : 0.0;
+            mt[h][k] = (i < n && j >= i && j < n) ? LinvT[i * n + j] : 0.0;
+        }
+    pdl_wait_and_release();
+    if (threadIdx.x < 64) sb[threadIdx.x] = threadIdx.x < n ? static_cast<double>(b[threadIdx.x]) : 0.0;
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const double v = warp_sum(fma(m[h][1], sb[lane + 32], m[h][0] * sb[lane]));
+        if (lane == 0) sy[warp + 32 * h] = v;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int i = warp + 32 * h;
+        const double v = warp_sum(fma(mt[h][1], sy[lane + 32], mt[h][0] * sy[lane]));
+        if (lane == 0 && i < n) u[i] = static_cast<T>(v);
+    }
+}
+
 template <class T>
 static void launch_coarse(amg_ctx *c, const T *b, T *u, cudaStream_t s) {
     if (c->nL <= 32) {
         launch_pdl(k_coarse_warp<T>, dim3(1), dim3(32), 0, s, c->nL, c->Linv, c->LinvT, b, u);
+    } else if (c->nL <= 64) {
+        launch_pdl(k_coarse_64<T>, dim3(1), dim3(1024), 0, s, c->nL, c->Linv, c->LinvT, b, u);
     } else {
         launch_pdl(k_coarse<T>, dim3(1), dim3(kBlock), 2 * sizeof(double) * c->nL, s, c->nL, c->Linv, c->LinvT, b, u);
     }
@@ -2455,9 +2486,9 @@ namespace amg {
 // coefficients in device memory (G x 5 FP32, level order) without a host
 // round trip; the caller validates the coefficients after its own
 // synchronisation and selects the smoother.
-static AsmQ asm_q_levels(const amg_ctx *c) {
+static AsmQ asm_q_levels(const amg_ctx *c, int l0, int l1) {
     AsmQ Q{};
-    for (int l = 0; l + 1 < static_cast<int>(c->lev.size()); ++l) {
+    for (int l = l0; l < l1; ++l) {
         const DevLevel &L = c->lev[l];
         const int k = Q.nlev++;
         Q.start[k + 1] = Q.start[k] + L.A.nnz;
@@ -2473,31 +2504,35 @@ static AsmQ asm_q_levels(const amg_ctx *c) {
     return Q;
 }
 
+static AsmMA asm_ma_levels(const amg_ctx *c, int l0, int l1) {
+    AsmMA M{};
+    for (int l = l0; l < l1; ++l) {
+        const DevLevel &L = c->lev[l];
+        if (!L.fast) continue;
+        const int j = M.nlev++;
+        M.start[j + 1] = M.start[j] + L.MA.nnz;
+        M.pp[j] = L.pp;
+        M.pq_p[j] = L.pq_p;
+        M.pq_q[j] = L.pq_q;
+        M.q32[j] = L.q32;
+        M.a32[j] = L.A.v32;
+        M.ma32[j] = L.MA.v32;
+        M.q64[j] = L.q64;
+        M.a64[j] = L.A.v64;
+        M.ma64[j] = L.MA.v64;
+    }
+    return M;
+}
+
 int enqueue_coeff_assembly(amg_ctx *c, const float *d_coef, cudaStream_t s) {
     const int nlev = static_cast<int>(c->lev.size());
     if (nlev - 1 > kAsmMaxLevels) return ctx_fail(c, "too many levels for the batched assembly"), AMG_ERR_ARG;
     // all levels' Q^-1 in one launch, then all latency-optimised levels' M A;
     // the FP32 V-cycle needs only the FP32 values (the coefficients stay in
     // wcoef for an FP64 assembly on request)
-    const AsmQ Q = asm_q_levels(c);
+    const AsmQ Q = asm_q_levels(c, 0, nlev - 1);
     const bool fp64 = c->opt.precision == AMG_FP64;
-    AsmMA M{};
-    for (int l = 0; l < nlev - 1; ++l) {
-        const DevLevel &L = c->lev[l];
-        if (L.fast) {
-            const int j = M.nlev++;
-            M.start[j + 1] = M.start[j] + L.MA.nnz;
-            M.pp[j] = L.pp;
-            M.pq_p[j] = L.pq_p;
-            M.pq_q[j] = L.pq_q;
-            M.q32[j] = L.q32;
-            M.a32[j] = L.A.v32;
-            M.ma32[j] = L.MA.v32;
-            M.q64[j] = L.q64;
-            M.a64[j] = L.A.v64;
-            M.ma64[j] = L.MA.v64;
-        }
-    }
+    const AsmMA M = asm_ma_levels(c, 0, nlev - 1);
     if (Q.nlev > 0 && Q.start[Q.nlev] > 0) {
         k_assemble_q_all<<<grid_for(Q.start[Q.nlev]), kBlock, 0, s>>>(Q, d_coef, 5, fp64 ? 1 : 0); AMG_COUNT();
     }
@@ -2512,39 +2547,29 @@ int enqueue_coeff_assembly(amg_ctx *c, const float *d_coef, cudaStream_t s) {
     return AMG_OK;
 }
 
-int set_coeffs_device(amg_ctx *c, const double *coef, int n_rows, cudaStream_t s) {
+int set_coeffs_device(amg_ctx *c, const double *coef, cudaStream_t s, bool sync) {
     const int nlev = static_cast<int>(c->lev.size());
-    for (int l = 0; l < nlev - 1; ++l) {
-        const DevLevel &L = c->lev[l];
-        const double *q = coef + 5 * l;
-        for (int k = 0; k < 5; ++k)
-            if (!std::isfinite(q[k])) return ctx_fail(c, "non-finite coefficient"), AMG_ERR_ARG;
-        k_assemble_q<<<grid_for(L.A.nnz), kBlock, 0, s>>>(L.A.nnz, L.isd, L.bx, L.bw, q[0], q[1], q[2], q[3],
-                                                          q[4], L.q64, L.q32); AMG_COUNT();
-        if (L.fast && c->opt.precision == AMG_FP64) {
-            k_assemble_ma<<<grid_for(L.MA.nnz), kBlock, 0, s>>>(L.MA.nnz, L.pp, L.pq_p, L.pq_q, L.q64, L.A.v64,
-                                                                L.MA.v64, L.MA.v32); AMG_COUNT();
-        } else if (L.fast) {
-            k_assemble_ma32<<<grid_for(L.MA.nnz), kBlock, 0, s>>>(L.MA.nnz, L.pp, L.pq_p, L.pq_q, L.q32, L.A.v32,
-                                                                  L.MA.v32); AMG_COUNT();
+    for (int k = 0; k < 5 * (nlev - 1); ++k)
+        if (!std::isfinite(coef[k])) return ctx_fail(c, "non-finite coefficient"), AMG_ERR_ARG;
+    for (int l0 = 0; l0 < nlev - 1; l0 += kAsmMaxLevels) {
+        const int l1 = std::min(nlev - 1, l0 + kAsmMaxLevels);
+        AsmCoef C{};
+        std::copy(coef + 5 * l0, coef + 5 * l1, &C.c[0][0]);
+        const AsmQ Q = asm_q_levels(c, l0, l1);
+        k_assemble_q_host<<<grid_for(std::max<long long>(Q.start[Q.nlev], Q.nlev)), kBlock, 0, s>>>(Q, C, c->scal, c->wcoef); AMG_COUNT();
+        const AsmMA M = asm_ma_levels(c, l0, l1);
+        if (M.nlev > 0 && M.start[M.nlev] > 0) {
+            k_assemble_ma_all<<<grid_for(M.start[M.nlev]), kBlock, 0, s>>>(M, c->opt.precision == AMG_FP64 ? 1 : 0); AMG_COUNT();
         }
     }
-    (void)n_rows;
-    {
-        std::vector<float> wc(8 * static_cast<size_t>(nlev), 0.0f);
-        for (int l = 0; l < nlev - 1; ++l) {
-            for (int k = 0; k < 5; ++k) wc[8 * l + k] = static_cast<float>(coef[5 * l + k]);
-            wc[8 * l + 5] = static_cast<float>(1.0 / c->scales[l]);
-        }
-        CK(cudaMemcpyAsync(c->wcoef, wc.data(), sizeof(float) * wc.size(), cudaMemcpyHostToDevice, s));
-        c->q_nodes = false;
-        c->q64_stale = false;
-    }
+    c->q_nodes = false;
+    c->q64_stale = false;
     c->tail[1].ok = false;
     CKL("assemble pseudo-inverse");
     // the solve kernels fetch matrix values ahead of their grid-dependency
-    // wait: finish writing them before any of those kernels is launched
-    CK(cudaStreamSynchronize(s));
+    // wait: finish writing them before any of those kernels is launched (a
+    // caller that does not wait starts its chain on s with a full dependency)
+    if (sync) CK(cudaStreamSynchronize(s));
     c->have_q = true;
     c->smoother = AMG_SMOOTHER_GNN;
     return AMG_OK;
@@ -2560,7 +2585,7 @@ int amg_set_coeffs(amg_ctx *c, const double *coef, int n_rows) {
     if (!coef || n_rows < static_cast<int>(c->lev.size()) - 1)
         return ctx_fail(c, "need one coefficient row per smoothed level"), AMG_ERR_ARG;
     CK(cudaSetDevice(c->opt.device));
-    int rc = set_coeffs_device(c, coef, n_rows, c->stream);
+    int rc = set_coeffs_device(c, coef, c->stream, true);
     if (!rc) rc = ensure_tail(c, c->stream);
     if (rc) return rc;
     CK(cudaStreamSynchronize(c->stream));
@@ -2594,14 +2619,13 @@ int amg_set_node_coeffs(amg_ctx *c, const double *coef, long long n_values) {
         const DevLevel &L = c->lev[l];
         k_assemble_q_nodes<<<grid_for(L.n), kBlock, 0, s>>>(L.n, L.A.rp, L.A.col, L.isd, L.bx, L.bw, d_c + off,
                                                              L.q64, L.q32); AMG_COUNT();
-        if (L.fast && c->opt.precision == AMG_FP64) {
-            k_assemble_ma<<<grid_for(L.MA.nnz), kBlock, 0, s>>>(L.MA.nnz, L.pp, L.pq_p, L.pq_q, L.q64, L.A.v64,
-                                                                L.MA.v64, L.MA.v32); AMG_COUNT();
-        } else if (L.fast) {
-            k_assemble_ma32<<<grid_for(L.MA.nnz), kBlock, 0, s>>>(L.MA.nnz, L.pp, L.pq_p, L.pq_q, L.q32, L.A.v32,
-                                                                  L.MA.v32); AMG_COUNT();
-        }
         off += 5LL * L.n;
+        e = cudaGetLastError();
+    }
+    for (int l0 = 0; l0 < nlev - 1 && e == cudaSuccess; l0 += kAsmMaxLevels) {
+        const AsmMA M = asm_ma_levels(c, l0, std::min(nlev - 1, l0 + kAsmMaxLevels));
+        if (M.nlev == 0 || M.start[M.nlev] == 0) continue;
+        k_assemble_ma_all<<<grid_for(M.start[M.nlev]), kBlock, 0, s>>>(M, c->opt.precision == AMG_FP64 ? 1 : 0); AMG_COUNT();
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -2628,7 +2652,7 @@ int amg_get_smoother(const amg_ctx *cc, int level, double *q_out) {
         if (c->q64_stale) {
             // the network's coefficients were assembled for the FP32 V-cycle
             // only: form the FP64 values from the kept FP32 coefficients
-            const AsmQ Q = asm_q_levels(c);
+            const AsmQ Q = asm_q_levels(c, 0, static_cast<int>(c->lev.size()) - 1);
             if (Q.start[Q.nlev] > 0) {
                 k_assemble_q_all<<<grid_for(Q.start[Q.nlev]), kBlock, 0, c->stream>>>(Q, c->wcoef, 8, 2); AMG_COUNT();
             }
@@ -3244,7 +3268,7 @@ extern "C" int amg_residual_norm_noalloc(int n, long long nnz, const int *d_row_
 }
 
 // ---------------------------------------------------------------------------
-// Training loss and the hand-written V-cycle adjoint (Sec. 3.3, N_vc = 1)
+// Training loss and the hand-written V-cycle adjoint (Sec. 3.3)
 // ---------------------------------------------------------------------------
 // Forward: one V-cycle from u = 0 with the pseudo-inverse smoother, keeping
 // every sweep's input residual r_k per level (the checkpoints).  A sweep is
@@ -3256,99 +3280,194 @@ extern "C" int amg_residual_norm_noalloc(int n, long long nnz, const int *d_row_
 //   dM_ij/d(o1, o2)     = (x, x^2) / (a_ii + a_jj),    x = a_ij / s.
 namespace {
 
+// One step of the adjoint on a row-group of A's pattern.  The sweep
+// u' = u + M r has rbar = M ubar', dL/dM_ij = ubar'_i r_j; one pass over the
+// pattern forms rbar (stored when rbar != nullptr), adds it to bbar (assigns
+// with `assign`) and adds the sweep's share of dL/dc to the block's own five
+// partial sums (a block always owns the same rows, so every sweep of a level
+// adds into one slot per block and the sums stay in a fixed order).  It
+// replaces five launches per sweep (gradient pass, its one-block sum, M ubar,
+// bbar += rbar): on the training meshes (2k to 20k rows) each pass is a few
+// microseconds of dependent loads, whatever it computes.  Pattern, Q^-1 and
+// basis entries are loaded ahead of the grid-dependency wait.
 template <class T, int TPR>
-__global__ void __launch_bounds__(kBlock) k_coef_grad(int n, const int *__restrict__ rp, const int *__restrict__ col,
-                                                      const double *__restrict__ bx, const double *__restrict__ bw,
-                                                      const T *__restrict__ ubar, const T *__restrict__ r,
-                                                      double *__restrict__ partial) {
-    constexpr int RPB = kBlock / TPR;
-    const int lane = threadIdx.x % TPR;
-    double g[5] = {0, 0, 0, 0, 0};
-    for (int base = blockIdx.x * RPB; base < n; base += gridDim.x * RPB) {
-        const int row = base + threadIdx.x / TPR;
-        double acc[5] = {0, 0, 0, 0, 0};
-        if (row < n) {
-            const double ui = static_cast<double>(ubar[row]);
-            for (int p = rp[row] + lane; p < rp[row + 1]; p += TPR) {
-                const int j = col[p];
-                const double x = bx[p], w = ui * static_cast<double>(r[j]) * bw[p];
-                if (j == row) {
-                    acc[0] += w;
-                    acc[1] += w * x;
-                    acc[2] += w * x * x;
+__global__ void __launch_bounds__(kBlock) k_adj_sweep(int n, const int *__restrict__ rp, const int *__restrict__ col,
+                                                      const T *__restrict__ q, const double *__restrict__ bx,
+                                                      const double *__restrict__ bw, const T *ubar, const T *r,
+                                                      T *rbar, T *bbar, int assign, double *partial) {
+    constexpr int E = 4;
+    const int gid = blockIdx.x * kBlock + threadIdx.x;
+    const int row = gid / TPR, lane = gid % TPR;
+    int base = 0, end = 0, c[E];
+    T m[E];
+    double x[E], w[E];
+    auto fetch = [&](int b0) {
+#pragma unroll
+        for (int j = 0; j < E; ++j) {
+            const int p = b0 + j * TPR;
+            const bool in = p < end;
+            c[j] = in ? __ldg(col + p) : 0;
+            m[j] = in ? __ldg(q + p) : T(0);
+            x[j] = in ? __ldg(bx + p) : 0.0;
+            w[j] = in ? __ldg(bw + p) : 0.0;
+        }
+    };
+    if (row < n) {
+        base = __ldg(rp + row) + lane;
+        end = __ldg(rp + row + 1);
+        fetch(base);
+    }
+    pdl_wait_and_release();
+    T acc = T(0);
+    double g[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    for (; base < end; base += E * TPR) {
+        T uj[E], rj[E];
+#pragma unroll
+        for (int j = 0; j < E; ++j) {
+            const bool in = base + j * TPR < end;
+            uj[j] = in ? ubar[c[j]] : T(0);
+            rj[j] = in ? r[c[j]] : T(0);
+        }
+#pragma unroll
+        for (int j = 0; j < E; ++j) {
+            acc += m[j] * uj[j];
+            const double v = static_cast<double>(rj[j]) * w[j], vx = v * x[j];
+            if (base + j * TPR < end) {
+                if (c[j] == row) {
+                    g[0] += v;
+                    g[1] += vx;
+                    g[2] = fma(vx, x[j], g[2]);
                 } else {
-                    acc[3] += w * x;
-                    acc[4] += w * x * x;
+                    g[3] += vx;
+                    g[4] = fma(vx, x[j], g[4]);
                 }
             }
         }
+        if (base + E * TPR < end) fetch(base + E * TPR);
+    }
+    acc = group_sum<TPR>(acc);
+    if (row < n) {
+        const double ui = static_cast<double>(ubar[row]);
 #pragma unroll
-        for (int k = 0; k < 5; ++k) g[k] += group_sum<TPR>(acc[k]);
+        for (int k = 0; k < 5; ++k) g[k] *= ui;
+        if (lane == 0) {
+            if (rbar) rbar[row] = acc;
+            bbar[row] = assign ? acc : bbar[row] + acc;
+        }
     }
     __shared__ double red[5][kBlock / 32];
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-        double v = (lane == 0) ? g[k] : 0.0;
-        v = warp_sum(v);
+        const double v = warp_sum(g[k]);
         if (threadIdx.x % 32 == 0) red[k][threadIdx.x / 32] = v;
     }
     __syncthreads();
     if (threadIdx.x < 5) {
-        double t = 0.0;
-        for (int w = 0; w < kBlock / 32; ++w) t += red[threadIdx.x][w];
+        double t = partial[blockIdx.x * 5 + threadIdx.x];
+        for (int k = 0; k < kBlock / 32; ++k) t += red[threadIdx.x][k];
         partial[blockIdx.x * 5 + threadIdx.x] = t;
     }
 }
 
-__global__ void k_coef_grad_final(int np, const double *__restrict__ partial, double *__restrict__ dc) {
-    if (threadIdx.x >= 5) return;
-    double t = 0.0;
-    for (int b = 0; b < np; ++b) t += partial[b * 5 + threadIdx.x];
-    dc[threadIdx.x] += t;
+// Adjoint of the restriction b_c = R r: rhobar = R^T bbar_c = P bbar_c, which
+// is also added to (or, with `assign`, becomes) bbar.
+template <class T, int TPR>
+__global__ void __launch_bounds__(kBlock) k_adj_restrict(int n, const int *__restrict__ rp, const int *__restrict__ col,
+                                                         const T *__restrict__ m, const T *x, T *rhobar, T *bbar,
+                                                         int assign) {
+    const int g = blockIdx.x * kBlock + threadIdx.x;
+    const int row = g / TPR, lane = g % TPR;
+    RowBatch<T> rb;   // matrix loads ahead of the wait (constant during a call)
+    row_prefetch<TPR>(rb, row < n, lane, rp, row, col, m);
+    pdl_wait_and_release();
+    T acc = T(0);
+    if (row < n) acc = row_dot_pref<TPR>(rb, col, m, Gather<T>{x});
+    acc = group_sum<TPR>(acc);
+    if (row < n && lane == 0) {
+        rhobar[row] = acc;
+        bbar[row] = assign ? acc : bbar[row] + acc;
+    }
 }
 
+// dL/dc of every level from its blocks' partial sums (one block per level).
+struct CoefPartials {
+    int nlev;
+    int nblk[kAsmMaxLevels];
+    const double *part[kAsmMaxLevels];
+};
+__global__ void __launch_bounds__(kBlock) k_coef_grad_final(CoefPartials P, int level0, double *__restrict__ dc) {
+    pdl_wait_and_release();
+    __shared__ double red[kBlock / 32];
+    const double *part = P.part[blockIdx.x];
+    const int nb = P.nblk[blockIdx.x];
+    for (int k = 0; k < 5; ++k) {
+        double v = 0.0;
+        for (int b = threadIdx.x; b < nb; b += kBlock) v += part[b * 5 + k];
+        v = warp_sum(v);
+        if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = v;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double t = 0.0;
+            for (int w = 0; w < kBlock / 32; ++w) t += red[w];
+            dc[5 * (level0 + blockIdx.x) + k] = t;
+        }
+        __syncthreads();
+    }
+}
+
+// y = y + x
 template <class T>
-__global__ void k_add(int n, T *__restrict__ y, const T *__restrict__ x) {
-    int i = blockIdx.x * kBlock + threadIdx.x;
+__global__ void __launch_bounds__(kBlock) k_add(int n, T *y, const T *x) {
+    pdl_wait_and_release();
+    const int i = blockIdx.x * kBlock + threadIdx.x;
     if (i < n) y[i] += x[i];
 }
 
+// Partial sums of r.r and f.f over the blocks' elements
 template <class T>
-__global__ void k_scale_copy(int n, T *__restrict__ y, const T *__restrict__ x, double a) {
-    int i = blockIdx.x * kBlock + threadIdx.x;
-    if (i < n) y[i] = static_cast<T>(a * static_cast<double>(x[i]));
-}
-
-template <class T>
-__global__ void __launch_bounds__(kBlock) k_dot_partial(int n, const T *__restrict__ x, const T *__restrict__ y,
-                                                        double *__restrict__ partial) {
-    double s = 0.0;
-    for (int i = blockIdx.x * kBlock + threadIdx.x; i < n; i += gridDim.x * kBlock)
-        s += static_cast<double>(x[i]) * static_cast<double>(y[i]);
-    block_partial(s, partial);
-}
-
-__global__ void k_sum_final(int np, const double *__restrict__ partial, double *__restrict__ out) {
-    __shared__ double red[32];
-    double v = 0.0;
-    for (int i = threadIdx.x; i < np; i += 1024) v += partial[i];
-    v = warp_sum(v);
-    if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = v;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        v = warp_sum(red[threadIdx.x]);
-        if (threadIdx.x == 0) *out = v;
+__global__ void __launch_bounds__(kBlock) k_loss_dots(int n, const T *r, const T *f, double *prr, double *pff) {
+    pdl_wait_and_release();
+    double a = 0.0, b = 0.0;
+    for (int i = blockIdx.x * kBlock + threadIdx.x; i < n; i += gridDim.x * kBlock) {
+        a += static_cast<double>(r[i]) * static_cast<double>(r[i]);
+        b += static_cast<double>(f[i]) * static_cast<double>(f[i]);
     }
+    block_partial2(a, b, prr, pff);
+}
+
+// scal[0] = r.r, scal[1] = f.f and seed = r / (ln 10 r.r): every block sums
+// the partials (in the same order), so no launch stands between
+template <class T>
+__global__ void __launch_bounds__(kBlock) k_loss_seed(int n, const T *r, T *seed, const double *prr, const double *pff,
+                                                      int np, double *scal) {
+    pdl_wait_and_release();
+    __shared__ double red[kBlock / 32];
+    const double rr = sum_partials(prr, np, red);
+    const double ff = sum_partials(pff, np, red);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        scal[0] = rr;
+        scal[1] = ff;
+    }
+    const double a = 1.0 / (2.302585092994045684 * rr);
+    for (int i = blockIdx.x * kBlock + threadIdx.x; i < n; i += gridDim.x * kBlock)
+        seed[i] = static_cast<T>(a * static_cast<double>(r[i]));
 }
 
 struct TrainBufs {
     int ncyc = 0, nsw = 0, nlev = 0;
-    std::vector<double *> ck;      // [cycle][level][sweep]: slot 0 = that cycle's b_l, k >= 1 = r of sweep k
-    std::vector<double *> ubar, tmp, bbar, zero;
+    std::vector<double *> ck;      // [cycle][level][sweep]: r of sweep k (slot 0: that cycle's b_l when nu1 > 0)
+    std::vector<double *> ubar, tmp, bbar;
+    std::vector<double *> part;    // per smoothed level: five partial sums of dL/dc per block
+    std::vector<int> nblk;
+    double *f = nullptr, *zero = nullptr;   // level 0: right-hand side, zeros
     double *xu = nullptr;          // level-0 iterate of the multi-cycle loss
-    double *dcoef = nullptr;       // n_levels x 5
-    double *scal = nullptr;        // 4 doubles
+    double *dcoef = nullptr;       // n_levels x 5, then r.r and f.f
+    double *h_out = nullptr;       // pinned copy of dcoef
+    size_t part_bytes = 0;
     char *arena = nullptr;
+    cudaGraphExec_t exec = nullptr;   // the call's kernels for graph_nvc cycles (from its second call on)
+    int graph_nvc = 0, calls = 0;
+    long long kernels = 0;
     double *slot(int cyc, int l, int k) const { return ck[(static_cast<size_t>(cyc) * nlev + l) * nsw + k]; }
 };
 
@@ -3363,7 +3482,8 @@ int train_bufs(amg_ctx *c, TrainBufs &tb, int ncyc) {
         tb.ubar.assign(nlev, nullptr);
         tb.tmp.assign(nlev, nullptr);
         tb.bbar.assign(nlev, nullptr);
-        tb.zero.assign(nlev, nullptr);
+        tb.part.assign(nlev, nullptr);
+        tb.nblk.assign(nlev, 0);
         for (int l = 0; l < nlev; ++l) {
             const int n = c->lev[l].n;
             for (int q = 0; q < ncyc; ++q)
@@ -3371,15 +3491,27 @@ int train_bufs(amg_ctx *c, TrainBufs &tb, int ncyc) {
             tb.ubar[l] = pl.take<double>(n);
             tb.tmp[l] = pl.take<double>(n);
             tb.bbar[l] = pl.take<double>(n);
-            tb.zero[l] = pl.take<double>(n);
         }
+        tb.f = pl.take<double>(c->lev[0].n);
+        tb.zero = pl.take<double>(c->lev[0].n);
         tb.xu = pl.take<double>(c->lev[0].n);
-        tb.dcoef = pl.take<double>(static_cast<size_t>(nlev) * 5);
-        tb.scal = pl.take<double>(4);
+        size_t blocks = 0;
+        for (int l = 0; l < nlev - 1; ++l) {
+            tb.nblk[l] = grid_for(static_cast<long long>(c->lev[l].n) * c->lev[l].A.tpr);
+            blocks += tb.nblk[l];
+        }
+        tb.part_bytes = blocks * 5 * sizeof(double);
+        double *p = pl.take<double>(std::max<size_t>(1, blocks * 5));
+        for (int l = 0; l < nlev - 1; ++l) {
+            tb.part[l] = p;
+            if (p) p += 5 * static_cast<size_t>(tb.nblk[l]);
+        }
+        tb.dcoef = pl.take<double>(static_cast<size_t>(nlev) * 5 + 2);
     };
     Planner pl;
     lay(pl);
     cudaError_t e = cudaMalloc(&tb.arena, pl.off);
+    if (e == cudaSuccess) e = cudaMallocHost(&tb.h_out, sizeof(double) * (static_cast<size_t>(nlev) * 5 + 2));
     if (e != cudaSuccess) return ctx_cuda_check(c, e, "cudaMalloc training buffers");
     const size_t bytes = pl.off;
     pl = Planner{};
@@ -3388,18 +3520,25 @@ int train_bufs(amg_ctx *c, TrainBufs &tb, int ncyc) {
     return ctx_cuda_check(c, cudaMemsetAsync(tb.arena, 0, bytes, c->stream), "memset training buffers");
 }
 
+// Right-hand side of level l in cycle cyc: written straight into the
+// checkpoint that the first sweep's gradient reads.
+template <class T>
+T *level_b(amg_ctx *c, const TrainBufs &tb, int cyc, int l) {
+    if (cyc == 0 && l == 0) return reinterpret_cast<T *>(tb.f);       // r_0 = f (u_0 = 0)
+    if (c->opt.nu1 > 0 && l < tb.nlev - 1) return reinterpret_cast<T *>(tb.slot(cyc, l, 0));
+    return reinterpret_cast<T *>(c->lev[l].vb);
+}
+
 template <class T>
 T *fwd_level_ckpt(amg_ctx *c, TrainBufs &tb, int cyc, int l, cudaStream_t s) {
     DevLevel &L = c->lev[l];
-    T *b = reinterpret_cast<T *>(L.vb), *u = reinterpret_cast<T *>(L.vu), *r = reinterpret_cast<T *>(L.vr);
-    const int nlev = static_cast<int>(c->lev.size());
-    const int nu1 = c->opt.nu1, nu2 = c->opt.nu2, nsw = nu1 + nu2;
-    if (l == nlev - 1) {
-        launch_pdl(k_coarse<T>, dim3(1), dim3(kBlock), 2 * sizeof(double) * c->nL, s, c->nL, c->Linv, c->LinvT, b, u);
+    T *b = level_b<T>(c, tb, cyc, l), *u = reinterpret_cast<T *>(L.vu), *r = reinterpret_cast<T *>(L.vr);
+    const int nu1 = c->opt.nu1, nsw = nu1 + c->opt.nu2;
+    if (l == tb.nlev - 1) {
+        launch_coarse<T>(c, b, u, s);
         return u;
     }
     auto ck = [&](int k) { return reinterpret_cast<T *>(tb.slot(cyc, l, k)); };
-    cudaMemcpyAsync(ck(0), b, sizeof(T) * L.n, cudaMemcpyDeviceToDevice, s);
     if (nu1 == 0) cudaMemsetAsync(u, 0, sizeof(T) * L.n, s);
     for (int k = 0; k < nu1; ++k) {
         if (k == 0) {
@@ -3410,88 +3549,73 @@ T *fwd_level_ckpt(amg_ctx *c, TrainBufs &tb, int cyc, int l, cudaStream_t s) {
         }
     }
     L_resid<T>(L.A, b, u, r, s);
-    L_spmv<T>(L.R, r, reinterpret_cast<T *>(c->lev[l + 1].vb), s);
+    L_spmv<T>(L.R, r, level_b<T>(c, tb, cyc, l + 1), s);
     T *e = fwd_level_ckpt<T>(c, tb, cyc, l + 1, s);
     L_apply<T>(L.P, mvals<T>(L.P), e, u, 1, s);
     for (int k = nu1; k < nsw; ++k) {
         L_resid<T>(L.A, b, u, ck(k), s);
         L_apply<T>(L.A, qvals<T>(L), ck(k), u, 1, s);
     }
-    (void)nsw;
     return u;
 }
 
-template <class T>
-void coef_grad(amg_ctx *c, TrainBufs &tb, int l, const T *ubar, const T *r, cudaStream_t s) {
-    const DevLevel &L = c->lev[l];
-    const DevMat &A = L.A;
-    const int nb = outer_blocks(A);
-#define CG_LAUNCH(TP)                                                                                          \
-    k_coef_grad<T, TP><<<nb, kBlock, 0, s>>>(A.nr, A.rp, A.col, L.bx, L.bw, ubar, r, c->partials); \
-    AMG_COUNT();
-    switch (A.tpr) {
-        case 1: CG_LAUNCH(1) break;
-        case 2: CG_LAUNCH(2) break;
-        case 4: CG_LAUNCH(4) break;
-        case 8: CG_LAUNCH(8) break;
-        case 16: CG_LAUNCH(16) break;
-        default: CG_LAUNCH(32) break;
+template <class T> struct AdjLaunch {
+    template <int TPR>
+    static void sweep(const DevLevel &L, const T *ubar, const T *r, T *rbar, T *bbar, int assign, double *part,
+                      cudaStream_t s) {
+        launch_pdl(k_adj_sweep<T, TPR>, dim3(grid_for(static_cast<long long>(L.n) * TPR)), dim3(kBlock), 0, s, L.n,
+                   L.A.rp, static_cast<const int *>(L.A.col), qvals<T>(L), static_cast<const double *>(L.bx),
+                   static_cast<const double *>(L.bw), ubar, r, rbar, bbar, assign, part);
     }
-#undef CG_LAUNCH
-    k_coef_grad_final<<<1, 32, 0, s>>>(nb, c->partials, tb.dcoef + 5 * l); AMG_COUNT();
-}
+    template <int TPR>
+    static void restrict_(const DevMat &P, const T *x, T *rhobar, T *bbar, int assign, cudaStream_t s) {
+        launch_pdl(k_adj_restrict<T, TPR>, dim3(grid_for(static_cast<long long>(P.nr) * TPR)), dim3(kBlock), 0, s, P.nr,
+                   P.rp, static_cast<const int *>(P.col), mvals<T>(P), x, rhobar, bbar, assign);
+    }
+};
 
-// Backward of one sweep u' = u + M r (r = b - A u): accumulate dL/dc, then
-// ubar <- ubar - A (M ubar) into `spare`, bbar += M ubar.  Returns the new ubar.
+// Backward of the V-cycle on level l: `in` = dL/d(level output); tb.bbar[l] =
+// dL/d(level right-hand side) out.  The adjoint alternates between tb.tmp[l]
+// and `other` (never writing `in` when the caller still needs it).
 template <class T>
-T *sweep_adjoint(amg_ctx *c, TrainBufs &tb, int l, T *ubar, T *spare, const T *r, T *bbar, cudaStream_t s) {
-    const DevLevel &L = c->lev[l];
-    coef_grad<T>(c, tb, l, ubar, r, s);
-    T *rbar = reinterpret_cast<T *>(L.vt);            // free during the backward pass
-    L_apply<T>(L.A, qvals<T>(L), ubar, rbar, 0, s);   // rbar = M ubar
-    L_resid<T>(L.A, ubar, rbar, spare, s);            // spare = ubar - A rbar
-    k_add<T><<<grid_for(L.n), kBlock, 0, s>>>(L.n, bbar, rbar); AMG_COUNT();
-    return spare;
-}
-
-// Backward of the V-cycle on level l: tb.ubar[l] = dL/d(level output) in,
-// tb.bbar[l] = dL/d(level right-hand side) out.
-template <class T>
-void bwd_level(amg_ctx *c, TrainBufs &tb, int cyc, int l, cudaStream_t s) {
+void bwd_level(amg_ctx *c, TrainBufs &tb, int cyc, int l, const T *in, T *other, cudaStream_t s) {
     DevLevel &L = c->lev[l];
-    const int nlev = static_cast<int>(c->lev.size());
-    const int nu1 = c->opt.nu1, nu2 = c->opt.nu2, nsw = nu1 + nu2;
-    T *ub = reinterpret_cast<T *>(tb.ubar[l]), *sp = reinterpret_cast<T *>(tb.tmp[l]);
+    const int nu1 = c->opt.nu1, nsw = nu1 + c->opt.nu2;
     T *bb = reinterpret_cast<T *>(tb.bbar[l]);
-    if (l == nlev - 1) {   // u = A_L^-1 b is self-adjoint
-        launch_pdl(k_coarse<T>, dim3(1), dim3(kBlock), 2 * sizeof(double) * c->nL, s, c->nL, c->Linv, c->LinvT, ub, bb);
+    if (l == tb.nlev - 1) {   // u = A_L^-1 b is self-adjoint
+        launch_coarse<T>(c, in, bb, s);
         return;
     }
-    auto ck = [&](int k) { return reinterpret_cast<const T *>(tb.slot(cyc, l, k)); };
-    cudaMemsetAsync(bb, 0, sizeof(T) * L.n, s);
-    for (int k = nsw - 1; k >= nu1; --k) {
-        T *nu = sweep_adjoint<T>(c, tb, l, ub, sp, ck(k), bb, s);
-        sp = ub;
-        ub = nu;
-    }
+    const T *ub = in;
+    T *out = reinterpret_cast<T *>(tb.tmp[l]), *spare = other;
+    T *rbar = reinterpret_cast<T *>(L.vt);            // free during the backward pass
+    int assign = 1;                                   // bbar's first contribution replaces the last call's
+    auto advance = [&]() {
+        ub = out;
+        std::swap(out, spare);
+    };
+    auto sweep = [&](int k) {                         // ubar <- ubar - A (M ubar), bbar += M ubar
+        TPR_DISPATCH(L.A.tpr, AdjLaunch<T>::template sweep, L, ub, reinterpret_cast<const T *>(tb.slot(cyc, l, k)), rbar,
+                     bb, assign, tb.part[l], s);
+        assign = 0;
+        L_resid<T>(L.A, ub, rbar, out, s);
+        advance();
+    };
+    for (int k = nsw - 1; k >= nu1; --k) sweep(k);
     // prolongation u += P e: ebar = P^T ubar = R ubar
-    L_spmv<T>(L.R, ub, reinterpret_cast<T *>(tb.ubar[l + 1]), s);
-    bwd_level<T>(c, tb, cyc, l + 1, s);
+    T *ebar = reinterpret_cast<T *>(tb.ubar[l + 1]);
+    L_spmv<T>(L.R, ub, ebar, s);
+    bwd_level<T>(c, tb, cyc, l + 1, ebar, ebar, s);
     // restriction b_{l+1} = R (b - A u): rhobar = R^T bbar_{l+1} = P bbar_{l+1}
-    T *rhobar = reinterpret_cast<T *>(L.vt);
-    L_spmv<T>(L.P, reinterpret_cast<const T *>(tb.bbar[l + 1]), rhobar, s);
-    k_add<T><<<grid_for(L.n), kBlock, 0, s>>>(L.n, bb, rhobar); AMG_COUNT();
-    L_resid<T>(L.A, ub, rhobar, sp, s);
-    std::swap(ub, sp);
-    for (int k = nu1 - 1; k >= 1; --k) {
-        T *nu = sweep_adjoint<T>(c, tb, l, ub, sp, ck(k), bb, s);
-        sp = ub;
-        ub = nu;
-    }
+    TPR_DISPATCH(L.P.tpr, AdjLaunch<T>::template restrict_, L.P, reinterpret_cast<const T *>(tb.bbar[l + 1]), rbar, bb,
+                 assign, s);
+    assign = 0;
+    L_resid<T>(L.A, ub, rbar, out, s);
+    advance();
+    for (int k = nu1 - 1; k >= 1; --k) sweep(k);
     if (nu1 >= 1) {        // first sweep from zero: u = M b
-        coef_grad<T>(c, tb, l, ub, ck(0), s);
-        L_apply<T>(L.A, qvals<T>(L), ub, reinterpret_cast<T *>(L.vt), 0, s);
-        k_add<T><<<grid_for(L.n), kBlock, 0, s>>>(L.n, bb, reinterpret_cast<const T *>(L.vt)); AMG_COUNT();
+        TPR_DISPATCH(L.A.tpr, AdjLaunch<T>::template sweep, L, ub, static_cast<const T *>(level_b<T>(c, tb, cyc, l)),
+                     static_cast<T *>(nullptr), bb, 0, tb.part[l], s);
     }
 }
 
@@ -3499,57 +3623,103 @@ void bwd_level(amg_ctx *c, TrainBufs &tb, int cyc, int l, cudaStream_t s) {
 // stationary V-cycle in refinement form), L = sum_n log10(||r_n|| / ||r_{n-1}||)
 // = log10(||r_N|| / ||f||).  Backward: ubar_N = -A r_N / (ln10 ||r_N||^2);
 // for n = N..1: rbar = B^T ubar (level adjoint, accumulating dL/dc), ubar -= A rbar.
+// Every kernel of it, from f in c->db to tb.dcoef; no host step in between.
 template <class T>
-int loss_grad(amg_ctx *c, TrainBufs &tb, const double *f, int nvc, double *loss, double *dc) {
-    cudaStream_t s = c->stream;
+void loss_enqueue(amg_ctx *c, TrainBufs &tb, int nvc, cudaStream_t s) {
     DevLevel &L0 = c->lev[0];
-    const int n0 = L0.n, nlev = static_cast<int>(c->lev.size());
-    T *fT = reinterpret_cast<T *>(tb.tmp[0]);
+    const int n0 = L0.n, nlev = tb.nlev;
+    T *fT = reinterpret_cast<T *>(tb.f);
     T *xu = reinterpret_cast<T *>(tb.xu);
-    T *b0 = reinterpret_cast<T *>(L0.vb);
-    CK(cudaMemcpyAsync(c->db, f, sizeof(double) * n0, cudaMemcpyHostToDevice, s));
-    launch_pdl(k_convert<double, T>, dim3(grid_for(n0)), dim3(kBlock), 0, s, n0, c->db, fT);
-    CK(cudaMemsetAsync(xu, 0, sizeof(T) * n0, s));
+    if (tb.part_bytes) cudaMemsetAsync(tb.part[0], 0, tb.part_bytes, s);
+    // the chain's first kernel waits for everything before it (Q^-1 is new)
+    k_convert<double, T><<<grid_for(n0), kBlock, 0, s>>>(n0, c->db, fT); AMG_COUNT();
     for (int q = 0; q < nvc; ++q) {
-        L_resid<T>(L0.A, fT, xu, b0, s);          // r_{q} = f - A u_q -> level-0 right-hand side
+        if (q > 0) L_resid<T>(L0.A, fT, xu, level_b<T>(c, tb, q, 0), s);   // r_q = f - A u_q
         T *e = fwd_level_ckpt<T>(c, tb, q, 0, s);
-        k_add<T><<<grid_for(n0), kBlock, 0, s>>>(n0, xu, e); AMG_COUNT();
+        if (q == 0) launch_pdl(k_convert<T, T>, dim3(grid_for(n0)), dim3(kBlock), 0, s, n0, static_cast<const T *>(e), xu);
+        else launch_pdl(k_add<T>, dim3(grid_for(n0)), dim3(kBlock), 0, s, n0, xu, static_cast<const T *>(e));
     }
     T *rN = reinterpret_cast<T *>(L0.vr);
     L_resid<T>(L0.A, fT, xu, rN, s);
     const int nb = std::min(grid_for(n0), kNumSMs * 8);
-    k_dot_partial<T><<<nb, kBlock, 0, s>>>(n0, rN, rN, c->partials); AMG_COUNT();
-    k_sum_final<<<1, 1024, 0, s>>>(nb, c->partials, tb.scal); AMG_COUNT();
-    k_dot_partial<T><<<nb, kBlock, 0, s>>>(n0, fT, fT, c->partials); AMG_COUNT();
-    k_sum_final<<<1, 1024, 0, s>>>(nb, c->partials, tb.scal + 1); AMG_COUNT();
-    double h[2] = {0, 0};
-    CK(cudaMemcpyAsync(h, tb.scal, sizeof(double) * 2, cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    const double rr = h[0], ff = h[1];
-    if (!(rr > 0.0) || !(ff > 0.0) || !std::isfinite(rr))
-        return ctx_fail(c, "loss undefined: zero or non-finite residual"), AMG_ERR_DIVERGED;
-    *loss = 0.5 * std::log10(rr / ff);
-    // ubar_N = -A (r_N / (ln10 ||r_N||^2)) into ubar[0].  The carried adjoint
-    // and its scratch use xu and vr of level 0, which the level adjoint never
+    double *prr = c->partials, *pff = c->partials + c->n_partials;
+    launch_pdl(k_loss_dots<T>, dim3(nb), dim3(kBlock), 0, s, n0, static_cast<const T *>(rN), static_cast<const T *>(fT),
+               prr, pff);
+    // ubar_N = -A (r_N / (ln10 ||r_N||^2)) into uacc.  The carried adjoint
+    // and its scratch use vr and xu of level 0, which the level adjoint never
     // touches (it works in ubar/tmp/bbar and vt).
-    T *seed = xu;                                   // the forward iterate is no longer needed
-    T *ub0 = reinterpret_cast<T *>(tb.ubar[0]);
-    k_scale_copy<T><<<grid_for(n0), kBlock, 0, s>>>(n0, seed, rN, 1.0 / (std::log(10.0) * rr)); AMG_COUNT();
-    L_resid<T>(L0.A, reinterpret_cast<const T *>(tb.zero[0]), seed, ub0, s);
-    CK(cudaMemsetAsync(tb.dcoef, 0, sizeof(double) * 5 * nlev, s));
-    T *uacc = rN;                                   // dL/du_q carried across cycles (r_N no longer needed)
-    CK(cudaMemcpyAsync(uacc, ub0, sizeof(T) * n0, cudaMemcpyDeviceToDevice, s));
+    T *seed = xu, *uacc = rN;
+    launch_pdl(k_loss_seed<T>, dim3(nb), dim3(kBlock), 0, s, n0, static_cast<const T *>(rN), seed,
+               static_cast<const double *>(prr), static_cast<const double *>(pff), nb, tb.dcoef + 5 * nlev);
+    L_resid<T>(L0.A, reinterpret_cast<const T *>(tb.zero), seed, uacc, s);
     for (int q = nvc - 1; q >= 0; --q) {
-        CK(cudaMemcpyAsync(ub0, uacc, sizeof(T) * n0, cudaMemcpyDeviceToDevice, s));   // ebar = ubar_{q+1}
-        bwd_level<T>(c, tb, q, 0, s);                                                // bbar[0] = rbar_q
+        bwd_level<T>(c, tb, q, 0, uacc, reinterpret_cast<T *>(tb.ubar[0]), s);       // bbar[0] = rbar_q
         if (q > 0) {
             L_resid<T>(L0.A, uacc, reinterpret_cast<const T *>(tb.bbar[0]), seed, s);   // ubar_q = ubar - A rbar
             std::swap(uacc, seed);
         }
     }
+    for (int l0 = 0; l0 < nlev - 1; l0 += kAsmMaxLevels) {
+        CoefPartials P{};
+        P.nlev = std::min(nlev - 1 - l0, kAsmMaxLevels);
+        for (int l = 0; l < P.nlev; ++l) {
+            P.nblk[l] = tb.nblk[l0 + l];
+            P.part[l] = tb.part[l0 + l];
+        }
+        launch_pdl(k_coef_grad_final, dim3(P.nlev), dim3(kBlock), 0, s, P, l0, tb.dcoef);
+    }
+}
+
+// Training calls a problem once per epoch with new coefficients: from the
+// second call with the same number of cycles on, its 300 to 400 kernels are
+// one graph launch.  12k-row mesh, three cycles: 2341 us a call with five
+// launches per adjoint sweep and a host step for the loss, 1235 us with the
+// fused passes launched singly (a first call), 1011 us as a graph.
+template <class T>
+int loss_grad(amg_ctx *c, TrainBufs &tb, const double *f, int nvc, double *loss, double *dc) {
+    cudaStream_t s = c->stream;
+    const int nlev = tb.nlev;
+    CK(cudaMemcpyAsync(c->db, f, sizeof(double) * c->lev[0].n, cudaMemcpyHostToDevice, s));
+    if (tb.graph_nvc != nvc) {
+        if (tb.exec) cudaGraphExecDestroy(tb.exec);
+        tb.exec = nullptr;
+        tb.graph_nvc = nvc;
+        tb.calls = 0;
+    }
+    if (!tb.exec && ++tb.calls == 2) {
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        const long long before = g_launches.load();
+        cudaGraph_t g = nullptr;
+        cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeRelaxed);
+        if (e == cudaSuccess) {
+            loss_enqueue<T>(c, tb, nvc, s);
+            e = cudaStreamEndCapture(s, &g);
+        }
+        tb.kernels = g_launches.load() - before;
+        g_launches.fetch_sub(tb.kernels);
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&tb.exec, g, 0);
+        if (g) cudaGraphDestroy(g);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            tb.exec = nullptr;
+        }
+    }
+    if (tb.exec) {
+        CK(cudaGraphLaunch(tb.exec, s));
+        g_launches.fetch_add(tb.kernels);
+    } else {
+        loss_enqueue<T>(c, tb, nvc, s);
+    }
     CKL("V-cycle adjoint");
-    CK(cudaMemcpyAsync(dc, tb.dcoef, sizeof(double) * 5 * nlev, cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(tb.h_out, tb.dcoef, sizeof(double) * (5 * nlev + 2), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
+    const double rr = tb.h_out[5 * nlev], ff = tb.h_out[5 * nlev + 1];
+    if (!(rr > 0.0) || !(ff > 0.0) || !std::isfinite(rr))
+        return ctx_fail(c, "loss undefined: zero or non-finite residual"), AMG_ERR_DIVERGED;
+    *loss = 0.5 * std::log10(rr / ff);
+    std::copy(tb.h_out, tb.h_out + 5 * nlev, dc);
     return AMG_OK;
 }
 
@@ -3562,7 +3732,7 @@ extern "C" int amg_loss_grad(amg_ctx *c, const double *coef, const double *f, in
     if (!coef || !f || !loss || !dc || n_vc < 1 || n_vc > 64) return ctx_fail(c, "bad argument"), AMG_ERR_ARG;
     CK(cudaSetDevice(c->opt.device));
     const int nlev = static_cast<int>(c->lev.size());
-    int rc = set_coeffs_device(c, coef, nlev, c->stream);
+    int rc = set_coeffs_device(c, coef, c->stream, false);
     if (rc) return rc;
     if (c->train && static_cast<TrainBufs *>(c->train)->ncyc < n_vc) train_bufs_free(c);
     if (!c->train) {
@@ -3570,6 +3740,7 @@ extern "C" int amg_loss_grad(amg_ctx *c, const double *coef, const double *f, in
         rc = train_bufs(c, *tb, n_vc);
         if (rc) {
             if (tb->arena) cudaFree(tb->arena);
+            if (tb->h_out) cudaFreeHost(tb->h_out);
             delete tb;
             return rc;
         }
@@ -3584,7 +3755,9 @@ namespace amg {
 void train_bufs_free(amg_ctx *c) {
     if (!c->train) return;
     TrainBufs *tb = static_cast<TrainBufs *>(c->train);
+    if (tb->exec) cudaGraphExecDestroy(tb->exec);
     if (tb->arena) cudaFree(tb->arena);
+    if (tb->h_out) cudaFreeHost(tb->h_out);
     delete tb;
     c->train = nullptr;
 }
