@@ -75,15 +75,17 @@ template <class T, int TPR, class CS = const int *>
 __global__ void __launch_bounds__(kBlock) k_resid(int n, const int *__restrict__ rp, CS col,
                                                   const T *__restrict__ a, const T *__restrict__ b,
                                                   const T *__restrict__ u, T *__restrict__ r) {
-    const int g = blockIdx.x * kBlock + threadIdx.x;
+    const int g = pass_block(col) * kBlock + threadIdx.x;
     const int row = g / TPR, lane = g % TPR;
     RowBatch<T> rb;   // matrix loads ahead of the wait (constant during a solve)
     row_prefetch<TPR>(rb, row < n, lane, rp, row, col, a);
     pdl_wait_and_release();
+    const bool own = row < n && lane == 0;
+    const T bi = own ? load_now(b + row) : T(0);
     T acc = T(0);
     if (row < n) acc = row_dot_pref<TPR>(rb, col, a, Gather<T>{u});
     acc = group_sum<TPR>(acc);
-    if (row < n && lane == 0) r[row] = b[row] - acc;
+    if (own) r[row] = bi - acc;
 }
 
 // y = M x   (restriction with R, or a plain product)
@@ -108,15 +110,17 @@ template <class T, int TPR, class CS = const int *>
 __global__ void __launch_bounds__(kBlock) k_apply(int n, const int *__restrict__ rp, CS col,
                                                   const T *__restrict__ m, const T *__restrict__ r,
                                                   T *__restrict__ u, int add) {
-    const int g = blockIdx.x * kBlock + threadIdx.x;
+    const int g = pass_block(col) * kBlock + threadIdx.x;
     const int row = g / TPR, lane = g % TPR;
     RowBatch<T> rb;   // matrix loads ahead of the wait (constant during a solve)
     row_prefetch<TPR>(rb, row < n, lane, rp, row, col, m);
     pdl_wait_and_release();
+    const bool own = row < n && lane == 0;
+    const T ui = own && add ? load_now(u + row) : T(0);
     T acc = T(0);
     if (row < n) acc = row_dot_pref<TPR>(rb, col, m, Gather<T>{r});
     acc = group_sum<TPR>(acc);
-    if (row < n && lane == 0) u[row] = (add ? u[row] : T(0)) + acc;
+    if (own) u[row] = ui + acc;
 }
 
 // u_out = u_in + (omega/a_ii) (b - A u_in)   (relaxed Jacobi, Sec. 2.3)
@@ -125,15 +129,18 @@ __global__ void __launch_bounds__(kBlock) k_jacobi(int n, const int *__restrict_
                                                    const T *__restrict__ a, const T *__restrict__ jac,
                                                    const T *__restrict__ b, const T *__restrict__ uin,
                                                    T *__restrict__ uout) {
-    const int g = blockIdx.x * kBlock + threadIdx.x;
+    const int g = pass_block(col) * kBlock + threadIdx.x;
     const int row = g / TPR, lane = g % TPR;
     RowBatch<T> rb;   // matrix loads ahead of the wait (constant during a solve)
     row_prefetch<TPR>(rb, row < n, lane, rp, row, col, a);
     pdl_wait_and_release();
+    const bool own = row < n && lane == 0;
+    const T ji = own ? load_now(jac + row) : T(0), bi = own ? load_now(b + row) : T(0);
+    const T ui = own ? load_now(uin + row) : T(0);
     T acc = T(0);
     if (row < n) acc = row_dot_pref<TPR>(rb, col, a, Gather<T>{uin});
     acc = group_sum<TPR>(acc);
-    if (row < n && lane == 0) uout[row] = uin[row] + jac[row] * (b[row] - acc);
+    if (own) uout[row] = ui + ji * (bi - acc);
 }
 
 // Single-pass pseudo-inverse sweep on latency-optimised levels:
@@ -147,15 +154,17 @@ __global__ void __launch_bounds__(kBlock) k_ma_sweep(int n, const int *__restric
     RowBatch<T> rb;   // matrix loads ahead of the wait (constant during a solve)
     row_prefetch<TPR>(rb, row < n, lane, rp, row, col, ma);
     pdl_wait_and_release();
+    const bool own = row < n && lane == 0;
+    const T wi = own ? load_now(w + row) : T(0), ui = own ? load_now(uin + row) : T(0);
     T acc = T(0);
     if (row < n) acc = row_dot_pref<TPR>(rb, col, ma, Gather<T>{uin});
     acc = group_sum<TPR>(acc);
-    if (row < n && lane == 0) uout[row] = uin[row] + (w[row] - acc);
+    if (own) uout[row] = ui + (wi - acc);
 }
 
 // First sweep from zero that also keeps w = M b: u = w = M b
-template <class T, int TPR, class CS = const int *>
-__global__ void __launch_bounds__(kBlock) k_apply_w(int n, const int *__restrict__ rp, CS col,
+template <class T, int TPR>
+__global__ void __launch_bounds__(kBlock) k_apply_w(int n, const int *__restrict__ rp, const int *__restrict__ col,
                                                     const T *__restrict__ m, const T *__restrict__ b,
                                                     T *__restrict__ u, T *__restrict__ w) {
     const int g = blockIdx.x * kBlock + threadIdx.x;
@@ -205,17 +214,19 @@ template <class T, int TPR, class CS = const int *>
 __global__ void __launch_bounds__(kBlock) k_jacobi_first2(int n, const int *__restrict__ rp, CS col,
                                                           const T *__restrict__ a, const T *__restrict__ jac,
                                                           const T *__restrict__ b, T *__restrict__ u) {
-    const int g = blockIdx.x * kBlock + threadIdx.x;
+    const int g = pass_block(col) * kBlock + threadIdx.x;
     const int row = g / TPR, lane = g % TPR;
     RowBatch<T> rb;   // matrix loads ahead of the wait (constant during a solve)
     row_prefetch<TPR>(rb, row < n, lane, rp, row, col, a);
     pdl_wait_and_release();
+    const bool own = row < n && lane == 0;
+    const T ji = own ? load_now(jac + row) : T(0), bi = own ? load_now(b + row) : T(0);
     T acc = T(0);
     if (row < n) acc = row_dot_pref<TPR>(rb, col, a, JacB<T>{jac, b});
     acc = group_sum<TPR>(acc);
-    if (row < n && lane == 0) {
-        const T u1 = jac[row] * b[row];
-        u[row] = u1 + jac[row] * (b[row] - acc);
+    if (own) {
+        const T u1 = ji * bi;
+        u[row] = u1 + ji * (bi - acc);
     }
 }
 
@@ -239,19 +250,22 @@ __global__ void __launch_bounds__(kBlock) k_cheb_step(int n, const int *__restri
                                                       const T *__restrict__ b, const T *__restrict__ uin,
                                                       T *__restrict__ uout, T *__restrict__ d, T cd, T cr,
                                                       int first) {
-    const int g = blockIdx.x * kBlock + threadIdx.x;
+    const int g = pass_block(col) * kBlock + threadIdx.x;
     const int row = g / TPR, lane = g % TPR;
     RowBatch<T> rb;   // matrix loads ahead of the wait (constant during a solve)
     row_prefetch<TPR>(rb, row < n, lane, rp, row, col, a);
     pdl_wait_and_release();
+    const bool own = row < n && lane == 0;
+    const T vi = own ? load_now(dinv + row) : T(0), bi = own ? load_now(b + row) : T(0);
+    const T ui = own ? load_now(uin + row) : T(0), d0 = own && !first ? load_now(d + row) : T(0);
     T acc = T(0);
     if (row < n) acc = row_dot_pref<TPR>(rb, col, a, Gather<T>{uin});
     acc = group_sum<TPR>(acc);
-    if (row < n && lane == 0) {
-        const T dr = cr * (dinv[row] * (b[row] - acc));
-        const T di = first ? dr : cd * d[row] + dr;
+    if (own) {
+        const T dr = cr * (vi * (bi - acc));
+        const T di = first ? dr : cd * d0 + dr;
         d[row] = di;
-        uout[row] = uin[row] + di;
+        uout[row] = ui + di;
     }
 }
 
@@ -984,12 +998,25 @@ template <> const float *jvals<float>(const DevLevel &L) { return L.j32; }
         default: KERNEL<32>(__VA_ARGS__); break;          \
     }
 
+// Calls f with the way M's passes read their columns (common.cuh).
+template <class F> static void launch_pass(const DevMat &M, const F &f) {
+    if (M.dcol && M.stream) {
+        f(ColStream{M.dcol, M.reverse});
+        M.reverse ^= 1;
+    } else if (M.dcol) {
+        f(ColDelta{M.dcol});
+    } else {
+        f(static_cast<const int *>(M.col));
+    }
+}
+
 template <class T> struct Launch {
     template <int TPR>
     static void resid(const DevMat &A, const T *b, const T *u, T *r, cudaStream_t s) {
         const dim3 g(grid_for(static_cast<long long>(A.nr) * TPR));
-        if (A.dcol) launch_pdl(k_resid<T, TPR, ColDelta>, g, dim3(kBlock), 0, s, A.nr, A.rp, ColDelta{A.dcol}, mvals<T>(A), b, u, r);
-        else launch_pdl(k_resid<T, TPR>, g, dim3(kBlock), 0, s, A.nr, A.rp, static_cast<const int *>(A.col), mvals<T>(A), b, u, r);
+        launch_pass(A, [&](auto cs) {
+            launch_pdl(k_resid<T, TPR, decltype(cs)>, g, dim3(kBlock), 0, s, A.nr, A.rp, cs, mvals<T>(A), b, u, r);
+        });
     }
     template <int TPR>
     static void spmv(const DevMat &M, const T *x, T *y, cudaStream_t s) {
@@ -999,14 +1026,16 @@ template <class T> struct Launch {
     template <int TPR>
     static void apply(const DevMat &M, const T *m, const T *r, T *u, int add, cudaStream_t s) {
         const dim3 g(grid_for(static_cast<long long>(M.nr) * TPR));
-        if (M.dcol) launch_pdl(k_apply<T, TPR, ColDelta>, g, dim3(kBlock), 0, s, M.nr, M.rp, ColDelta{M.dcol}, m, r, u, add);
-        else launch_pdl(k_apply<T, TPR>, g, dim3(kBlock), 0, s, M.nr, M.rp, static_cast<const int *>(M.col), m, r, u, add);
+        launch_pass(M, [&](auto cs) {
+            launch_pdl(k_apply<T, TPR, decltype(cs)>, g, dim3(kBlock), 0, s, M.nr, M.rp, cs, m, r, u, add);
+        });
     }
     template <int TPR>
     static void jacobi(const DevMat &A, const T *jac, const T *b, const T *uin, T *uout, cudaStream_t s) {
         const dim3 g(grid_for(static_cast<long long>(A.nr) * TPR));
-        if (A.dcol) launch_pdl(k_jacobi<T, TPR, ColDelta>, g, dim3(kBlock), 0, s, A.nr, A.rp, ColDelta{A.dcol}, mvals<T>(A), jac, b, uin, uout);
-        else launch_pdl(k_jacobi<T, TPR>, g, dim3(kBlock), 0, s, A.nr, A.rp, static_cast<const int *>(A.col), mvals<T>(A), jac, b, uin, uout);
+        launch_pass(A, [&](auto cs) {
+            launch_pdl(k_jacobi<T, TPR, decltype(cs)>, g, dim3(kBlock), 0, s, A.nr, A.rp, cs, mvals<T>(A), jac, b, uin, uout);
+        });
     }
     template <int TPR>
     static void ma_sweep(const DevMat &MA, const T *w, const T *uin, T *uout, cudaStream_t s) {
@@ -1016,8 +1045,7 @@ template <class T> struct Launch {
     template <int TPR>
     static void apply_w(const DevMat &A, const T *m, const T *b, T *u, T *w, cudaStream_t s) {
         const dim3 g(grid_for(static_cast<long long>(A.nr) * TPR));
-        if (A.dcol) launch_pdl(k_apply_w<T, TPR, ColDelta>, g, dim3(kBlock), 0, s, A.nr, A.rp, ColDelta{A.dcol}, m, b, u, w);
-        else launch_pdl(k_apply_w<T, TPR>, g, dim3(kBlock), 0, s, A.nr, A.rp, static_cast<const int *>(A.col), m, b, u, w);
+        launch_pdl(k_apply_w<T, TPR>, g, dim3(kBlock), 0, s, A.nr, A.rp, A.col, m, b, u, w);
     }
     template <int TPR>
     static void resid_restrict(const DevMat &R, const DevMat &RA, const T *b, const T *u, T *bc, cudaStream_t s) {
@@ -1027,8 +1055,9 @@ template <class T> struct Launch {
     template <int TPR>
     static void jacobi_first2(const DevMat &A, const T *jac, const T *b, T *u, cudaStream_t s) {
         const dim3 g(grid_for(static_cast<long long>(A.nr) * TPR));
-        if (A.dcol) launch_pdl(k_jacobi_first2<T, TPR, ColDelta>, g, dim3(kBlock), 0, s, A.nr, A.rp, ColDelta{A.dcol}, mvals<T>(A), jac, b, u);
-        else launch_pdl(k_jacobi_first2<T, TPR>, g, dim3(kBlock), 0, s, A.nr, A.rp, static_cast<const int *>(A.col), mvals<T>(A), jac, b, u);
+        launch_pass(A, [&](auto cs) {
+            launch_pdl(k_jacobi_first2<T, TPR, decltype(cs)>, g, dim3(kBlock), 0, s, A.nr, A.rp, cs, mvals<T>(A), jac, b, u);
+        });
     }
     template <int TPR>
     static void outer(const DevMat &A, const double *b, const double *x, T *rT, double *partial, int nblk,
@@ -1051,12 +1080,10 @@ template <class T> struct ChebLaunch {
     static void step(const DevLevel &L, const T *b, const T *uin, T *uout, T *d, T cd, T cr, int first,
                      cudaStream_t s) {
         const dim3 g(grid_for(static_cast<long long>(L.n) * TPR));
-        if (L.A.dcol)
-            launch_pdl(k_cheb_step<T, TPR, ColDelta>, g, dim3(kBlock), 0, s, L.n, L.A.rp, ColDelta{L.A.dcol},
-                       mvals<T>(L.A), dinvvals<T>(L), b, uin, uout, d, cd, cr, first);
-        else
-            launch_pdl(k_cheb_step<T, TPR>, g, dim3(kBlock), 0, s, L.n, L.A.rp, static_cast<const int *>(L.A.col),
-                       mvals<T>(L.A), dinvvals<T>(L), b, uin, uout, d, cd, cr, first);
+        launch_pass(L.A, [&](auto cs) {
+            launch_pdl(k_cheb_step<T, TPR, decltype(cs)>, g, dim3(kBlock), 0, s, L.n, L.A.rp, cs, mvals<T>(L.A),
+                       dinvvals<T>(L), b, uin, uout, d, cd, cr, first);
+        });
     }
 };
 
@@ -1937,6 +1964,15 @@ static void layout_mat(Planner &pl, DevMat &m, const HostCSR &h) {
     m.v32 = pl.take<float>(std::max<long long>(1, h.nnz()));
 }
 
+// A level streams from HBM when the values of A and Q^-1, their columns and
+// four vectors are a quarter more than the 129 MB of L2.  Measured (evict-first
+// values on / off): 2.5M rows (210 MB) residual 27.9 / 32.9 us, Q^-1 pass 26.0
+// / 32.7; 1.1M rows (138 MB) 19.8 / 20.1 and 20.2 / 19.0; 1M rows of a 5-point
+// grid (68 MB) 9.0 / 7.5, so below the line the values are left to L2.  With
+// the row's own values loaded early (load_now) and the policy made once the
+// 2.5M-row passes take 24.4 and 23.7 us, a V-cycle there 604 instead of 682.
+constexpr double kStreamBytes = 161e6;
+
 // Warp slices of the finest level's FP64 operator (see Ell64): rows sorted
 // by length, longest first, within windows of kEllWindow rows (stable, so
 // equal lengths keep their order: a counting sort per window), the slice
@@ -1984,7 +2020,11 @@ static void layout(amg_ctx *c, Planner &pl) {
             layout_mat(pl, L.R, H.R);
             // 16-bit column offsets for the two-pass (HBM-sized) levels; dropped
             // after the upload if some offset does not fit
-            if (!H.fast) L.A.dcol = pl.take<short>(std::max(1, L.A.nnz));
+            if (!H.fast) {
+                L.A.dcol = pl.take<short>(std::max(1, L.A.nnz));
+                const double tb = c->opt.precision == AMG_FP64 ? sizeof(double) : sizeof(float);
+                L.A.stream = (2 * tb + 2) * L.A.nnz + 4 * tb * L.n > kStreamBytes;
+            }
         }
         L.diag = pl.take<double>(L.n);
         L.bx = pl.take<double>(std::max(1, L.A.nnz));

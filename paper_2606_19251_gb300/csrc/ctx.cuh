@@ -16,6 +16,8 @@ struct DevMat {
     int nr = 0, nc = 0, nnz = 0, tpr = 2;
     int *rp = nullptr, *col = nullptr;
     short *dcol = nullptr;                     // col - row in 16 bits (square levels whose offsets fit), or null
+    bool stream = false;                       // this matrix and Q^-1 on its pattern together pass L2 (ColStream)
+    mutable int reverse = 0;                   // direction of its next streaming pass
     double *v64 = nullptr;
     float *v32 = nullptr;
 };
