@@ -1971,7 +1971,7 @@ static void layout_mat(Planner &pl, DevMat &m, const HostCSR &h) {
 // grid (68 MB) 9.0 / 7.5, so below the line the values are left to L2.  With
 // the row's own values loaded early (load_now) and the policy made once the
 // 2.5M-row passes take 24.4 and 23.7 us, a V-cycle there 604 instead of 682.
-constexpr double kStreamBytes = 161e6;
+constexpr double kStreamBytes = 129e6;
 
 // Warp slices of the finest level's FP64 operator (see Ell64): rows sorted
 // by length, longest first, within windows of kEllWindow rows (stable, so
