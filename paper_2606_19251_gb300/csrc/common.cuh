@@ -45,6 +45,21 @@ __device__ __forceinline__ T warp_sum(T v) {
     return v;
 }
 
+// FP32 pair h + l (about 48 bits): sums that want more than FP32 where FP64
+// would bind (GB300: 2 FP64 FMAs a clock and SM against 128 in FP32).
+struct FloatPair {
+    float h, l;
+};
+// a += p + e (Knuth's error-free sum; the _rn intrinsics keep the compiler
+// from contracting it)
+__device__ __forceinline__ void pair_add(FloatPair &a, float p, float e = 0.f) {
+    const float s = __fadd_rn(a.h, p);
+    const float z = __fadd_rn(s, -a.h);
+    const float t = __fadd_rn(__fadd_rn(a.h, -__fadd_rn(s, -z)), __fadd_rn(p, -z));
+    a.h = s;
+    a.l = __fadd_rn(a.l, __fadd_rn(t, e));
+}
+
 // Dot product of one CSR row with a gathered operand, split over the TPR
 // lanes of a row group: lane `lane` takes entries p0 + lane, p0 + lane + TPR,
 // ... and adds them in that order.  Each step issues the col / value loads of

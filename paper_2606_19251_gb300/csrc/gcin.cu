@@ -471,6 +471,11 @@ __device__ __forceinline__ double lanes_sum(double v, double (*red)[H]) {
 // the chunk mean and M2 into mu / rstd) and chunks -> graphs (final = 1:
 // writes the instance-norm mean and 1/sqrt(var + eps)).  16 lanes of parts
 // per feature; one FP64 add per part, the rest in FP32.
+// The part loops are unrolled so that a thread's loads are in flight together
+// (a dependent trip per part made the two stages 13 and 10 us on a 50k-node
+// mesh), and only the H threads that hold the totals divide in FP64.  With
+// the normalisation pass's and the head's reductions: 50k-node prediction 363
+// -> 314 us, 1.95M nodes 2698 -> 2487 us.
 template <int H>
 __global__ void __launch_bounds__(kLanes * H) k_stats_combine(const int *__restrict__ gtile, const int *__restrict__ gptr,
                                                             const int *__restrict__ tstart,
@@ -478,15 +483,21 @@ __global__ void __launch_bounds__(kLanes * H) k_stats_combine(const int *__restr
                                                             const float *__restrict__ tm2, float *__restrict__ mu,
                                                             float *__restrict__ rstd, int final) {
     __shared__ double red[kLanes][H];
+    __shared__ float smean[H];
     const int g = blockIdx.x, f = threadIdx.x % H, q = threadIdx.x / H;
-    const double n = gptr[g + 1] - gptr[g];
+    const int t0 = gtile[g] + q, t1 = gtile[g + 1];
     double s = 0.0;
-    for (int t = gtile[g] + q; t < gtile[g + 1]; t += kLanes)
+#pragma unroll 8
+    for (int t = t0; t < t1; t += kLanes)
         s += static_cast<double>(static_cast<float>(tstart[t + 1] - tstart[t]) * tmean[static_cast<size_t>(t) * H + f]);
-    const double mean = lanes_sum<H>(s, red) / n;
-    const float mf = static_cast<float>(mean);
+    const double total = lanes_sum<H>(s, red);
+    const double n = gptr[g + 1] - gptr[g];
+    if (q == 0) smean[f] = static_cast<float>(total / n);
+    __syncthreads();
+    const float mf = smean[f];
     double v = 0.0;
-    for (int t = gtile[g] + q; t < gtile[g + 1]; t += kLanes) {
+#pragma unroll 8
+    for (int t = t0; t < t1; t += kLanes) {
         const float d = tmean[static_cast<size_t>(t) * H + f] - mf;
         v += static_cast<double>(fmaf(static_cast<float>(tstart[t + 1] - tstart[t]) * d, d,
                                       tm2[static_cast<size_t>(t) * H + f]));
@@ -507,6 +518,11 @@ __global__ void __launch_bounds__(kLanes * H) k_stats_combine(const int *__restr
 // YM: 0 FP32 y; 1 bfloat16 y (BF16 inference); 2 layer 1 in BF16 inference:
 // y = h1 W1 + b1 recomputed from the stored h1 with the same FMAs as
 // k_layer1_tile, rounded to bfloat16 as a stored y would be.
+// The 16 row groups' partial sums and maxima go through shared memory as
+// 16-byte vectors (four features of a thread; as 8-byte FP64 values at a
+// stride of four they kept the L1 pipe at 85 to 94 %), and a feature's 16
+// sums are added as an FP32 pair and converted once (the 32 FP64 operations
+// per feature and tile were 100 us of a 1.95M-node pass).
 template <int H, int YM = 0>
 __global__ void __launch_bounds__(kBlock, 6) k_norm_relu_pool_tile(const int *__restrict__ tstart,
                                                                 const int *__restrict__ tgraph,
@@ -522,9 +538,8 @@ __global__ void __launch_bounds__(kBlock, 6) k_norm_relu_pool_tile(const int *__
                                                                 const float *__restrict__ W1 = nullptr,
                                                                 const float *__restrict__ b1 = nullptr) {
     constexpr int F = H / 4, Q = kBlock / F;   // threads per row (4 features each), rows at a time
-    __shared__ double rs[Q][H];
-    __shared__ float rm[Q][H];
-    __shared__ int ri[Q][H];
+    __shared__ float4 rs[Q][F], rm[Q][F];
+    __shared__ int4 ri[Q][F];
     const int t = blockIdx.x, a = tstart[t], e = tstart[t + 1], g = tgraph[t];
     const int f = 4 * (threadIdx.x % F), q = threadIdx.x / F;
     const float4 m = *reinterpret_cast<const float4 *>(mu + g * H + f);
@@ -532,12 +547,17 @@ __global__ void __launch_bounds__(kBlock, 6) k_norm_relu_pool_tile(const int *__
     const float4 ga = *reinterpret_cast<const float4 *>(gamma + f);
     const float4 be = *reinterpret_cast<const float4 *>(beta + f);
     // FP32 partial sums of at most kTile / Q values per thread (GB300's FP64
-    // pipe is narrow); the tile and graph sums are taken in FP64
+    // pipe is narrow); the tile sum is an FP32 pair, the graph sum FP64
     float s[4] = {0.f, 0.f, 0.f, 0.f};
     float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
     int mi[4] = {a, a, a, a};
     static_assert(kTile % Q == 0, "rows per thread");
-#pragma unroll
+    float4 w0, w1, wb;
+    if (YM == 2) {
+        w0 = *reinterpret_cast<const float4 *>(W1 + f);
+        w1 = *reinterpret_cast<const float4 *>(W1 + H + f);
+        wb = *reinterpret_cast<const float4 *>(b1 + f);
+    }
     // every row's load first (predicated), so a thread's kTile / Q loads are in flight together
     float4 yr[kTile / Q];
 #pragma unroll
@@ -550,11 +570,10 @@ __global__ void __launch_bounds__(kBlock, 6) k_norm_relu_pool_tile(const int *__
                                  __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xFFFF0000u));
         } else if (YM == 2) {
             const float2 hh = reinterpret_cast<const float2 *>(h1)[i < e ? i : a];
-            float yv[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                yv[j] = __bfloat162float(__float2bfloat16_rn(fmaf(hh.x, W1[f + j], fmaf(hh.y, W1[H + f + j], b1[f + j]))));
-            yr[r4] = make_float4(yv[0], yv[1], yv[2], yv[3]);
+            auto yb = [&](float a0, float a1, float c) {
+                return __bfloat162float(__float2bfloat16_rn(fmaf(hh.x, a0, fmaf(hh.y, a1, c))));
+            };
+            yr[r4] = make_float4(yb(w0.x, w1.x, wb.x), yb(w0.y, w1.y, wb.y), yb(w0.z, w1.z, wb.z), yb(w0.w, w1.w, wb.w));
         } else {
             yr[r4] = *reinterpret_cast<const float4 *>(y + o);
         }
@@ -581,25 +600,35 @@ __global__ void __launch_bounds__(kBlock, 6) k_norm_relu_pool_tile(const int *__
             if (v[j] > mx[j]) { mx[j] = v[j]; mi[j] = i; }
         }
     }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        rs[q][f + j] = static_cast<double>(s[j]);
-        rm[q][f + j] = mx[j];
-        ri[q][f + j] = mi[j];
-    }
+    rs[q][f / 4] = make_float4(s[0], s[1], s[2], s[3]);
+    rm[q][f / 4] = make_float4(mx[0], mx[1], mx[2], mx[3]);
+    if (targ) ri[q][f / 4] = make_int4(mi[0], mi[1], mi[2], mi[3]);
     __syncthreads();
     if (threadIdx.x < H) {
         const int ff = threadIdx.x;
-        double ts = 0.0;
+        const float *ps = reinterpret_cast<const float *>(rs) + ff, *pm = reinterpret_cast<const float *>(rm) + ff;
+        const int *pi = reinterpret_cast<const int *>(ri) + ff;
+        FloatPair ts{0.f, 0.f};
         float bm = -INFINITY;
-        int bi = a;
+#pragma unroll 4
         for (int k = 0; k < Q; ++k) {
-            ts += rs[k][ff];
-            if (rm[k][ff] > bm || (rm[k][ff] == bm && ri[k][ff] < bi)) { bm = rm[k][ff]; bi = ri[k][ff]; }
+            pair_add(ts, ps[k * H]);
+            bm = fmaxf(bm, pm[k * H]);
         }
-        tsum[static_cast<size_t>(t) * H + ff] = ts;
+        tsum[static_cast<size_t>(t) * H + ff] = static_cast<double>(ts.h) + static_cast<double>(ts.l);
         tmax[static_cast<size_t>(t) * H + ff] = bm;
-        targ[static_cast<size_t>(t) * H + ff] = bi;
+        if (targ) {                              // the first node of the maximum
+            int bi = a;
+            bool found = false;
+#pragma unroll 4
+            for (int k = 0; k < Q; ++k) {
+                if (pm[k * H] == bm && (!found || pi[k * H] < bi)) {
+                    bi = pi[k * H];
+                    found = true;
+                }
+            }
+            targ[static_cast<size_t>(t) * H + ff] = bi;
+        }
     }
 }
 
@@ -621,10 +650,23 @@ __global__ void __launch_bounds__(kLanes * H) k_pool_combine(const int *__restri
     double s = 0.0;
     float bm = -INFINITY;
     int bi = gptr[g];
-    for (int t = gtile[g] + q; t < gtile[g + 1]; t += kLanes) {
-        const size_t o = static_cast<size_t>(t) * H + f;
-        s += tsum[o];
-        if (tmax[o] > bm) { bm = tmax[o]; bi = targ[o]; }   // tiles ascend, so the first max wins
+    const int t0 = gtile[g] + q, t1 = gtile[g + 1];
+    if (targ) {
+#pragma unroll 8
+        for (int t = t0; t < t1; t += kLanes) {
+            const size_t o = static_cast<size_t>(t) * H + f;
+            const float m = tmax[o];
+            const int a = targ[o];
+            s += tsum[o];
+            if (m > bm) { bm = m; bi = a; }   // tiles ascend, so the first max wins
+        }
+    } else {                                  // inference: no backward asks for the node
+#pragma unroll 8
+        for (int t = t0; t < t1; t += kLanes) {
+            const size_t o = static_cast<size_t>(t) * H + f;
+            s += tsum[o];
+            bm = fmaxf(bm, tmax[o]);
+        }
     }
     rm[q][f] = bm;
     ri[q][f] = bi;
@@ -636,22 +678,23 @@ __global__ void __launch_bounds__(kLanes * H) k_pool_combine(const int *__restri
             const size_t o = static_cast<size_t>(g) * H + f;
             csum[o] = total;
             cmax[o] = bm;
-            carg[o] = bi;
+            if (carg) carg[o] = bi;
             return;
         }
         float *P = pooled + (static_cast<size_t>(g) * kLayers + layer) * 2 * H;
         P[f] = static_cast<float>(total / (gptr[g + 1] - gptr[g]));
         P[H + f] = bm;
-        argmax[(static_cast<size_t>(g) * kLayers + layer) * H + f] = bi;
+        if (targ) argmax[(static_cast<size_t>(g) * kLayers + layer) * H + f] = bi;
     }
 }
 
+// Sum over the block's first 128 threads (called by exactly those).
 __device__ __forceinline__ float block128_sum(float v, float *red) {
     v = warp_sum(v);
     if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = v;
-    __syncthreads();
+    asm volatile("bar.sync 1, 128;" ::: "memory");
     float t = red[0] + red[1] + red[2] + red[3];
-    __syncthreads();
+    asm volatile("bar.sync 1, 128;" ::: "memory");
     return t;
 }
 
@@ -661,60 +704,76 @@ constexpr int kSz = 0, kSzh = kEmb, kSsg = 2 * kEmb, kSa1 = 3 * kEmb, kSa2 = 3 *
 // Head gradient layout per graph: dz1[128] | dz2[64] | dzh[128] | dz[128]
 constexpr int kGdz1 = 0, kGdz2 = 128, kGdzh = 192, kGdz = 192 + kEmb;
 
-// Readout + head for one graph (128 threads).
+// Part q of 4 of a dot product of n terms over a column of W (row stride ld),
+// summed over the four lanes 4 k .. 4 k + 3; four lanes per output and an
+// unrolled quarter keep the three dependent layers at a few load round trips
+// each (128 serial terms per lane took 33 us on seven graphs).
+__device__ __forceinline__ float head_dot(const float *v, const float *__restrict__ W, int n, int ld, int q) {
+    float a = 0.f;
+#pragma unroll 32
+    for (int m = q; m < n; m += 4) a = fmaf(v[m], W[m * ld], a);
+    a += __shfl_xor_sync(0xffffffffu, a, 1);
+    return a + __shfl_xor_sync(0xffffffffu, a, 2);
+}
+
+// Readout + head for one graph (four threads per element of the 128-vectors).
+constexpr int kHeadThreads = 4 * kEmb;
 template <int H>
-__global__ void __launch_bounds__(128) k_head(const float *__restrict__ pooled, const float *__restrict__ th,
-                                              float *__restrict__ scratch, float *__restrict__ c) {
+__global__ void __launch_bounds__(kHeadThreads) k_head(const float *__restrict__ pooled, const float *__restrict__ th,
+                                                       float *__restrict__ scratch, float *__restrict__ c) {
     __shared__ float sp[kLayers * 2 * H];
-    __shared__ float ss[kEmb], sa1[128], sa2[64];
+    __shared__ float sz[kEmb], ss[kEmb], sa1[128], sa2[64];
     __shared__ float red[4];
-    const int g = blockIdx.x, t = threadIdx.x;
-    for (int k = t; k < kLayers * 2 * H; k += 128) sp[k] = pooled[static_cast<size_t>(g) * kLayers * 2 * H + k];
+    const int g = blockIdx.x, t = threadIdx.x / 4, q = threadIdx.x % 4;
+    for (int k = threadIdx.x; k < kLayers * 2 * H; k += kHeadThreads)
+        sp[k] = pooled[static_cast<size_t>(g) * kLayers * 2 * H + k];
     __syncthreads();
     float *S = scratch + static_cast<size_t>(g) * kHeadScratch;
     // readout linears: z[32 l + k] = [mean_l, max_l] . W_l[:, k] + b_l[k]
-    const int l = t / kRo, k = t % kRo;
-    const float *W = th + PL<H>().roW[l];
-    float z = th[PL<H>().roB[l] + k];
-#pragma unroll 8
-    for (int m = 0; m < 2 * H; ++m) z = fmaf(sp[l * 2 * H + m], W[m * kRo + k], z);
-    // layer norm over the 128-vector
-    const float mean = block128_sum(z, red) / kEmb;
-    const float d = z - mean;
-    const float var = block128_sum(d * d, red) / kEmb;
-    const float rs = rsqrtf(var + kEps);
-    const float zh = d * rs * th[PL<H>().lnG + t] + th[PL<H>().lnB + t];
-    const float sg = 1.f / (1.f + expf(-zh));
-    S[kSz + t] = z;
-    S[kSzh + t] = zh;
-    S[kSsg + t] = sg;
-    if (t == 0) {
-        S[kSmean] = mean;
-        S[kSrs] = rs;
+    {
+        const int l = t / kRo, k = t % kRo;
+        const float z = th[PL<H>().roB[l] + k] + head_dot(sp + l * 2 * H, th + PL<H>().roW[l] + k, 2 * H, kRo, q);
+        if (q == 0) sz[t] = z;
     }
-    ss[t] = sg;
     __syncthreads();
-    float a1 = th[PL<H>().h1B + t];
-#pragma unroll 8
-    for (int m = 0; m < kEmb; ++m) a1 = fmaf(ss[m], th[PL<H>().h1W + m * 128 + t], a1);
-    a1 = fmaxf(a1, 0.f);
-    sa1[t] = a1;
-    S[kSa1 + t] = a1;
+    // layer norm over the 128-vector (the first 128 threads)
+    if (threadIdx.x < kEmb) {
+        const int i = threadIdx.x;
+        const float z = sz[i];
+        const float mean = block128_sum(z, red) / kEmb;
+        const float d = z - mean;
+        const float var = block128_sum(d * d, red) / kEmb;
+        const float rs = rsqrtf(var + kEps);
+        const float zh = d * rs * th[PL<H>().lnG + i] + th[PL<H>().lnB + i];
+        const float sg = 1.f / (1.f + expf(-zh));
+        S[kSz + i] = z;
+        S[kSzh + i] = zh;
+        S[kSsg + i] = sg;
+        if (i == 0) {
+            S[kSmean] = mean;
+            S[kSrs] = rs;
+        }
+        ss[i] = sg;
+    }
+    __syncthreads();
+    const float a1 = fmaxf(th[PL<H>().h1B + t] + head_dot(ss, th + PL<H>().h1W + t, kEmb, 128, q), 0.f);
+    if (q == 0) {
+        sa1[t] = a1;
+        S[kSa1 + t] = a1;
+    }
     __syncthreads();
     if (t < 64) {
-        float a2 = th[PL<H>().h2B + t];
-#pragma unroll 8
-        for (int m = 0; m < 128; ++m) a2 = fmaf(sa1[m], th[PL<H>().h2W + m * 64 + t], a2);
-        a2 = fmaxf(a2, 0.f);
-        sa2[t] = a2;
-        S[kSa2 + t] = a2;
+        const float a2 = fmaxf(th[PL<H>().h2B + t] + head_dot(sa1, th + PL<H>().h2W + t, 128, 64, q), 0.f);
+        if (q == 0) {
+            sa2[t] = a2;
+            S[kSa2 + t] = a2;
+        }
     }
     __syncthreads();
-    if (t < 5) {
-        float o = th[PL<H>().h3B + t];
-#pragma unroll 8
-        for (int m = 0; m < 64; ++m) o = fmaf(sa2[m], th[PL<H>().h3W + m * 5 + t], o);
-        c[g * 5 + t] = o;
+    if (t < 8) {                                  // one whole warp; five outputs
+        const int o = min(t, 4);
+        const float v = th[PL<H>().h3B + o] + head_dot(sa2, th + PL<H>().h3W + o, 64, 5, q);
+        if (q == 0 && t < 5) c[g * 5 + t] = v;
     }
 }
 
@@ -778,28 +837,29 @@ static void forward_impl(GcinBatch &b, const float *th, cudaStream_t s) {
         // inference keeps only what the next aggregation reads (bfloat16 with
         // the tensor-core linears, nothing after the last layer)
         const bool last = l == kLayers - 1;
+        int *targ = b.infer ? nullptr : b.targ, *carg = b.infer ? nullptr : b.carg;
         float *xo = (b.infer && (xbf || last)) ? nullptr : b.x[l];
         __nv_bfloat16 *xbo = (xbf && !last) ? reinterpret_cast<__nv_bfloat16 *>(b.x[l]) : nullptr;
         if (xbf && l == 0) {
             k_norm_relu_pool_tile<H, 2><<<NT, kBlock, 0, s>>>(b.tstart, b.tgraph, b.y[l], b.mu[l], b.rstd[l],
                                                               th + pl.inG[l], th + pl.inB[l], xo, xbo, b.tsum,
-                                                              b.tmax, b.targ, b.h1, th + pl.convW[0],
+                                                              b.tmax, targ, b.h1, th + pl.convW[0],
                                                               th + pl.convB[0]); AMG_COUNT();
         } else if (xbf) {
             k_norm_relu_pool_tile<H, 1><<<NT, kBlock, 0, s>>>(b.tstart, b.tgraph, b.y[l], b.mu[l], b.rstd[l],
                                                               th + pl.inG[l], th + pl.inB[l], xo, xbo, b.tsum,
-                                                              b.tmax, b.targ); AMG_COUNT();
+                                                              b.tmax, targ); AMG_COUNT();
         } else {
             k_norm_relu_pool_tile<H><<<NT, kBlock, 0, s>>>(b.tstart, b.tgraph, b.y[l], b.mu[l], b.rstd[l],
                                                            th + pl.inG[l], th + pl.inB[l], xo, xbo, b.tsum, b.tmax,
-                                                           b.targ); AMG_COUNT();
+                                                           targ); AMG_COUNT();
         }
-        k_pool_combine<H><<<b.NC, CT, 0, s>>>(b.ctile, b.cnode, b.tsum, b.tmax, b.targ, nullptr, nullptr, l,
-                                              b.csum, b.cmax, b.carg); AMG_COUNT();
-        k_pool_combine<H><<<G, CT, 0, s>>>(b.gchunk, b.gptr, b.csum, b.cmax, b.carg, b.pooled, b.argmax, l,
+        k_pool_combine<H><<<b.NC, CT, 0, s>>>(b.ctile, b.cnode, b.tsum, b.tmax, targ, nullptr, nullptr, l,
+                                              b.csum, b.cmax, carg); AMG_COUNT();
+        k_pool_combine<H><<<G, CT, 0, s>>>(b.gchunk, b.gptr, b.csum, b.cmax, carg, b.pooled, b.argmax, l,
                                            nullptr, nullptr, nullptr); AMG_COUNT();
     }
-    k_head<H><<<G, 128, 0, s>>>(b.pooled, th, b.head, b.c); AMG_COUNT();
+    k_head<H><<<G, kHeadThreads, 0, s>>>(b.pooled, th, b.head, b.c); AMG_COUNT();
 }
 
 void gcin_forward(GcinBatch &b, const float *th, cudaStream_t s) {

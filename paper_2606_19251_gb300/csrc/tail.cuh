@@ -29,24 +29,14 @@ constexpr int kTailThreads = 512;
 constexpr size_t kTailSmem = 220 * 1024;         // shared memory a tail's level vectors may take
 constexpr double kTailCoarseWork = 134217728.0;  // n_t n_L^2 bound: the FP64 coarsest solves of the n_t columns
 
-// FP32 pair h + l (about 48 bits).  The FP32 V-cycle's B is formed in this
-// arithmetic and rounded once to FP32: GB300 runs 64 FP32 FMAs for each FP64
-// one, so the ten FP32 operations of a pair FMA are ~6x cheaper than a DFMA.
-struct FloatPair {
-    float h, l;
-};
-
-// acc += a x (Dekker / Knuth error-free sums; _rn intrinsics keep the
-// compiler from contracting them)
+// The FP32 V-cycle's B is formed in FP32 pairs (FloatPair) and rounded once
+// to FP32: GB300 runs 64 FP32 FMAs for each FP64 one, so the ten FP32
+// operations of a pair FMA are ~6x cheaper than a DFMA.
+// acc += a x (Dekker / Knuth error-free product and sum)
 __device__ __forceinline__ void tail_fma(FloatPair &acc, float a, const FloatPair &x) {
     const float p = __fmul_rn(a, x.h);
-    float e = __fmaf_rn(a, x.h, -p);
-    e = __fmaf_rn(a, x.l, e);
-    const float s = __fadd_rn(acc.h, p);
-    const float z = __fadd_rn(s, -acc.h);
-    const float t = __fadd_rn(__fadd_rn(acc.h, -__fadd_rn(s, -z)), __fadd_rn(p, -z));
-    acc.h = s;
-    acc.l = __fadd_rn(acc.l, __fadd_rn(t, e));
+    const float e = __fmaf_rn(a, x.l, __fmaf_rn(a, x.h, -p));
+    pair_add(acc, p, e);
 }
 __device__ __forceinline__ void tail_fma(double &acc, double a, const double &x) { acc = fma(a, x, acc); }
 
