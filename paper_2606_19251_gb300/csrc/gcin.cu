@@ -41,13 +41,18 @@ __host__ __device__ constexpr int num_params() { return make_layout(H).total; }
 // batch construction
 // ---------------------------------------------------------------------------
 __global__ void k_cat_graph(int n, int nnz, const int *__restrict__ rp, const int *__restrict__ col,
-                            const double *__restrict__ v, int node_off, int edge_off, int g,
-                            int *__restrict__ rp_out, int *__restrict__ col_out, float *__restrict__ w_out,
-                            double *__restrict__ w64_out, int *__restrict__ gid) {
+                            const double *__restrict__ v, const double *__restrict__ diag, int node_off,
+                            int edge_off, int g, int *__restrict__ rp_out, int *__restrict__ col_out,
+                            float *__restrict__ w_out, double *__restrict__ w64_out, double *__restrict__ x0,
+                            int *__restrict__ gid) {
     const int t = blockIdx.x * kBlock + threadIdx.x;
     if (t < n) {
         rp_out[node_off + t] = rp[t] + edge_off;
         gid[node_off + t] = g;
+        // raw features [a_ii, deg_i] (Algorithm 1 step 3; deg = off-diagonal
+        // pattern entries, every row holding its diagonal)
+        x0[2 * static_cast<size_t>(node_off + t)] = diag[t];
+        x0[2 * static_cast<size_t>(node_off + t) + 1] = static_cast<double>(rp[t + 1] - rp[t] - 1);
     }
     if (t < nnz) {
         col_out[edge_off + t] = col[t] + node_off;
@@ -103,7 +108,6 @@ static void batch_layout(GcinBatch &b, Planner &pl, bool backward) {
     b.head = pl.take<float>(G * kHeadScratch);
     b.c = pl.take<float>(G * 5);
     b.err = pl.take<int>(4);
-    b.wtile = pl.take<unsigned char>(static_cast<size_t>(kLayers - 1) * kHidden * kHidden * 2);
     if (backward) {
         b.dc = pl.take<float>(G * 5);
         b.dhead = pl.take<float>(G * kHeadGrad);
@@ -190,8 +194,8 @@ int gcin_batch_build(GcinBatch &b, int n_problems, amg_ctx *const *problems, cud
     for (int m = 0; m < n_problems; ++m) {
         for (const auto &L : problems[m]->lev) {
             const int work = std::max(L.n, L.A.nnz);
-            k_cat_graph<<<grid_for(work), kBlock, 0, s>>>(L.n, L.A.nnz, L.A.rp, L.A.col, L.A.v64, gptr[g],
-                                                          static_cast<int>(eoff), g, b.rp, b.col, b.w, b.w64,
+            k_cat_graph<<<grid_for(work), kBlock, 0, s>>>(L.n, L.A.nnz, L.A.rp, L.A.col, L.A.v64, L.diag, gptr[g],
+                                                          static_cast<int>(eoff), g, b.rp, b.col, b.w, b.w64, b.x0,
                                                           b.gid); AMG_COUNT();
             eoff += L.A.nnz;
             ++g;
@@ -211,21 +215,6 @@ int gcin_batch_build(GcinBatch &b, int n_problems, amg_ctx *const *problems, cud
 // ---------------------------------------------------------------------------
 // forward kernels
 // ---------------------------------------------------------------------------
-// x0_i = [a_ii, deg_i] (Algorithm 1 step 3; deg = off-diagonal pattern entries)
-__global__ void k_feat0(int N, const int *__restrict__ rp, const int *__restrict__ col,
-                        const double *__restrict__ w64, double *__restrict__ x0) {
-    int i = blockIdx.x * kBlock + threadIdx.x;
-    if (i >= N) return;
-    double d = 0.0;
-    int deg = 0;
-    for (int p = rp[i]; p < rp[i + 1]; ++p) {
-        if (col[p] == i) d += w64[p];
-        else ++deg;
-    }
-    x0[2 * i] = d;
-    x0[2 * i + 1] = static_cast<double>(deg);
-}
-
 // mean and M2 (sum of squared deviations) per feature of the tile's y rows;
 // the block's threads form kBlock / H groups of H (one thread per feature)
 template <int H>
@@ -263,75 +252,115 @@ __device__ __forceinline__ void tile_stats(const float (*sY)[H + 1], int nn, flo
     }
 }
 
-// Layer 1: h = A_hat x0 (FP64 sums of the raw features, four threads per
-// node), y = h W + b (K = 2: FMA units); tile stats.
 // bfloat16 copy of four FP32 values (round to nearest even), as 8 bytes
 __device__ __forceinline__ uint2 bf16x4(float a, float b, float c, float d) {
     __nv_bfloat162 lo = __floats2bfloat162_rn(a, b), hi = __floats2bfloat162_rn(c, d);
     return make_uint2(*reinterpret_cast<unsigned *>(&lo), *reinterpret_cast<unsigned *>(&hi));
 }
 
-// YB (BF16 inference): y only feeds the tile statistics (FP32); h1 is stored
-// and the normalisation pass recomputes y from it.
+// Layer 1: h = A_hat x0 (FP64 sums of the raw features, two lanes per node),
+// y = h W + b (K = 2: FMA units); tile stats.  YB (BF16 inference): y only
+// feeds the tile statistics (FP32); h1 is stored and the normalisation pass
+// recomputes y from it (8 bytes per node instead of 128).
+// Bound by the FP64 pipe (two DFMAs per entry, 2 lanes a clock and SM): two
+// lanes per node waste less of it on short rows than four and exchange their
+// sums with one addition each.  A thread owns one feature and keeps its column
+// of W, so y needs no shared memory; its two accumulators per statistic are
+// the groups of tile_stats.  1.95M nodes: 228 us with four lanes, y staged in
+// shared memory and W read per node (L1 pipe 84 %).
+constexpr int kL1Threads = 2 * kTile;
 template <int H, bool YB = false>
-__global__ void __launch_bounds__(kBlock) k_layer1_tile(const int *__restrict__ rp, const int *__restrict__ col,
-                                                        const double *__restrict__ w64, const double *__restrict__ x0,
-                                                        const float *__restrict__ W, const float *__restrict__ bias,
-                                                        const int *__restrict__ tstart, float *__restrict__ h1,
-                                                        float *__restrict__ y, float *__restrict__ tmean,
-                                                        float *__restrict__ tm2) {
-    __shared__ float sY[kTile][H + 1];
-    __shared__ float sH[kTile][2];
+__global__ void __launch_bounds__(kL1Threads, 12) k_layer1_tile(const int *__restrict__ rp, const int *__restrict__ col,
+                                                                const double *__restrict__ w64,
+                                                                const double *__restrict__ x0,
+                                                                const float *__restrict__ W,
+                                                                const float *__restrict__ bias,
+                                                                const int *__restrict__ tstart, float *__restrict__ h1,
+                                                                float *__restrict__ y, float *__restrict__ tmean,
+                                                                float *__restrict__ tm2) {
+    constexpr int Q = kL1Threads / H;            // threads per feature; 2 Q groups of nodes
+    __shared__ float2 sH[kTile];
+    __shared__ float red[2 * Q][H];
     const int t = blockIdx.x, a = tstart[t], nn = tstart[t + 1] - a;
     {
-        static_assert(kTile * 4 == kBlock, "four threads per node of a tile");
-        // four threads per node (kTile * 4 = kBlock), entries p0 + q, p0 + q + 4,
-        // ...; the four partial sums are added pairwise, the same in each lane
-        const int k = threadIdx.x >> 2, q = threadIdx.x & 3;
+        const int k = threadIdx.x >> 1, q = threadIdx.x & 1;
         double a0 = 0.0, a1 = 0.0;
         if (k < nn) {
-            const int i = a + k;
-            for (int p = rp[i] + q; p < rp[i + 1]; p += 4) {
-                const double wv = w64[p];
-                const double2 xj = reinterpret_cast<const double2 *>(x0)[col[p]];
-                a0 += wv * xj.x;
-                a1 += wv * xj.y;
+            const int e = rp[a + k + 1];
+            for (int p = rp[a + k] + q; p < e; p += 8) {
+                int c[4];
+                double w[4];
+                double2 x[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    c[j] = p + 2 * j < e ? col[p + 2 * j] : 0;
+                    w[j] = p + 2 * j < e ? w64[p + 2 * j] : 0.0;
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (p + 2 * j < e) x[j] = reinterpret_cast<const double2 *>(x0)[c[j]];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (p + 2 * j < e) {
+                        a0 = fma(w[j], x[j].x, a0);
+                        a1 = fma(w[j], x[j].y, a1);
+                    }
+                }
             }
         }
-        a0 += __shfl_xor_sync(0xffffffffu, a0, 1);
-        a1 += __shfl_xor_sync(0xffffffffu, a1, 1);
-        a0 += __shfl_xor_sync(0xffffffffu, a0, 2);
-        a1 += __shfl_xor_sync(0xffffffffu, a1, 2);
-        if (k < nn && q == 0) {
-            const float h0 = static_cast<float>(a0), hv1 = static_cast<float>(a1);
-            reinterpret_cast<float2 *>(h1)[a + k] = make_float2(h0, hv1);
-            sH[k][0] = h0;
-            sH[k][1] = hv1;
+        // lane 0 ends with the first feature's sum, lane 1 with the second's
+        const double other = __shfl_xor_sync(0xffffffffu, q ? a0 : a1, 1);
+        const float h = static_cast<float>((q ? a1 : a0) + other);
+        if (k < nn) {
+            h1[2 * static_cast<size_t>(a) + threadIdx.x] = h;
+            reinterpret_cast<float *>(sH)[threadIdx.x] = h;
         }
     }
+    const int f = threadIdx.x % H, q = threadIdx.x / H;
+    const float w0 = W[f], w1 = W[H + f], bf = bias[f];
     __syncthreads();
-    // 64 nodes x H features: thread -> node k = tid / 4, features FT (tid % 4) .. + FT - 1
-    constexpr int FT = H / 4;
-    const int k = threadIdx.x / 4, f0 = FT * (threadIdx.x % 4);
-    if (k < nn) {
-        const float h0 = sH[k][0], hv1 = sH[k][1];
-        float out[FT];
-#pragma unroll
-        for (int q = 0; q < FT; ++q) {
-            const int f = f0 + q;
-            out[q] = fmaf(h0, W[f], fmaf(hv1, W[H + f], bias[f]));
-            sY[k][f] = out[q];
-        }
-        // BF16 inference stores no y: the normalisation pass forms it again
-        // from h1 (8 bytes per node instead of 128)
-        if (!YB) {
-            float4 *yo = reinterpret_cast<float4 *>(y + static_cast<size_t>(a + k) * H + f0);
-#pragma unroll
-            for (int q = 0; q < FT / 4; ++q) yo[q] = make_float4(out[4 * q], out[4 * q + 1], out[4 * q + 2], out[4 * q + 3]);
+    auto yval = [&](int k) {
+        const float2 h = sH[k];
+        return fmaf(h.x, w0, fmaf(h.y, w1, bf));
+    };
+    float s0 = 0.f, s1 = 0.f;                    // groups q and q + Q of the tile's nodes
+#pragma unroll 4
+    for (int k = q; k < nn; k += 2 * Q) {
+        const float v0 = yval(k);
+        s0 += v0;
+        if (!YB) y[static_cast<size_t>(a + k) * H + f] = v0;
+        if (k + Q < nn) {
+            const float v1 = yval(k + Q);
+            s1 += v1;
+            if (!YB) y[static_cast<size_t>(a + k + Q) * H + f] = v1;
         }
     }
-    __syncthreads();
-    tile_stats<H>(sY, nn, tmean + static_cast<size_t>(t) * H, tm2 + static_cast<size_t>(t) * H);
+    auto total = [&](float g0, float g1) {       // the groups' sums in group order
+        red[q][f] = g0;
+        red[q + Q][f] = g1;
+        __syncthreads();
+        float r = red[0][f];
+#pragma unroll
+        for (int j = 1; j < 2 * Q; ++j) r += red[j][f];
+        __syncthreads();
+        return r;
+    };
+    const float m = total(s0, s1) / nn;
+    float v0 = 0.f, v1 = 0.f;
+#pragma unroll 4
+    for (int k = q; k < nn; k += 2 * Q) {
+        const float d0 = yval(k) - m;
+        v0 = fmaf(d0, d0, v0);
+        if (k + Q < nn) {
+            const float d1 = yval(k + Q) - m;
+            v1 = fmaf(d1, d1, v1);
+        }
+    }
+    const float m2 = total(v0, v1);
+    if (q == 0) {
+        tmean[static_cast<size_t>(t) * H + f] = m;
+        tm2[static_cast<size_t>(t) * H + f] = m2;
+    }
 }
 
 // h_i = sum_p w_p x_{col p} with L = H / 4 lanes per row and 32 / L rows per
@@ -805,18 +834,13 @@ static void forward_impl(GcinBatch &b, const float *th, cudaStream_t s) {
     constexpr int CT = combine_threads<H>();
     const bool xb16 = b.bf16 && b.infer;   // BF16 inference on the tensor cores
     const bool xbf = xb16 && kInferBF16Acts;   // ... with y and x stored in bfloat16
-    if (xb16) {
-        k_pack_wtile<H><<<kLayers - 1, kBlock, 0, s>>>(th + pl.convW[1], th + pl.convW[2], th + pl.convW[3],
-                                                      b.wtile); AMG_COUNT();
-    }
-    k_feat0<<<grid_for(N), kBlock, 0, s>>>(N, b.rp, b.col, b.w64, b.x0); AMG_COUNT();
     for (int l = 0; l < kLayers; ++l) {
         if (l == 0 && xbf) {
-            k_layer1_tile<H, true><<<NT, kBlock, 0, s>>>(b.rp, b.col, b.w64, b.x0, th + pl.convW[0],
+            k_layer1_tile<H, true><<<NT, kL1Threads, 0, s>>>(b.rp, b.col, b.w64, b.x0, th + pl.convW[0],
                                                          th + pl.convB[0], b.tstart, b.h1, b.y[0], b.tmean,
                                                          b.tm2); AMG_COUNT();
         } else if (l == 0) {
-            k_layer1_tile<H><<<NT, kBlock, 0, s>>>(b.rp, b.col, b.w64, b.x0, th + pl.convW[0], th + pl.convB[0],
+            k_layer1_tile<H><<<NT, kL1Threads, 0, s>>>(b.rp, b.col, b.w64, b.x0, th + pl.convW[0], th + pl.convB[0],
                                                    b.tstart, b.h1, b.y[0], b.tmean, b.tm2); AMG_COUNT();
         } else if (xb16) {
             k_agg_lin_tc<H, true><<<(NT + 1) / 2, kBlock, tc_smem<H>(), s>>>(
@@ -860,6 +884,17 @@ static void forward_impl(GcinBatch &b, const float *th, cudaStream_t s) {
                                            nullptr, nullptr, nullptr); AMG_COUNT();
     }
     k_head<H><<<G, kHeadThreads, 0, s>>>(b.pooled, th, b.head, b.c); AMG_COUNT();
+}
+
+// The layer 2..4 B tiles of BF16 inference, laid out when the parameters are
+// loaded (gnn_load_params) instead of in every prediction.
+static void pack_wtiles(int H, const float *th, unsigned char *out, cudaStream_t s) {
+    const ParamLayout &pl = host_layout(H);
+    if (H == kHidden32)
+        k_pack_wtile<kHidden32><<<kLayers - 1, kBlock, 0, s>>>(th + pl.convW[1], th + pl.convW[2], th + pl.convW[3], out);
+    else
+        k_pack_wtile<kHidden><<<kLayers - 1, kBlock, 0, s>>>(th + pl.convW[1], th + pl.convW[2], th + pl.convW[3], out);
+    AMG_COUNT();
 }
 
 void gcin_forward(GcinBatch &b, const float *th, cudaStream_t s) {
@@ -1342,7 +1377,10 @@ int gnn_load_params(amg_ctx *c, const float *theta, long long n) {
     if (e != cudaSuccess) return ctx_cuda_check(c, e, "cudaSetDevice");
     if (!c->gnn) {
         c->gnn = new GcinEngine();
-        e = cudaMalloc(&c->gnn->theta, sizeof(float) * kNumParams);
+        // the parameters and, 256-byte aligned behind them, the packed B tiles
+        const size_t tb = (sizeof(float) * kNumParams + 255) / 256 * 256;
+        e = cudaMalloc(&c->gnn->theta, tb + static_cast<size_t>(kLayers - 1) * kHidden * kHidden * 2);
+        if (e == cudaSuccess) c->gnn->wtile = reinterpret_cast<unsigned char *>(c->gnn->theta) + tb;
         if (e != cudaSuccess) {
             delete c->gnn;
             c->gnn = nullptr;
@@ -1350,6 +1388,10 @@ int gnn_load_params(amg_ctx *c, const float *theta, long long n) {
         }
     }
     e = cudaMemcpyAsync(c->gnn->theta, theta, sizeof(float) * n, cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess) {
+        pack_wtiles(H, c->gnn->theta, c->gnn->wtile, c->stream);
+        e = cudaGetLastError();
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return ctx_cuda_check(c, e, "upload params");
     c->gnn->have_params = true;
@@ -1376,6 +1418,7 @@ int gnn_predict_coeffs(amg_ctx *c, double *c_out) {
     g->batch.bf16 = (c->opt.gnn_precision == AMG_GNN_BF16) ? 1 : 0;
     g->batch.infer = 1;
     g->batch.hidden = g->hidden;
+    g->batch.wtile = g->wtile;
     // forward + smoother assembly (straight from the device coefficients) run
     // as one CUDA graph, captured once per batch and arithmetic: ~40 small
     // kernels whose host launch cost would otherwise exceed their run time

@@ -79,7 +79,7 @@ struct GcinBatch {
     int hidden = kHidden;                // GCIN width H of the parameters (64 or 32)
     int bf16 = 0;                        // layers 2..4 on tensor cores (BF16 operands, FP32 accumulation)
     int infer = 0;                       // inference only: no h, x in bfloat16 with bf16 (nothing kept for a backward)
-    unsigned char *wtile = nullptr;      // layers 2..4: round(W)^T as BF16 tensor-core B tiles (bf16 inference)
+    const unsigned char *wtile = nullptr;   // the engine's packed B tiles (bf16 inference)
     int *err = nullptr;                  // device error flag (tensor-core wait timeout)
     long long E = 0;
     int *rp = nullptr, *col = nullptr, *gptr = nullptr, *gid = nullptr;
@@ -139,6 +139,7 @@ constexpr int kHeadGrad = 128 /*dz1*/ + 64 /*dz2*/ + kEmb /*dzh*/ + kEmb /*dz*/;
 
 struct GcinEngine {
     float *theta = nullptr;              // room for the widest network
+    unsigned char *wtile = nullptr;      // layers 2..4: round(W)^T as BF16 tensor-core B tiles, packed from theta
     bool have_params = false;
     int hidden = kHidden;                // width of the loaded parameters
     GcinBatch batch;

@@ -10,7 +10,7 @@
 //      per row, each lane reading its entry's (column, weight) pair) and store
 //      h in BF16 into the A tile (128 x H, K-major, canonical no-swizzle
 //      core-matrix layout); W^T goes to the B tile (H x H, K-major) in BF16
-//      (pre-packed once per inference in BF16 inference);
+//      (packed with the parameters in BF16 inference);
 //   2. one thread issues H / 16 x tcgen05.mma.kind::f16 (M 128, N H, K 16)
 //      into an H-column TMEM accumulator and commits to an mbarrier;
 //   3. warps 0..3 read their 32 TMEM lanes (rows) with tcgen05.ld, add the
