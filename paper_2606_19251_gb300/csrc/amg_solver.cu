@@ -332,16 +332,116 @@ __global__ void __launch_bounds__(kBlock) k_coarse(int n, const double *__restri
 // ---------------------------------------------------------------------------
 // kernels: FP64 outer loop with deterministic norms
 // ---------------------------------------------------------------------------
+// Sum of the block's values into *out: one warp adds eight per lane and then
+// its lanes, 13 FP64 instructions per block instead of 5 per warp and 5 more
+// (GB300's FP64 pipe takes 16 cycles for each; outer residual of 2.5M rows
+// 76.8 -> 65.1 us).
 __device__ __forceinline__ void block_partial(double v, double *out) {
-    __shared__ double red[kBlock / 32];
-    v = warp_sum(v);
-    if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = v;
+    __shared__ double red[kBlock];
+    red[threadIdx.x] = v;
     __syncthreads();
     if (threadIdx.x < 32) {
-        double w = threadIdx.x < kBlock / 32 ? red[threadIdx.x] : 0.0;
+        double w = red[threadIdx.x];
+#pragma unroll
+        for (int k = 1; k < kBlock / 32; ++k) w += red[threadIdx.x + 32 * k];
         w = warp_sum(w);
         if (threadIdx.x == 0) out[blockIdx.x] = w;
     }
+}
+
+// True in every thread of the block that arrives last at *ticket; the other
+// blocks' partial sums are then visible to it (read them with __ldcg).  The
+// last block resets the ticket, so each launch finds it at zero.
+__device__ __forceinline__ bool last_block(unsigned *ticket) {
+    __shared__ int s_last;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        const unsigned t = atomicAdd(ticket, 1u);
+        s_last = (t == gridDim.x - 1);
+        if (s_last) {
+            *ticket = 0u;
+            __threadfence();
+        }
+    }
+    __syncthreads();
+    return s_last != 0;
+}
+
+// Fixed-order sum of the np partials by one block; the total in thread 0.
+__device__ __forceinline__ double sum_blocks(const double *part, int np) {
+    __shared__ double red[kBlock / 32];
+    double v = 0.0;
+    for (int i = threadIdx.x; i < np; i += kBlock) v += __ldcg(part + i);
+    v = warp_sum(v);
+    __syncthreads();
+    if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = v;
+    __syncthreads();
+    double t = 0.0;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < kBlock / 32; ++w) t += red[w];
+    return t;
+}
+
+// Smallest of hist[k - off - 9 .. k - off].
+__device__ __forceinline__ double window_min(const double *hist, int k, int off) {
+    double m = hist[k - off];
+    for (int j = 1; j < 10; ++j) m = fmin(m, hist[k - off - j]);
+    return m;
+}
+
+// What the last block of a pass does with the sum of its partials.
+struct NormRule {
+    SolveState *st = nullptr;              // null: nothing
+    double *hist = nullptr;
+    int mode = 0;                          // 0: ||b||; 1: residual history and stopping rule
+    int use_cond = 0;                      // set the solve graph's WHILE condition
+    cudaGraphConditionalHandle cond = 0;
+};
+
+// mode 1: residual history entry k and the stopping rule (Sec. 4 tolerance,
+// divergence, stagnation, iteration cap).  One thread.
+__device__ __forceinline__ void apply_norm_rule(const NormRule &R, double sum) {
+    SolveState *st = R.st;
+    const double nrm = sqrt(sum);
+    if (R.mode == 0) {
+        st->bnorm = nrm > 0.0 ? nrm : 1.0;
+        return;
+    }
+    if (st->breakdown) {   // conjugate gradients broke down: the iterate and history stay
+        st->status = AMG_ERR_DIVERGED;
+        if (R.use_cond) cudaGraphSetConditional(R.cond, 0u);
+        return;
+    }
+    double *hist = R.hist;
+    const int k = st->k;
+    const double rel = nrm / st->bnorm;
+    hist[k] = rel;
+    int status = kRunning;
+    if (k == 0) {
+        st->r0 = nrm;
+        if (!isfinite(nrm)) status = AMG_ERR_DIVERGED;
+        else if (rel <= st->tol) status = AMG_OK;
+        else if (st->max_iter <= 0) status = AMG_ERR_MAXITER;
+    } else {
+        if (!isfinite(nrm) || nrm > 1e3 * st->r0) status = AMG_ERR_DIVERGED;
+        else if (rel <= st->tol) status = AMG_OK;
+        else if (k >= 10 && st->stall > 0.0 && rel > st->stall * hist[k - 10]) status = kStalled;
+        else if (k >= 20 && window_min(hist, k, 0) > 0.99 * window_min(hist, k, 10)) status = AMG_ERR_STAGNATED;
+        else if (k >= st->max_iter) status = AMG_ERR_MAXITER;
+    }
+    st->status = status;
+    st->k = k + 1;
+    if (R.use_cond) cudaGraphSetConditional(R.cond, status == kRunning ? 1u : 0u);
+}
+
+// The norm of a pass: the block's partial, and in the last block the total
+// and its rule, without a launch of its own (a one-block kernel of 2 to 3 us
+// per iteration).
+__device__ __forceinline__ void norm_of_blocks(double v, double *partial, const NormRule &R) {
+    block_partial(v, partial);
+    if (!R.st || !last_block(&R.st->ticket)) return;
+    const double sum = sum_blocks(partial, gridDim.x);
+    if (threadIdx.x == 0) apply_norm_rule(R, sum);
 }
 
 // r = b - A x (FP64), rT = (T) r, r64 = r (when given), partial[block] = sum
@@ -351,7 +451,7 @@ __global__ void __launch_bounds__(kBlock) k_outer_resid(int n, const int *__rest
                                                         const int *__restrict__ col, const double *__restrict__ a,
                                                         const double *__restrict__ b, const double *__restrict__ x,
                                                         T *__restrict__ rT, double *__restrict__ partial,
-                                                        double *__restrict__ r64) {
+                                                        double *__restrict__ r64, NormRule rule) {
     pdl_wait_and_release();
     constexpr int RPB = kBlock / TPR;
     const int lane = threadIdx.x % TPR;
@@ -371,7 +471,7 @@ __global__ void __launch_bounds__(kBlock) k_outer_resid(int n, const int *__rest
             sq += r * r;
         }
     }
-    block_partial(sq, partial);
+    norm_of_blocks(sq, partial, rule);
 }
 
 // The finest level's FP64 operator for the outer-loop passes, in warp
@@ -419,7 +519,8 @@ __device__ __forceinline__ double ell_dot(const Ell64 &E, int s, int lane, doubl
 template <class T>
 __global__ void __launch_bounds__(kBlock) k_outer_ell(Ell64 E, const double *__restrict__ b,
                                                       const double *__restrict__ x, T *__restrict__ rT,
-                                                      double *__restrict__ partial, double *__restrict__ r64) {
+                                                      double *__restrict__ partial, double *__restrict__ r64,
+                                                      NormRule rule) {
     pdl_wait_and_release();
     const int lane = threadIdx.x & 31;
     double sq = 0.0;
@@ -433,12 +534,30 @@ __global__ void __launch_bounds__(kBlock) k_outer_ell(Ell64 E, const double *__r
             sq = fma(r, r, sq);
         }
     }
-    block_partial(sq, partial);
+    norm_of_blocks(sq, partial, rule);
+}
+
+// The step length of a conjugate-gradient iteration, in the last block of
+// the pass that forms q = A p: alpha = (z.r) / (p.q); p.q <= 0 (or not
+// finite) is a breakdown.
+__device__ __forceinline__ void pcg_alpha(double pq_part, double *partial, SolveState *st) {
+    block_partial(pq_part, partial);
+    if (!last_block(&st->ticket)) return;
+    const double pq = sum_blocks(partial, gridDim.x);
+    if (threadIdx.x != 0) return;
+    if (st->breakdown || !(pq > 0.0) || !isfinite(pq)) {
+        st->breakdown = 1;
+    } else {
+        st->alpha = st->rho / pq;
+        st->rho_old = st->rho;
+        st->restart = 0;
+    }
 }
 
 // q = A p (FP64) over warp slices, partial p.q
 __global__ void __launch_bounds__(kBlock) k_pcg_spmv_ell(Ell64 E, const double *__restrict__ p,
-                                                         double *__restrict__ q, double *__restrict__ partial) {
+                                                         double *__restrict__ q, double *__restrict__ partial,
+                                                         SolveState *st) {
     pdl_wait_and_release();
     const int lane = threadIdx.x & 31;
     double pq = 0.0;
@@ -451,7 +570,7 @@ __global__ void __launch_bounds__(kBlock) k_pcg_spmv_ell(Ell64 E, const double *
             pq = fma(p[row], a, pq);
         }
     }
-    block_partial(pq, partial);
+    pcg_alpha(pq, partial, st);
 }
 
 // d_p = col_p - i in 16 bits for row i; flag = 1 if some offset does not fit
@@ -489,12 +608,12 @@ __global__ void __launch_bounds__(kBlock) k_ell_fill(int nslice, const int *__re
     }
 }
 
-__global__ void __launch_bounds__(kBlock) k_sqnorm_partial(int n, const double *__restrict__ v,
-                                                           double *__restrict__ partial) {
+__global__ void __launch_bounds__(kBlock) k_sqnorm(int n, const double *__restrict__ v, double *__restrict__ partial,
+                                                   NormRule rule) {
     pdl_wait_and_release();
     double sq = 0.0;
     for (int i = blockIdx.x * kBlock + threadIdx.x; i < n; i += gridDim.x * kBlock) sq += v[i] * v[i];
-    block_partial(sq, partial);
+    norm_of_blocks(sq, partial, rule);
 }
 
 // ---------------------------------------------------------------------------
@@ -515,56 +634,49 @@ __device__ __forceinline__ double sum_partials(const double *__restrict__ part, 
 }
 
 __device__ __forceinline__ void block_partial2(double a, double b, double *outa, double *outb) {
-    __shared__ double ra[kBlock / 32], rb[kBlock / 32];
-    a = warp_sum(a);
-    b = warp_sum(b);
-    if (threadIdx.x % 32 == 0) {
-        ra[threadIdx.x / 32] = a;
-        rb[threadIdx.x / 32] = b;
-    }
+    block_partial(a, outa);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double ta = 0.0, tb = 0.0;
-        for (int w = 0; w < kBlock / 32; ++w) {
-            ta += ra[w];
-            tb += rb[w];
-        }
-        outa[blockIdx.x] = ta;
-        outb[blockIdx.x] = tb;
-    }
+    block_partial(b, outb);
 }
 
-// z = (double) e (the V-cycle's output); partials of z.r and z.r_prev
+// z = (double) e (the V-cycle's output); in the last block rho = z.r and
+// beta = (z.r - z.r_prev) / rho_old (0 after a restart); z.r <= 0 (or not
+// finite) is a breakdown.  The scalars of an iteration are formed once here,
+// in pcg_alpha and in the norm rule: summed and divided in every block of the
+// next pass they cost 50 to 60 FP64 instructions per warp (262k rows: 88 us of
+// a 202 us iteration, now 39 of 153).
 template <class T>
 __global__ void __launch_bounds__(kBlock) k_pcg_dots(int n, const T *__restrict__ e, const double *__restrict__ r,
                                                      const double *__restrict__ rprev, double *__restrict__ z,
-                                                     double *__restrict__ pzr, double *__restrict__ pzrp) {
+                                                     double *__restrict__ pzr, double *__restrict__ pzrp,
+                                                     SolveState *st) {
     pdl_wait_and_release();
     double a = 0.0, b = 0.0;
     for (int i = blockIdx.x * kBlock + threadIdx.x; i < n; i += gridDim.x * kBlock) {
         const double zi = static_cast<double>(e[i]);
         z[i] = zi;
-        a += zi * r[i];
-        b += zi * rprev[i];
+        a = fma(zi, r[i], a);
+        b = fma(zi, rprev[i], b);
     }
     block_partial2(a, b, pzr, pzrp);
-}
-
-// p = z (restart) or p = z + beta p with beta = (z.r - z.r_prev) / rho_old;
-// z.r <= 0 (or not finite) is a breakdown.
-__global__ void __launch_bounds__(kBlock) k_pcg_dir(int n, const double *__restrict__ z, double *__restrict__ p,
-                                                    const double *__restrict__ pzr, const double *__restrict__ pzrp,
-                                                    int np, SolveState *st) {
-    pdl_wait_and_release();
-    __shared__ double red[kBlock / 32];
-    const double rho = sum_partials(pzr, np, red);
-    const double zrp = sum_partials(pzrp, np, red);
+    if (!last_block(&st->ticket)) return;
+    const double rho = sum_blocks(pzr, gridDim.x), zrp = sum_blocks(pzrp, gridDim.x);
+    if (threadIdx.x != 0) return;
     if (!(rho > 0.0) || !isfinite(rho) || st->breakdown) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) st->breakdown = 1;
+        st->breakdown = 1;
         return;
     }
+    st->rho = rho;
+    st->beta = st->restart ? 0.0 : (rho - zrp) / st->rho_old;
+}
+
+// p = z (restart) or p = z + beta p
+__global__ void __launch_bounds__(kBlock) k_pcg_dir(int n, const double *__restrict__ z, double *__restrict__ p,
+                                                    const SolveState *st) {
+    pdl_wait_and_release();
+    if (st->breakdown) return;
     const bool restart = st->restart != 0;
-    const double beta = restart ? 0.0 : (rho - zrp) / st->rho_old;
+    const double beta = st->beta;
     for (int i = blockIdx.x * kBlock + threadIdx.x; i < n; i += gridDim.x * kBlock)
         p[i] = restart ? z[i] : z[i] + beta * p[i];
 }
@@ -573,7 +685,8 @@ __global__ void __launch_bounds__(kBlock) k_pcg_dir(int n, const double *__restr
 template <int TPR>
 __global__ void __launch_bounds__(kBlock) k_pcg_spmv(int n, const int *__restrict__ rp, const int *__restrict__ col,
                                                      const double *__restrict__ a, const double *__restrict__ p,
-                                                     double *__restrict__ q, double *__restrict__ partial) {
+                                                     double *__restrict__ q, double *__restrict__ partial,
+                                                     SolveState *st) {
     pdl_wait_and_release();
     constexpr int RPB = kBlock / TPR;
     const int lane = threadIdx.x % TPR;
@@ -588,25 +701,20 @@ __global__ void __launch_bounds__(kBlock) k_pcg_spmv(int n, const int *__restric
             pq += p[row] * acc;
         }
     }
-    block_partial(pq, partial);
+    pcg_alpha(pq, partial, st);
 }
 
-// alpha = (z.r) / (p.Ap); x += alpha p; r_prev = r; r -= alpha q; rT = (T) r;
-// partial ||r||^2.  p.Ap <= 0 (or not finite) is a breakdown.
+// x += alpha p; r_prev = r; r -= alpha q; rT = (T) r; ||r|| and the stopping
+// rule in the last block.  Nothing after a breakdown.
 template <class T>
 __global__ void __launch_bounds__(kBlock) k_pcg_update(int n, double *__restrict__ x, double *__restrict__ r,
                                                        double *__restrict__ rprev, const double *__restrict__ p,
                                                        const double *__restrict__ q, T *__restrict__ rT,
-                                                       const double *__restrict__ pzr, const double *__restrict__ ppq,
-                                                       int np, SolveState *st, double *__restrict__ prr) {
+                                                       double *__restrict__ prr, NormRule rule) {
     pdl_wait_and_release();
-    __shared__ double red[kBlock / 32];
-    const double rho = sum_partials(pzr, np, red);
-    const double pq = sum_partials(ppq, np, red);
-    const bool bad = st->breakdown || !(pq > 0.0) || !isfinite(pq);
     double rr = 0.0;
-    if (!bad) {
-        const double alpha = rho / pq;
+    if (!rule.st->breakdown) {
+        const double alpha = rule.st->alpha;
         for (int i = blockIdx.x * kBlock + threadIdx.x; i < n; i += gridDim.x * kBlock) {
             x[i] += alpha * p[i];
             const double ri = r[i];
@@ -614,18 +722,10 @@ __global__ void __launch_bounds__(kBlock) k_pcg_update(int n, double *__restrict
             rprev[i] = ri;
             r[i] = rn;
             rT[i] = static_cast<T>(rn);
-            rr += rn * rn;
+            rr = fma(rn, rn, rr);
         }
     }
-    block_partial(rr, prr);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        if (bad) {
-            st->breakdown = 1;
-        } else {
-            st->rho_old = rho;
-            st->restart = 0;
-        }
-    }
+    norm_of_blocks(rr, prr, rule);
 }
 
 __global__ void k_state_init(SolveState *st, double tol, int max_iter, double stall) {
@@ -640,6 +740,7 @@ __global__ void k_state_init(SolveState *st, double tol, int max_iter, double st
     st->rho_old = 0.0;
     st->restart = 1;
     st->breakdown = 0;
+    st->ticket = 0u;
 }
 
 // Continue a stalled solve with another smoother (history and count go on).
@@ -648,60 +749,6 @@ __global__ void k_state_continue(SolveState *st) {
     st->status = kRunning;
     st->stall = 0.0;
     st->restart = 1;
-}
-
-// Smallest of hist[k - off - 9 .. k - off].
-__device__ __forceinline__ double window_min(const double *hist, int k, int off) {
-    double m = hist[k - off];
-    for (int j = 1; j < 10; ++j) m = fmin(m, hist[k - off - j]);
-    return m;
-}
-
-// Sum the partials in a fixed order.  mode 0: ||b||.  mode 1: residual
-// history entry k and the stopping rule (Sec. 4 tolerance, divergence,
-// stagnation, iteration cap).
-__global__ void __launch_bounds__(1024) k_norm_final(const double *__restrict__ partial, int np, SolveState *st,
-                                                     double *__restrict__ hist, int mode, int use_cond,
-                                                     cudaGraphConditionalHandle cond) {
-    pdl_wait_and_release();
-    __shared__ double red[32];
-    double v = 0.0;
-    for (int i = threadIdx.x; i < np; i += 1024) v += partial[i];
-    v = warp_sum(v);
-    if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = v;
-    __syncthreads();
-    if (threadIdx.x >= 32) return;
-    v = warp_sum(red[threadIdx.x]);
-    if (threadIdx.x != 0) return;
-    const double nrm = sqrt(v);
-    if (mode == 0) {
-        st->bnorm = nrm > 0.0 ? nrm : 1.0;
-        return;
-    }
-    if (st->breakdown) {   // conjugate gradients broke down: the iterate and history stay
-        st->status = AMG_ERR_DIVERGED;
-        if (use_cond) cudaGraphSetConditional(cond, 0u);
-        return;
-    }
-    const int k = st->k;
-    const double rel = nrm / st->bnorm;
-    hist[k] = rel;
-    int status = kRunning;
-    if (k == 0) {
-        st->r0 = nrm;
-        if (!isfinite(nrm)) status = AMG_ERR_DIVERGED;
-        else if (rel <= st->tol) status = AMG_OK;
-        else if (st->max_iter <= 0) status = AMG_ERR_MAXITER;
-    } else {
-        if (!isfinite(nrm) || nrm > 1e3 * st->r0) status = AMG_ERR_DIVERGED;
-        else if (rel <= st->tol) status = AMG_OK;
-        else if (k >= 10 && st->stall > 0.0 && rel > st->stall * hist[k - 10]) status = kStalled;
-        else if (k >= 20 && window_min(hist, k, 0) > 0.99 * window_min(hist, k, 10)) status = AMG_ERR_STAGNATED;
-        else if (k >= st->max_iter) status = AMG_ERR_MAXITER;
-    }
-    st->status = status;
-    st->k = k + 1;
-    if (use_cond) cudaGraphSetConditional(cond, status == kRunning ? 1u : 0u);
 }
 
 // An empty dependent launch: the floor of one step of a chain of
@@ -1061,13 +1108,14 @@ template <class T> struct Launch {
     }
     template <int TPR>
     static void outer(const DevMat &A, const double *b, const double *x, T *rT, double *partial, int nblk,
-                      double *r64, cudaStream_t s) {
+                      double *r64, const NormRule &rule, cudaStream_t s) {
         launch_pdl(k_outer_resid<T, TPR>, dim3(nblk), dim3(kBlock), 0, s, A.nr, A.rp, A.col, A.v64, b, x, rT, partial,
-                   r64);
+                   r64, rule);
     }
     template <int TPR>
-    static void pcg_spmv(const DevMat &A, const double *p, double *q, double *partial, int nblk, cudaStream_t s) {
-        launch_pdl(k_pcg_spmv<TPR>, dim3(nblk), dim3(kBlock), 0, s, A.nr, A.rp, A.col, A.v64, p, q, partial);
+    static void pcg_spmv(const DevMat &A, const double *p, double *q, double *partial, int nblk, SolveState *st,
+                         cudaStream_t s) {
+        launch_pdl(k_pcg_spmv<TPR>, dim3(nblk), dim3(kBlock), 0, s, A.nr, A.rp, A.col, A.v64, p, q, partial, st);
     }
 };
 
@@ -1144,8 +1192,8 @@ static int outer_blocks(const DevMat &A) {
 // FP64 outer residual with nb = outer_blocks(A) partial sums.
 template <class T>
 static void L_outer(const DevMat &A, const double *b, const double *x, T *rT, double *partial, int nb,
-                    cudaStream_t s, double *r64 = nullptr) {
-    TPR_DISPATCH(A.tpr, Launch<T>::template outer, A, b, x, rT, partial, nb, r64, s);
+                    cudaStream_t s, double *r64, const NormRule &rule) {
+    TPR_DISPATCH(A.tpr, Launch<T>::template outer, A, b, x, rT, partial, nb, r64, rule, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -1715,28 +1763,34 @@ static int ell_blocks(const amg_ctx *c) {
     return static_cast<int>(std::max(1LL, std::min<long long>(need, static_cast<long long>(kNumSMs) * kOuterBlocksPerSM)));
 }
 
-// FP64 outer residual r = b - A x with its FP32 copy and norm partials;
-// returns the number of partial sums.
+// FP64 outer residual r = b - A x with its FP32 copy, norm partials and the
+// norm's rule.
 template <class T>
-static int launch_outer(amg_ctx *c, cudaStream_t s, T *rT, double *r64) {
+static void launch_outer(amg_ctx *c, cudaStream_t s, T *rT, double *r64, const NormRule &rule) {
     if (c->ell_nslice > 0) {
-        const int nb = ell_blocks(c);
-        launch_pdl(k_outer_ell<T>, dim3(nb), dim3(kBlock), 0, s, ell_of(c), static_cast<const double *>(c->db),
-                   static_cast<const double *>(c->dx), rT, c->partials, r64);
-        return nb;
+        launch_pdl(k_outer_ell<T>, dim3(ell_blocks(c)), dim3(kBlock), 0, s, ell_of(c), static_cast<const double *>(c->db),
+                   static_cast<const double *>(c->dx), rT, c->partials, r64, rule);
+        return;
     }
     const DevMat &A = c->lev[0].A;
-    const int nb = outer_blocks(A);
-    L_outer<T>(A, c->db, c->dx, rT, c->partials, nb, s, r64);
-    return nb;
+    L_outer<T>(A, c->db, c->dx, rT, c->partials, outer_blocks(A), s, r64, rule);
+}
+
+static NormRule norm_rule(const amg_ctx *c, int mode, int use_cond = 0, cudaGraphConditionalHandle cond = 0) {
+    NormRule r;
+    r.st = c->state;
+    r.hist = c->hist;
+    r.mode = mode;
+    r.use_cond = use_cond;
+    r.cond = cond;
+    return r;
 }
 
 template <class T>
 static void enqueue_outer_residual(amg_ctx *c, cudaStream_t s, int use_cond = 0,
                                    cudaGraphConditionalHandle cond = 0) {
     double *r64 = (c->opt.outer == AMG_OUTER_PCG) ? c->pcg : nullptr;   // CG keeps r in FP64
-    const int nb = launch_outer<T>(c, s, reinterpret_cast<T *>(c->lev[0].vb), r64);
-    launch_pdl(k_norm_final, dim3(1), dim3(1024), 0, s, c->partials, nb, c->state, c->hist, 1, use_cond, cond);
+    launch_outer<T>(c, s, reinterpret_cast<T *>(c->lev[0].vb), r64, norm_rule(c, 1, use_cond, cond));
 }
 
 // One conjugate-gradient iteration preconditioned by a V-cycle on r (held in
@@ -1750,18 +1804,16 @@ static void enqueue_pcg_iteration(amg_ctx *c, cudaStream_t s, int use_cond, cuda
     double *P0 = c->partials, *P1 = P0 + c->n_partials, *P2 = P1 + c->n_partials, *P3 = P2 + c->n_partials;
     T *e = vcycle_level<T>(c, 0, s);
     launch_pdl(k_pcg_dots<T>, dim3(nb), dim3(kBlock), 0, s, n, static_cast<const T *>(e),
-               static_cast<const double *>(r), static_cast<const double *>(rprev), z, P0, P1);
+               static_cast<const double *>(r), static_cast<const double *>(rprev), z, P0, P1, c->state);
     launch_pdl(k_pcg_dir, dim3(nb), dim3(kBlock), 0, s, n, static_cast<const double *>(z), p,
-               static_cast<const double *>(P0), static_cast<const double *>(P1), nb, c->state);
+               static_cast<const SolveState *>(c->state));
     if (c->ell_nslice > 0)
-        launch_pdl(k_pcg_spmv_ell, dim3(nb), dim3(kBlock), 0, s, ell_of(c), static_cast<const double *>(p), q, P2);
+        launch_pdl(k_pcg_spmv_ell, dim3(nb), dim3(kBlock), 0, s, ell_of(c), static_cast<const double *>(p), q, P2,
+                   c->state);
     else
-        TPR_DISPATCH(A.tpr, Launch<T>::template pcg_spmv, A, p, q, P2, nb, s);
+        TPR_DISPATCH(A.tpr, Launch<T>::template pcg_spmv, A, p, q, P2, nb, c->state, s);
     launch_pdl(k_pcg_update<T>, dim3(nb), dim3(kBlock), 0, s, n, c->dx, r, rprev, static_cast<const double *>(p),
-               static_cast<const double *>(q), reinterpret_cast<T *>(c->lev[0].vb), static_cast<const double *>(P0),
-               static_cast<const double *>(P2), nb, c->state, P3);
-    launch_pdl(k_norm_final, dim3(1), dim3(1024), 0, s, static_cast<const double *>(P3), nb, c->state, c->hist, 1,
-               use_cond, cond);
+               static_cast<const double *>(q), reinterpret_cast<T *>(c->lev[0].vb), P3, norm_rule(c, 1, use_cond, cond));
 }
 
 template <class T>
@@ -1771,8 +1823,7 @@ static void enqueue_init(amg_ctx *c, cudaStream_t s, double tol, int max_iter) {
     const double stall = (c->smoother == AMG_SMOOTHER_GNN) ? c->stall_ratio : 0.0;
     cudaMemsetAsync(c->dflag + 1, 0, sizeof(int), s);   // wavefront wait flag of this solve
     launch_pdl(k_state_init, dim3(1), dim3(1), 0, s, c->state, tol, max_iter, stall);
-    launch_pdl(k_sqnorm_partial, dim3(nb), dim3(kBlock), 0, s, n0, c->db, c->partials);
-    launch_pdl(k_norm_final, dim3(1), dim3(1024), 0, s, c->partials, nb, c->state, c->hist, 0, 0, 0);
+    launch_pdl(k_sqnorm, dim3(nb), dim3(kBlock), 0, s, n0, c->db, c->partials, norm_rule(c, 0));
     enqueue_outer_residual<T>(c, s);
 }
 
@@ -3090,7 +3141,7 @@ int kernel_launch(amg_ctx *c, int which, int l, int reps, cudaStream_t s, double
         case AMG_K_OUTER: {
             const DevMat &A = c->lev[0].A;
             by = 4.0 * (A.nr + 1) + 12.0 * A.nnz + 16.0 * A.nr + tb * A.nr;
-            for (int k = 0; k < reps; ++k) launch_outer<T>(c, s, reinterpret_cast<T *>(c->lev[0].vr), nullptr);
+            for (int k = 0; k < reps; ++k) launch_outer<T>(c, s, reinterpret_cast<T *>(c->lev[0].vr), nullptr, NormRule{});
             break;
         }
         case AMG_K_MASWEEP:

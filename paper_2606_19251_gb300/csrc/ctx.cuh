@@ -83,6 +83,8 @@ struct SolveState {
     double rho_old; // conjugate gradients: z.r of the previous iteration
     int restart;    // conjugate gradients: next direction is p = z
     int breakdown;  // conjugate gradients: z.r or p.Ap not positive
+    double rho, alpha, beta;   // conjugate gradients: z.r, step length, direction update of this iteration
+    unsigned ticket;           // blocks done with the running pass (last_block)
 };
 
 // Whole-solve CUDA graph: a kernel node copies the device-side status into
