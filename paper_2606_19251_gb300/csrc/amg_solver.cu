@@ -393,20 +393,15 @@ __device__ __forceinline__ double window_min(const double *hist, int k, int off)
 struct NormRule {
     SolveState *st = nullptr;              // null: nothing
     double *hist = nullptr;
-    int mode = 0;                          // 0: ||b||; 1: residual history and stopping rule
     int use_cond = 0;                      // set the solve graph's WHILE condition
     cudaGraphConditionalHandle cond = 0;
 };
 
-// mode 1: residual history entry k and the stopping rule (Sec. 4 tolerance,
+// Residual history entry k and the stopping rule (Sec. 4 tolerance,
 // divergence, stagnation, iteration cap).  One thread.
 __device__ __forceinline__ void apply_norm_rule(const NormRule &R, double sum) {
     SolveState *st = R.st;
     const double nrm = sqrt(sum);
-    if (R.mode == 0) {
-        st->bnorm = nrm > 0.0 ? nrm : 1.0;
-        return;
-    }
     if (st->breakdown) {   // conjugate gradients broke down: the iterate and history stay
         st->status = AMG_ERR_DIVERGED;
         if (R.use_cond) cudaGraphSetConditional(R.cond, 0u);
@@ -608,12 +603,29 @@ __global__ void __launch_bounds__(kBlock) k_ell_fill(int nslice, const int *__re
     }
 }
 
-__global__ void __launch_bounds__(kBlock) k_sqnorm(int n, const double *__restrict__ v, double *__restrict__ partial,
-                                                   NormRule rule) {
+// Start of a solve: the state's fields and ||b||, in the last block of the
+// pass over b (its ticket is the only field that must hold a value before).
+__global__ void __launch_bounds__(kBlock) k_solve_init(int n, const double *__restrict__ b, double *__restrict__ partial,
+                                                       SolveState *st, double tol, int max_iter, double stall) {
     pdl_wait_and_release();
     double sq = 0.0;
-    for (int i = blockIdx.x * kBlock + threadIdx.x; i < n; i += gridDim.x * kBlock) sq += v[i] * v[i];
-    norm_of_blocks(sq, partial, rule);
+    for (int i = blockIdx.x * kBlock + threadIdx.x; i < n; i += gridDim.x * kBlock) sq += b[i] * b[i];
+    block_partial(sq, partial);
+    if (!last_block(&st->init_ticket)) return;
+    const double nrm = sqrt(sum_blocks(partial, gridDim.x));
+    if (threadIdx.x != 0) return;
+    st->k = 0;
+    st->status = kRunning;
+    st->max_iter = max_iter;
+    st->tol = tol;
+    st->bnorm = nrm > 0.0 ? nrm : 1.0;
+    st->r0 = 0.0;
+    st->stall = stall;
+    st->rho_old = 0.0;
+    st->restart = 1;
+    st->breakdown = 0;
+    st->ticket = 0u;
+    st->wait_error = 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -726,21 +738,6 @@ __global__ void __launch_bounds__(kBlock) k_pcg_update(int n, double *__restrict
         }
     }
     norm_of_blocks(rr, prr, rule);
-}
-
-__global__ void k_state_init(SolveState *st, double tol, int max_iter, double stall) {
-    pdl_wait_and_release();
-    st->k = 0;
-    st->status = kRunning;
-    st->max_iter = max_iter;
-    st->tol = tol;
-    st->bnorm = 1.0;
-    st->r0 = 0.0;
-    st->stall = stall;
-    st->rho_old = 0.0;
-    st->restart = 1;
-    st->breakdown = 0;
-    st->ticket = 0u;
 }
 
 // Continue a stalled solve with another smoother (history and count go on).
@@ -1363,7 +1360,7 @@ static WfChain<T> wf_chain_for(amg_ctx *c, int l, const T *b) {
     a.pv = mvals<T>(L.P);
     a.b = b;
     for (int k = 0; k < kWfBufs; ++k) a.v[k] = reinterpret_cast<T *>(L.wf_buf + static_cast<size_t>(k) * L.n);
-    a.err = c->dflag + 1;
+    a.err = &c->state->wait_error;
     return ch;
 }
 
@@ -1776,11 +1773,10 @@ static void launch_outer(amg_ctx *c, cudaStream_t s, T *rT, double *r64, const N
     L_outer<T>(A, c->db, c->dx, rT, c->partials, outer_blocks(A), s, r64, rule);
 }
 
-static NormRule norm_rule(const amg_ctx *c, int mode, int use_cond = 0, cudaGraphConditionalHandle cond = 0) {
+static NormRule norm_rule(const amg_ctx *c, int use_cond = 0, cudaGraphConditionalHandle cond = 0) {
     NormRule r;
     r.st = c->state;
     r.hist = c->hist;
-    r.mode = mode;
     r.use_cond = use_cond;
     r.cond = cond;
     return r;
@@ -1790,7 +1786,7 @@ template <class T>
 static void enqueue_outer_residual(amg_ctx *c, cudaStream_t s, int use_cond = 0,
                                    cudaGraphConditionalHandle cond = 0) {
     double *r64 = (c->opt.outer == AMG_OUTER_PCG) ? c->pcg : nullptr;   // CG keeps r in FP64
-    launch_outer<T>(c, s, reinterpret_cast<T *>(c->lev[0].vb), r64, norm_rule(c, 1, use_cond, cond));
+    launch_outer<T>(c, s, reinterpret_cast<T *>(c->lev[0].vb), r64, norm_rule(c, use_cond, cond));
 }
 
 // One conjugate-gradient iteration preconditioned by a V-cycle on r (held in
@@ -1813,7 +1809,7 @@ static void enqueue_pcg_iteration(amg_ctx *c, cudaStream_t s, int use_cond, cuda
     else
         TPR_DISPATCH(A.tpr, Launch<T>::template pcg_spmv, A, p, q, P2, nb, c->state, s);
     launch_pdl(k_pcg_update<T>, dim3(nb), dim3(kBlock), 0, s, n, c->dx, r, rprev, static_cast<const double *>(p),
-               static_cast<const double *>(q), reinterpret_cast<T *>(c->lev[0].vb), P3, norm_rule(c, 1, use_cond, cond));
+               static_cast<const double *>(q), reinterpret_cast<T *>(c->lev[0].vb), P3, norm_rule(c, use_cond, cond));
 }
 
 template <class T>
@@ -1821,9 +1817,8 @@ static void enqueue_init(amg_ctx *c, cudaStream_t s, double tol, int max_iter) {
     const int n0 = c->lev[0].n;
     const int nb = std::min(grid_for(n0), kNumSMs * 8);
     const double stall = (c->smoother == AMG_SMOOTHER_GNN) ? c->stall_ratio : 0.0;
-    cudaMemsetAsync(c->dflag + 1, 0, sizeof(int), s);   // wavefront wait flag of this solve
-    launch_pdl(k_state_init, dim3(1), dim3(1), 0, s, c->state, tol, max_iter, stall);
-    launch_pdl(k_sqnorm, dim3(nb), dim3(kBlock), 0, s, n0, c->db, c->partials, norm_rule(c, 0));
+    launch_pdl(k_solve_init, dim3(nb), dim3(kBlock), 0, s, n0, static_cast<const double *>(c->db), c->partials, c->state,
+               tol, max_iter, stall);
     enqueue_outer_residual<T>(c, s);
 }
 
@@ -1937,9 +1932,21 @@ static int ensure_graph(amg_ctx *c) {
     return AMG_OK;
 }
 
-// Solve on the staging buffers c->db / c->dx.
+// The solve's state, the first history entries and (x_out) the iterate to the
+// caller: one wait for the stream.
+static int solve_outputs(amg_ctx *c, cudaStream_t s, double *x_out, cudaMemcpyKind kind) {
+    if (x_out) CK(cudaMemcpyAsync(x_out, c->dx, sizeof(double) * c->lev[0].n, kind, s));
+    CK(cudaMemcpyAsync(c->h_state, c->state, kHistOffset + sizeof(double) * std::min(c->hist_cap, kHistFirst),
+                       cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    return AMG_OK;
+}
+
+// Solve on the staging buffers c->db / c->dx; the iterate goes to x_out (may
+// be null).
 template <class T>
-static int solve_staged(amg_ctx *c, cudaStream_t s, double tol, int *n_vc, double *hist) {
+static int solve_staged(amg_ctx *c, cudaStream_t s, double tol, int *n_vc, double *hist, double *x_out,
+                        cudaMemcpyKind kind) {
     const int max_iter = c->opt.max_iter;
     int rc = ensure_tail(c, s);
     if (!rc) rc = ensure_graph<T>(c);
@@ -1948,8 +1955,7 @@ static int solve_staged(amg_ctx *c, cudaStream_t s, double tol, int *n_vc, doubl
     CKL("solve init launch");
     const SolveGraph &G = c->sgraph[c->smoother + 3 * c->opt.outer];
     CK(cudaGraphLaunch(G.exec, s));
-    CK(cudaMemcpyAsync(c->h_state, c->state, sizeof(SolveState), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
+    if ((rc = solve_outputs(c, s, x_out, kind))) return rc;
     int nh = c->h_state->k;
     g_launches.fetch_add(1 + static_cast<long long>(nh - 1) * G.body_kernels);
     c->last_rerouted = 0;
@@ -1964,17 +1970,20 @@ static int solve_staged(amg_ctx *c, cudaStream_t s, double tol, int *n_vc, doubl
         launch_pdl(k_state_continue, dim3(1), dim3(1), 0, s, c->state);
         const SolveGraph &GJ = c->sgraph[AMG_SMOOTHER_JACOBI + 3 * c->opt.outer];
         CK(cudaGraphLaunch(GJ.exec, s));
-        CK(cudaMemcpyAsync(c->h_state, c->state, sizeof(SolveState), cudaMemcpyDeviceToHost, s));
-        CK(cudaStreamSynchronize(s));
+        if ((rc = solve_outputs(c, s, x_out, kind))) return rc;
         g_launches.fetch_add(1 + static_cast<long long>(c->h_state->k - nh) * GJ.body_kernels);
         nh = c->h_state->k;
     }
     if (n_vc) *n_vc = nh - 1;
-    if (hist) CK(cudaMemcpyAsync(hist, c->hist, sizeof(double) * nh, cudaMemcpyDeviceToHost, s));
-    int wferr = 0;
-    CK(cudaMemcpyAsync(&wferr, c->dflag + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    if (wferr) {
+    if (hist) {
+        const int first = std::min(nh, std::min(c->hist_cap, kHistFirst));
+        std::memcpy(hist, reinterpret_cast<const char *>(c->h_state) + kHistOffset, sizeof(double) * first);
+        if (nh > first) {
+            CK(cudaMemcpyAsync(hist + first, c->hist + first, sizeof(double) * (nh - first), cudaMemcpyDeviceToHost, s));
+            CK(cudaStreamSynchronize(s));
+        }
+    }
+    if (c->h_state->wait_error) {
         ctx_fail(c, "a wavefront smoothing kernel gave up waiting for a dependency (bounded wait ran out)");
         return AMG_ERR_DEVICE_FLAG;
     }
@@ -2150,8 +2159,10 @@ static void layout(amg_ctx *c, Planner &pl) {
     c->partials = pl.take<double>(5 * c->n_partials);  // up to 5 partial sums per block
     c->scal = pl.take<double>(nlev);
     c->wcoef = pl.take<float>(8 * static_cast<size_t>(nlev));
-    c->state = pl.take<SolveState>(1);
-    c->hist = pl.take<double>(c->opt.max_iter + 1);
+    c->hist_cap = c->opt.max_iter + 1;
+    char *out = pl.take<char>(kHistOffset + sizeof(double) * c->hist_cap);
+    c->state = reinterpret_cast<SolveState *>(out);
+    c->hist = out ? reinterpret_cast<double *>(out + kHistOffset) : nullptr;
     c->dflag = pl.take<int>(4);
     c->dcol_flag = pl.take<int>(nlev);
 }
@@ -2380,7 +2391,7 @@ int amg_create(amg_ctx **ctx, const amg_options *opt) {
     }
     c->opt = o;
     e = cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaMallocHost(&c->h_state, sizeof(SolveState));
+    if (e == cudaSuccess) e = cudaMallocHost(&c->h_state, kHistOffset + sizeof(double) * kHistFirst);
     if (e != cudaSuccess) {
         g_create_err = std::string("stream/pinned allocation: ") + cudaGetErrorString(e);
         if (c->stream) cudaStreamDestroy(c->stream);
@@ -2770,9 +2781,10 @@ int amg_get_smoother(const amg_ctx *cc, int level, double *q_out) {
     return AMG_OK;
 }
 
-static int solve_dispatch(amg_ctx *c, cudaStream_t s, double tol, int *n_vc, double *hist) {
-    if (c->opt.precision == AMG_FP64) return solve_staged<double>(c, s, tol, n_vc, hist);
-    return solve_staged<float>(c, s, tol, n_vc, hist);
+static int solve_dispatch(amg_ctx *c, cudaStream_t s, double tol, int *n_vc, double *hist, double *x_out = nullptr,
+                          cudaMemcpyKind kind = cudaMemcpyDeviceToDevice) {
+    if (c->opt.precision == AMG_FP64) return solve_staged<double>(c, s, tol, n_vc, hist, x_out, kind);
+    return solve_staged<float>(c, s, tol, n_vc, hist, x_out, kind);
 }
 
 static int check_ready(amg_ctx *c) {
@@ -2793,10 +2805,8 @@ int amg_solve(amg_ctx *c, const double *b, double *x, double rtol, int *n_vc, do
     cudaStream_t s = c->stream;
     CK(cudaMemcpyAsync(c->db, b, sizeof(double) * n0, cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(c->dx, x, sizeof(double) * n0, cudaMemcpyHostToDevice, s));
-    rc = solve_dispatch(c, s, rtol, n_vc, hist);
+    rc = solve_dispatch(c, s, rtol, n_vc, hist, x, cudaMemcpyDeviceToHost);
     if (rc == AMG_ERR_CUDA) return rc;
-    CK(cudaMemcpyAsync(x, c->dx, sizeof(double) * n0, cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
     if (rc != AMG_OK && rc != AMG_ERR_DEVICE_FLAG)
         c->err = "solve ended without reaching the tolerance (status " + std::to_string(rc) + ")";
     else if (c->last_rerouted) c->err = "learned smoother stalled; solve finished with Jacobi (rerouted)";
@@ -2815,10 +2825,8 @@ int amg_solve_device(amg_ctx *c, const double *d_b, double *d_x, double rtol, vo
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     CK(cudaMemcpyAsync(c->db, d_b, sizeof(double) * n0, cudaMemcpyDeviceToDevice, s));
     CK(cudaMemcpyAsync(c->dx, d_x, sizeof(double) * n0, cudaMemcpyDeviceToDevice, s));
-    rc = solve_dispatch(c, s, rtol, n_vc, hist);
+    rc = solve_dispatch(c, s, rtol, n_vc, hist, d_x, cudaMemcpyDeviceToDevice);
     if (rc == AMG_ERR_CUDA) return rc;
-    CK(cudaMemcpyAsync(d_x, c->dx, sizeof(double) * n0, cudaMemcpyDeviceToDevice, s));
-    CK(cudaStreamSynchronize(s));
     if (rc != AMG_OK && rc != AMG_ERR_DEVICE_FLAG)
         c->err = "solve ended without reaching the tolerance (status " + std::to_string(rc) + ")";
     else if (c->last_rerouted) c->err = "learned smoother stalled; solve finished with Jacobi (rerouted)";
@@ -2874,7 +2882,7 @@ static void smooth_level_device(amg_ctx *c, int l, const double *d_b, double *d_
     launch_pdl(k_convert<double, T>, dim3(grid_for(n)), dim3(kBlock), 0, s, n, d_u, u);
     T *res = nullptr;
     if (nsw > 0 && L.wf && c->smoother != AMG_SMOOTHER_CHEB) {
-        cudaMemsetAsync(c->dflag + 1, 0, sizeof(int), s);
+        cudaMemsetAsync(&c->state->wait_error, 0, sizeof(int), s);
         res = wf_smooth<T>(c, l, s, b, u, nsw);
     }
     if (!res) res = smooth<T>(c, l, s, b, u, reinterpret_cast<T *>(L.vt), reinterpret_cast<T *>(L.vr), nsw, false);
@@ -3177,7 +3185,7 @@ int kernel_launch(amg_ctx *c, int which, int l, int reps, cudaStream_t s, double
             by = pre ? smooth_bytes(c, L, tb, c->opt.nu1, true) + pass_bytes(L.A, tb, L.n, 2)
                      : pass_bytes(L.P, tb, L.P.nc, 2) + smooth_bytes(c, L, tb, c->opt.nu2, false);
             const T *e = reinterpret_cast<const T *>(c->lev[l + 1].vu);
-            cudaMemsetAsync(c->dflag + 1, 0, sizeof(int), s);
+            cudaMemsetAsync(&c->state->wait_error, 0, sizeof(int), s);
             for (int k = 0; k < reps; ++k) {
                 int ui = 0, ri = 0;
                 if (pre) wf_pre<T>(c, l, s, b, ui, ri);

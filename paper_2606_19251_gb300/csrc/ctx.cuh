@@ -85,7 +85,15 @@ struct SolveState {
     int breakdown;  // conjugate gradients: z.r or p.Ap not positive
     double rho, alpha, beta;   // conjugate gradients: z.r, step length, direction update of this iteration
     unsigned ticket;           // blocks done with the running pass (last_block)
+    unsigned init_ticket;      // the same for the pass that starts a solve (it resets the fields above)
+    int wait_error;            // a wavefront kernel's bounded wait ran out
 };
+
+// The state and the first entries of the residual history lie together, so a
+// solve's host outputs are one copy and one synchronisation.
+constexpr size_t kHistOffset = 256;            // bytes from the state to the history
+constexpr int kHistFirst = 512;                // history entries copied with the state
+static_assert(sizeof(SolveState) <= kHistOffset, "the history follows the state");
 
 // Whole-solve CUDA graph: a kernel node copies the device-side status into
 // a conditional handle, and a WHILE node repeats the captured iteration body
@@ -128,7 +136,8 @@ struct amg_ctx {
     int n_partials = 0;
     double *scal = nullptr;                    // device s_l
     amg::SolveState *state = nullptr;
-    double *hist = nullptr;                    // max_iter + 1
+    double *hist = nullptr;                    // max_iter + 1, kHistOffset behind the state
+    int hist_cap = 0;
     int *dflag = nullptr;
     int *dcol_flag = nullptr;                  // per level: 1 if a column offset does not fit 16 bits
     char *arena = nullptr;
