@@ -3384,6 +3384,54 @@ extern "C" int amg_residual_norm_noalloc(int n, long long nnz, const int *d_row_
 //   dM_ij/d(o1, o2)     = (x, x^2) / (a_ii + a_jj),    x = a_ij / s.
 namespace {
 
+// What dL/dc needs of the pseudo-inverse basis, in FP32 pairs (FP32 V-cycle)
+// or FP64: per entry x / (a_ii + a_jj) and x^2 / (a_ii + a_jj) with x = a_ij / s
+// (zero on the diagonal), per row (1, x, x^2) / a_ii with x = a_ii / s.  Laid
+// out with the training buffers.
+template <class V> struct AdjBasis {
+    const V *o1, *o2, *d;
+};
+template <class V>
+__global__ void __launch_bounds__(kBlock) k_adj_basis(int n, const int *__restrict__ rp, const int *__restrict__ col,
+                                                      const double *__restrict__ bx, const double *__restrict__ bw,
+                                                      V *__restrict__ o1, V *__restrict__ o2, V *__restrict__ d) {
+    const int i = blockIdx.x * kBlock + threadIdx.x;
+    if (i >= n) return;
+    for (int p = rp[i]; p < rp[i + 1]; ++p) {
+        const double x = bx[p], w = bw[p];
+        const bool diag = col[p] == i;
+        tail_set(o1[p], diag ? 0.0 : w * x);
+        tail_set(o2[p], diag ? 0.0 : w * x * x);
+        if (diag) {
+            tail_set(d[3 * static_cast<size_t>(i)], w);
+            tail_set(d[3 * static_cast<size_t>(i) + 1], w * x);
+            tail_set(d[3 * static_cast<size_t>(i) + 2], w * x * x);
+        }
+    }
+}
+
+__device__ __forceinline__ void adj_add(FloatPair &a, const FloatPair &b) { pair_add(a, b.h, b.l); }
+__device__ __forceinline__ void adj_add(double &a, double b) { a += b; }
+// u r v for the row's own values u, r and a basis value v
+__device__ __forceinline__ FloatPair adj_prod(float u, float r, const FloatPair &v) {
+    const float t = __fmul_rn(u, r), tl = __fmaf_rn(u, r, -t);
+    FloatPair o{__fmul_rn(t, v.h), 0.f};
+    o.l = __fmaf_rn(t, v.l, __fmaf_rn(tl, v.h, __fmaf_rn(t, v.h, -o.h)));
+    return o;
+}
+__device__ __forceinline__ double adj_prod(double u, double r, double v) { return u * r * v; }
+// u v
+__device__ __forceinline__ FloatPair adj_scale(float u, const FloatPair &v) {
+    FloatPair o{__fmul_rn(u, v.h), 0.f};
+    o.l = __fmaf_rn(u, v.l, __fmaf_rn(u, v.h, -o.h));
+    return o;
+}
+__device__ __forceinline__ double adj_scale(double u, double v) { return u * v; }
+__device__ __forceinline__ FloatPair adj_shfl(const FloatPair &v, int o) {
+    return {__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)};
+}
+__device__ __forceinline__ double adj_shfl(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+
 // One step of the adjoint on a row-group of A's pattern.  The sweep
 // u' = u + M r has rbar = M ubar', dL/dM_ij = ubar'_i r_j; one pass over the
 // pattern forms rbar (stored when rbar != nullptr), adds it to bbar (assigns
@@ -3393,18 +3441,22 @@ namespace {
 // replaces five launches per sweep (gradient pass, its one-block sum, M ubar,
 // bbar += rbar): on the training meshes (2k to 20k rows) each pass is a few
 // microseconds of dependent loads, whatever it computes.  Pattern, Q^-1 and
-// basis entries are loaded ahead of the grid-dependency wait.
-template <class T, int TPR>
+// basis entries are loaded ahead of the grid-dependency wait.  With the FP32
+// V-cycle the gradient's sums are FP32 pairs: in FP64 they were about 100
+// instructions a warp of 64 cycles each on a sub-partition's FP64 unit (7 of
+// the pass's 9 us on every level).
+template <class T, class V, int TPR>
 __global__ void __launch_bounds__(kBlock) k_adj_sweep(int n, const int *__restrict__ rp, const int *__restrict__ col,
-                                                      const T *__restrict__ q, const double *__restrict__ bx,
-                                                      const double *__restrict__ bw, const T *ubar, const T *r,
-                                                      T *rbar, T *bbar, int assign, double *partial) {
+                                                      const T *__restrict__ q, AdjBasis<V> basis, const T *ubar,
+                                                      const T *r, T *rbar, T *bbar, int assign, double *partial) {
     constexpr int E = 4;
     const int gid = blockIdx.x * kBlock + threadIdx.x;
     const int row = gid / TPR, lane = gid % TPR;
+    V zero;
+    tail_set(zero, 0.0);
     int base = 0, end = 0, c[E];
     T m[E];
-    double x[E], w[E];
+    V o1[E], o2[E], d[3] = {zero, zero, zero};
     auto fetch = [&](int b0) {
 #pragma unroll
         for (int j = 0; j < E; ++j) {
@@ -3412,18 +3464,25 @@ __global__ void __launch_bounds__(kBlock) k_adj_sweep(int n, const int *__restri
             const bool in = p < end;
             c[j] = in ? __ldg(col + p) : 0;
             m[j] = in ? __ldg(q + p) : T(0);
-            x[j] = in ? __ldg(bx + p) : 0.0;
-            w[j] = in ? __ldg(bw + p) : 0.0;
+            o1[j] = in ? basis.o1[p] : zero;
+            o2[j] = in ? basis.o2[p] : zero;
         }
     };
+    const bool own = row < n && lane == 0;
     if (row < n) {
         base = __ldg(rp + row) + lane;
         end = __ldg(rp + row + 1);
         fetch(base);
     }
+    if (own) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) d[k] = basis.d[3 * static_cast<size_t>(row) + k];
+    }
     pdl_wait_and_release();
+    const T ui = row < n ? load_now(ubar + row) : T(0), ri = own ? load_now(r + row) : T(0);
+    const T bi = own && !assign ? load_now(bbar + row) : T(0);
     T acc = T(0);
-    double g[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    V g[5] = {zero, zero, zero, zero, zero};
     for (; base < end; base += E * TPR) {
         T uj[E], rj[E];
 #pragma unroll
@@ -3435,41 +3494,33 @@ __global__ void __launch_bounds__(kBlock) k_adj_sweep(int n, const int *__restri
 #pragma unroll
         for (int j = 0; j < E; ++j) {
             acc += m[j] * uj[j];
-            const double v = static_cast<double>(rj[j]) * w[j], vx = v * x[j];
-            if (base + j * TPR < end) {
-                if (c[j] == row) {
-                    g[0] += v;
-                    g[1] += vx;
-                    g[2] = fma(vx, x[j], g[2]);
-                } else {
-                    g[3] += vx;
-                    g[4] = fma(vx, x[j], g[4]);
-                }
-            }
+            tail_fma(g[3], rj[j], o1[j]);
+            tail_fma(g[4], rj[j], o2[j]);
         }
         if (base + E * TPR < end) fetch(base + E * TPR);
     }
     acc = group_sum<TPR>(acc);
-    if (row < n) {
-        const double ui = static_cast<double>(ubar[row]);
+    g[3] = adj_scale(ui, g[3]);
+    g[4] = adj_scale(ui, g[4]);
+    if (own) {
+        if (rbar) rbar[row] = acc;
+        bbar[row] = assign ? acc : bi + acc;
 #pragma unroll
-        for (int k = 0; k < 5; ++k) g[k] *= ui;
-        if (lane == 0) {
-            if (rbar) rbar[row] = acc;
-            bbar[row] = assign ? acc : bbar[row] + acc;
-        }
+        for (int k = 0; k < 3; ++k) g[k] = adj_prod(ui, ri, d[k]);
     }
-    __shared__ double red[5][kBlock / 32];
+    __shared__ V red[5][kBlock / 32];
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-        const double v = warp_sum(g[k]);
-        if (threadIdx.x % 32 == 0) red[k][threadIdx.x / 32] = v;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) adj_add(g[k], adj_shfl(g[k], o));
+        if (threadIdx.x % 32 == 0) red[k][threadIdx.x / 32] = g[k];
     }
     __syncthreads();
     if (threadIdx.x < 5) {
-        double t = partial[blockIdx.x * 5 + threadIdx.x];
-        for (int k = 0; k < kBlock / 32; ++k) t += red[threadIdx.x][k];
-        partial[blockIdx.x * 5 + threadIdx.x] = t;
+        V t = red[threadIdx.x][0];
+#pragma unroll
+        for (int k = 1; k < kBlock / 32; ++k) adj_add(t, red[threadIdx.x][k]);
+        partial[blockIdx.x * 5 + threadIdx.x] += tail_get(t);
     }
 }
 
@@ -3562,6 +3613,7 @@ struct TrainBufs {
     std::vector<double *> ck;      // [cycle][level][sweep]: r of sweep k (slot 0: that cycle's b_l when nu1 > 0)
     std::vector<double *> ubar, tmp, bbar;
     std::vector<double *> part;    // per smoothed level: five partial sums of dL/dc per block
+    std::vector<double *> o1, o2, od;   // per smoothed level: the gradient's basis (AdjBasis, 8 bytes a value)
     std::vector<int> nblk;
     double *f = nullptr, *zero = nullptr;   // level 0: right-hand side, zeros
     double *xu = nullptr;          // level-0 iterate of the multi-cycle loss
@@ -3574,6 +3626,14 @@ struct TrainBufs {
     long long kernels = 0;
     double *slot(int cyc, int l, int k) const { return ck[(static_cast<size_t>(cyc) * nlev + l) * nsw + k]; }
 };
+
+template <class V>
+void adj_basis(amg_ctx *c, const TrainBufs &tb, int l) {
+    const DevLevel &L = c->lev[l];
+    k_adj_basis<V><<<grid_for(L.n), kBlock, 0, c->stream>>>(L.n, L.A.rp, L.A.col, L.bx, L.bw,
+                                                            reinterpret_cast<V *>(tb.o1[l]), reinterpret_cast<V *>(tb.o2[l]),
+                                                            reinterpret_cast<V *>(tb.od[l])); AMG_COUNT();
+}
 
 int train_bufs(amg_ctx *c, TrainBufs &tb, int ncyc) {
     const int nlev = static_cast<int>(c->lev.size());
@@ -3588,6 +3648,14 @@ int train_bufs(amg_ctx *c, TrainBufs &tb, int ncyc) {
         tb.bbar.assign(nlev, nullptr);
         tb.part.assign(nlev, nullptr);
         tb.nblk.assign(nlev, 0);
+        tb.o1.assign(nlev, nullptr);
+        tb.o2.assign(nlev, nullptr);
+        tb.od.assign(nlev, nullptr);
+        for (int l = 0; l < nlev - 1; ++l) {
+            tb.o1[l] = pl.take<double>(c->lev[l].A.nnz);
+            tb.o2[l] = pl.take<double>(c->lev[l].A.nnz);
+            tb.od[l] = pl.take<double>(3 * static_cast<size_t>(c->lev[l].n));
+        }
         for (int l = 0; l < nlev; ++l) {
             const int n = c->lev[l].n;
             for (int q = 0; q < ncyc; ++q)
@@ -3621,7 +3689,13 @@ int train_bufs(amg_ctx *c, TrainBufs &tb, int ncyc) {
     pl = Planner{};
     pl.base = tb.arena;
     lay(pl);
-    return ctx_cuda_check(c, cudaMemsetAsync(tb.arena, 0, bytes, c->stream), "memset training buffers");
+    const int rc = ctx_cuda_check(c, cudaMemsetAsync(tb.arena, 0, bytes, c->stream), "memset training buffers");
+    if (rc) return rc;
+    for (int l = 0; l < nlev - 1; ++l) {
+        if (c->opt.precision == AMG_FP64) adj_basis<double>(c, tb, l);
+        else adj_basis<FloatPair>(c, tb, l);
+    }
+    return ctx_cuda_check(c, cudaGetLastError(), "training basis");
 }
 
 // Right-hand side of level l in cycle cyc: written straight into the
@@ -3665,11 +3739,14 @@ T *fwd_level_ckpt(amg_ctx *c, TrainBufs &tb, int cyc, int l, cudaStream_t s) {
 
 template <class T> struct AdjLaunch {
     template <int TPR>
-    static void sweep(const DevLevel &L, const T *ubar, const T *r, T *rbar, T *bbar, int assign, double *part,
-                      cudaStream_t s) {
-        launch_pdl(k_adj_sweep<T, TPR>, dim3(grid_for(static_cast<long long>(L.n) * TPR)), dim3(kBlock), 0, s, L.n,
-                   L.A.rp, static_cast<const int *>(L.A.col), qvals<T>(L), static_cast<const double *>(L.bx),
-                   static_cast<const double *>(L.bw), ubar, r, rbar, bbar, assign, part);
+    static void sweep(const DevLevel &L, const TrainBufs &tb, int l, const T *ubar, const T *r, T *rbar, T *bbar,
+                      int assign, cudaStream_t s) {
+        using V = typename std::conditional<std::is_same<T, float>::value, FloatPair, double>::type;
+        const AdjBasis<V> basis{reinterpret_cast<const V *>(tb.o1[l]), reinterpret_cast<const V *>(tb.o2[l]),
+                                reinterpret_cast<const V *>(tb.od[l])};
+        launch_pdl(k_adj_sweep<T, V, TPR>, dim3(grid_for(static_cast<long long>(L.n) * TPR)), dim3(kBlock), 0, s, L.n,
+                   L.A.rp, static_cast<const int *>(L.A.col), qvals<T>(L), basis, ubar, r, rbar, bbar, assign,
+                   tb.part[l]);
     }
     template <int TPR>
     static void restrict_(const DevMat &P, const T *x, T *rhobar, T *bbar, int assign, cudaStream_t s) {
@@ -3699,8 +3776,8 @@ void bwd_level(amg_ctx *c, TrainBufs &tb, int cyc, int l, const T *in, T *other,
         std::swap(out, spare);
     };
     auto sweep = [&](int k) {                         // ubar <- ubar - A (M ubar), bbar += M ubar
-        TPR_DISPATCH(L.A.tpr, AdjLaunch<T>::template sweep, L, ub, reinterpret_cast<const T *>(tb.slot(cyc, l, k)), rbar,
-                     bb, assign, tb.part[l], s);
+        TPR_DISPATCH(L.A.tpr, AdjLaunch<T>::template sweep, L, tb, l, ub,
+                     reinterpret_cast<const T *>(tb.slot(cyc, l, k)), rbar, bb, assign, s);
         assign = 0;
         L_resid<T>(L.A, ub, rbar, out, s);
         advance();
@@ -3718,8 +3795,8 @@ void bwd_level(amg_ctx *c, TrainBufs &tb, int cyc, int l, const T *in, T *other,
     advance();
     for (int k = nu1 - 1; k >= 1; --k) sweep(k);
     if (nu1 >= 1) {        // first sweep from zero: u = M b
-        TPR_DISPATCH(L.A.tpr, AdjLaunch<T>::template sweep, L, ub, static_cast<const T *>(level_b<T>(c, tb, cyc, l)),
-                     static_cast<T *>(nullptr), bb, 0, tb.part[l], s);
+        TPR_DISPATCH(L.A.tpr, AdjLaunch<T>::template sweep, L, tb, l, ub,
+                     static_cast<const T *>(level_b<T>(c, tb, cyc, l)), static_cast<T *>(nullptr), bb, 0, s);
     }
 }
 
@@ -3778,7 +3855,8 @@ void loss_enqueue(amg_ctx *c, TrainBufs &tb, int nvc, cudaStream_t s) {
 // second call with the same number of cycles on, its 300 to 400 kernels are
 // one graph launch.  12k-row mesh, three cycles: 2341 us a call with five
 // launches per adjoint sweep and a host step for the loss, 1235 us with the
-// fused passes launched singly (a first call), 1011 us as a graph.
+// fused passes launched singly (a first call), 1011 us as a graph, 749 us
+// with the gradient's sums in FP32 pairs (k_adj_sweep).
 template <class T>
 int loss_grad(amg_ctx *c, TrainBufs &tb, const double *f, int nvc, double *loss, double *dc) {
     cudaStream_t s = c->stream;
