@@ -1471,7 +1471,13 @@ static T *smooth(amg_ctx *c, int l, cudaStream_t s, const T *b, T *cur, T *alt, 
     const bool gnn = (c->smoother == AMG_SMOOTHER_GNN);
     if (nsweeps == 0 && zero_init) cudaMemsetAsync(cur, 0, sizeof(T) * L.n, s);
     if (c->smoother == AMG_SMOOTHER_CHEB) return cheb_smooth<T>(c, L, s, b, cur, alt, nsweeps, zero_init);
-    for (int k = 0; k < nsweeps; ++k) {
+    int k = 0;
+    // two Jacobi sweeps from zero in one pass (1025^2 grid: V-cycle 176.0 -> 169.5 us)
+    if (!gnn && zero_init && nsweeps >= 2) {
+        TPR_DISPATCH(L.A.tpr, Launch<T>::template jacobi_first2, L.A, jvals<T>(L), b, cur, s);
+        k = 2;
+    }
+    for (; k < nsweeps; ++k) {
         const bool first = (k == 0 && zero_init);
         if (gnn) {
             if (first) {
@@ -3061,7 +3067,12 @@ double smooth_bytes(const amg_ctx *c, const DevLevel &L, int tb, int nsweeps, bo
     if (c->smoother == AMG_SMOOTHER_CHEB) return cheb_bytes(c, L, tb, nsweeps, zero_init);
     const bool gnn = (c->smoother == AMG_SMOOTHER_GNN);
     double b = 0.0;
-    for (int k = 0; k < nsweeps; ++k) {
+    int k = 0;
+    if (!gnn && zero_init && nsweeps >= 2) {
+        b += pass_bytes(L.A, tb, 2.0 * L.n, 1);                                // two Jacobi sweeps
+        k = 2;
+    }
+    for (; k < nsweeps; ++k) {
         const bool first = (k == 0 && zero_init);
         if (gnn) {
             if (first) b += pass_bytes(L.A, tb, L.n, 1);                       // u = Q b
