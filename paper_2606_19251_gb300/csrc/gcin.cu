@@ -217,8 +217,8 @@ int gcin_batch_build(GcinBatch &b, int n_problems, amg_ctx *const *problems, cud
 // ---------------------------------------------------------------------------
 // mean and M2 (sum of squared deviations) per feature of the tile's y rows;
 // the block's threads form kBlock / H groups of H (one thread per feature)
-template <int H>
-__device__ __forceinline__ void tile_stats(const float (*sY)[H + 1], int nn, float *tmean, float *tm2) {
+template <int H, int YS = H + 1>
+__device__ __forceinline__ void tile_stats(const float (*sY)[YS], int nn, float *tmean, float *tm2) {
     constexpr int Q = kBlock / H;
     __shared__ float red[Q][H];
     __shared__ float smean[H];
