@@ -493,46 +493,65 @@ __device__ __forceinline__ double lanes_sum(double v, double (*red)[H]) {
     return t;
 }
 
+// The same for FP32 pairs; the total in the threads with tid < H.
+template <int H>
+__device__ __forceinline__ FloatPair lanes_sum_pair(FloatPair v, FloatPair (*red)[H]) {
+    const int f = threadIdx.x % H, q = threadIdx.x / H;
+    red[q][f] = v;
+    __syncthreads();
+    for (int w = kLanes / 2; w > 0; w >>= 1) {
+        if (q < w) {
+            const FloatPair o = red[q + w][f];
+            pair_add(v, o.h, o.l);
+            red[q][f] = v;
+        }
+        __syncthreads();
+    }
+    return v;
+}
+__device__ __forceinline__ double pair_value(const FloatPair &v) { return static_cast<double>(v.h) + static_cast<double>(v.l); }
+
 // Group statistics from part statistics (biased variance):
 // mean = sum_t n_t mean_t / n, M2 = sum_t [M2_t + n_t (mean_t - mean)^2].
 // Parts t of group g are gtile[g] .. gtile[g+1] with node ranges
 // tstart[t] .. tstart[t+1].  Run twice: tiles -> chunks (final = 0: writes
 // the chunk mean and M2 into mu / rstd) and chunks -> graphs (final = 1:
 // writes the instance-norm mean and 1/sqrt(var + eps)).  16 lanes of parts
-// per feature; one FP64 add per part, the rest in FP32.
-// The part loops are unrolled so that a thread's loads are in flight together
-// (a dependent trip per part made the two stages 13 and 10 us on a 50k-node
-// mesh), and only the H threads that hold the totals divide in FP64.  With
-// the normalisation pass's and the head's reductions: 50k-node prediction 363
-// -> 314 us, 1.95M nodes 2698 -> 2487 us.
+// per feature, summed as FP32 pairs; FP64 only for the totals' divisions.
+// In FP64 each part cost two instructions of 64 cycles on a sub-partition's
+// FP64 unit (7 of a stage's 12 us on a 50k-node mesh); the part loops are
+// unrolled so that a thread's loads are in flight together.  With the
+// normalisation pass's and the head's reductions: prediction on 50k rows 363
+// -> 314 us and, with pairs here and in the pooling, 301 -> 263 us; on 1.2M rows
+// 2698 -> 2487 and 2235 -> 2114 us.
 template <int H>
 __global__ void __launch_bounds__(kLanes * H) k_stats_combine(const int *__restrict__ gtile, const int *__restrict__ gptr,
                                                             const int *__restrict__ tstart,
                                                             const float *__restrict__ tmean,
                                                             const float *__restrict__ tm2, float *__restrict__ mu,
                                                             float *__restrict__ rstd, int final) {
-    __shared__ double red[kLanes][H];
+    __shared__ FloatPair red[kLanes][H];
     __shared__ float smean[H];
     const int g = blockIdx.x, f = threadIdx.x % H, q = threadIdx.x / H;
     const int t0 = gtile[g] + q, t1 = gtile[g + 1];
-    double s = 0.0;
+    FloatPair s{0.f, 0.f};
 #pragma unroll 8
     for (int t = t0; t < t1; t += kLanes)
-        s += static_cast<double>(static_cast<float>(tstart[t + 1] - tstart[t]) * tmean[static_cast<size_t>(t) * H + f]);
-    const double total = lanes_sum<H>(s, red);
-    const double n = gptr[g + 1] - gptr[g];
-    if (q == 0) smean[f] = static_cast<float>(total / n);
+        pair_add(s, static_cast<float>(tstart[t + 1] - tstart[t]) * tmean[static_cast<size_t>(t) * H + f]);
+    s = lanes_sum_pair<H>(s, red);
+    const int n = gptr[g + 1] - gptr[g];
+    if (q == 0) smean[f] = static_cast<float>(pair_value(s) / n);
     __syncthreads();
     const float mf = smean[f];
-    double v = 0.0;
+    FloatPair v{0.f, 0.f};
 #pragma unroll 8
     for (int t = t0; t < t1; t += kLanes) {
         const float d = tmean[static_cast<size_t>(t) * H + f] - mf;
-        v += static_cast<double>(fmaf(static_cast<float>(tstart[t + 1] - tstart[t]) * d, d,
-                                      tm2[static_cast<size_t>(t) * H + f]));
+        pair_add(v, fmaf(static_cast<float>(tstart[t + 1] - tstart[t]) * d, d, tm2[static_cast<size_t>(t) * H + f]));
     }
-    const double m2 = lanes_sum<H>(v, red);
+    v = lanes_sum_pair<H>(v, red);
     if (q == 0) {
+        const double m2 = pair_value(v);
         mu[static_cast<size_t>(g) * H + f] = mf;
         rstd[static_cast<size_t>(g) * H + f] =
             final ? static_cast<float>(1.0 / sqrt(m2 / n + static_cast<double>(kEps))) : static_cast<float>(m2);
@@ -550,8 +569,8 @@ __global__ void __launch_bounds__(kLanes * H) k_stats_combine(const int *__restr
 // The 16 row groups' partial sums and maxima go through shared memory as
 // 16-byte vectors (four features of a thread; as 8-byte FP64 values at a
 // stride of four they kept the L1 pipe at 85 to 94 %), and a feature's 16
-// sums are added as an FP32 pair and converted once (the 32 FP64 operations
-// per feature and tile were 100 us of a 1.95M-node pass).
+// sums are added as an FP32 pair (the 32 FP64 operations per feature and tile
+// were 100 us of a 1.95M-node pass).
 template <int H, int YM = 0>
 __global__ void __launch_bounds__(kBlock, 6) k_norm_relu_pool_tile(const int *__restrict__ tstart,
                                                                 const int *__restrict__ tgraph,
@@ -561,7 +580,7 @@ __global__ void __launch_bounds__(kBlock, 6) k_norm_relu_pool_tile(const int *__
                                                                 const float *__restrict__ gamma,
                                                                 const float *__restrict__ beta, float *__restrict__ x,
                                                                 __nv_bfloat16 *__restrict__ xb,
-                                                                double *__restrict__ tsum, float *__restrict__ tmax,
+                                                                FloatPair *__restrict__ tsum, float *__restrict__ tmax,
                                                                 int *__restrict__ targ,
                                                                 const float *__restrict__ h1 = nullptr,
                                                                 const float *__restrict__ W1 = nullptr,
@@ -576,7 +595,7 @@ __global__ void __launch_bounds__(kBlock, 6) k_norm_relu_pool_tile(const int *__
     const float4 ga = *reinterpret_cast<const float4 *>(gamma + f);
     const float4 be = *reinterpret_cast<const float4 *>(beta + f);
     // FP32 partial sums of at most kTile / Q values per thread (GB300's FP64
-    // pipe is narrow); the tile sum is an FP32 pair, the graph sum FP64
+    // pipe is narrow); tile and graph sums are FP32 pairs
     float s[4] = {0.f, 0.f, 0.f, 0.f};
     float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
     int mi[4] = {a, a, a, a};
@@ -644,7 +663,7 @@ __global__ void __launch_bounds__(kBlock, 6) k_norm_relu_pool_tile(const int *__
             pair_add(ts, ps[k * H]);
             bm = fmaxf(bm, pm[k * H]);
         }
-        tsum[static_cast<size_t>(t) * H + ff] = static_cast<double>(ts.h) + static_cast<double>(ts.l);
+        tsum[static_cast<size_t>(t) * H + ff] = ts;
         tmax[static_cast<size_t>(t) * H + ff] = bm;
         if (targ) {                              // the first node of the maximum
             int bi = a;
@@ -666,17 +685,17 @@ __global__ void __launch_bounds__(kBlock, 6) k_norm_relu_pool_tile(const int *__
 // max and argmax) and chunks -> graphs (writes the pooled mean and max).
 template <int H>
 __global__ void __launch_bounds__(kLanes * H) k_pool_combine(const int *__restrict__ gtile, const int *__restrict__ gptr,
-                                                           const double *__restrict__ tsum,
+                                                           const FloatPair *__restrict__ tsum,
                                                            const float *__restrict__ tmax,
                                                            const int *__restrict__ targ, float *__restrict__ pooled,
                                                            int *__restrict__ argmax, int layer,
-                                                           double *__restrict__ csum, float *__restrict__ cmax,
+                                                           FloatPair *__restrict__ csum, float *__restrict__ cmax,
                                                            int *__restrict__ carg) {
-    __shared__ double red[kLanes][H];
+    __shared__ FloatPair red[kLanes][H];
     __shared__ float rm[kLanes][H];
     __shared__ int ri[kLanes][H];
     const int g = blockIdx.x, f = threadIdx.x % H, q = threadIdx.x / H;
-    double s = 0.0;
+    FloatPair s{0.f, 0.f};
     float bm = -INFINITY;
     int bi = gptr[g];
     const int t0 = gtile[g] + q, t1 = gtile[g + 1];
@@ -686,20 +705,22 @@ __global__ void __launch_bounds__(kLanes * H) k_pool_combine(const int *__restri
             const size_t o = static_cast<size_t>(t) * H + f;
             const float m = tmax[o];
             const int a = targ[o];
-            s += tsum[o];
+            const FloatPair p = tsum[o];
+            pair_add(s, p.h, p.l);
             if (m > bm) { bm = m; bi = a; }   // tiles ascend, so the first max wins
         }
     } else {                                  // inference: no backward asks for the node
 #pragma unroll 8
         for (int t = t0; t < t1; t += kLanes) {
             const size_t o = static_cast<size_t>(t) * H + f;
-            s += tsum[o];
+            const FloatPair p = tsum[o];
+            pair_add(s, p.h, p.l);
             bm = fmaxf(bm, tmax[o]);
         }
     }
     rm[q][f] = bm;
     ri[q][f] = bi;
-    const double total = lanes_sum<H>(s, red);
+    const FloatPair total = lanes_sum_pair<H>(s, red);
     if (q == 0) {
         for (int k = 1; k < kLanes; ++k)
             if (rm[k][f] > bm || (rm[k][f] == bm && ri[k][f] < bi)) { bm = rm[k][f]; bi = ri[k][f]; }
@@ -711,7 +732,7 @@ __global__ void __launch_bounds__(kLanes * H) k_pool_combine(const int *__restri
             return;
         }
         float *P = pooled + (static_cast<size_t>(g) * kLayers + layer) * 2 * H;
-        P[f] = static_cast<float>(total / (gptr[g + 1] - gptr[g]));
+        P[f] = static_cast<float>(pair_value(total) / (gptr[g + 1] - gptr[g]));
         P[H + f] = bm;
         if (targ) argmax[(static_cast<size_t>(g) * kLayers + layer) * H + f] = bi;
     }
@@ -861,26 +882,27 @@ static void forward_impl(GcinBatch &b, const float *th, cudaStream_t s) {
         // inference keeps only what the next aggregation reads (bfloat16 with
         // the tensor-core linears, nothing after the last layer)
         const bool last = l == kLayers - 1;
+        FloatPair *tsum = reinterpret_cast<FloatPair *>(b.tsum), *csum = reinterpret_cast<FloatPair *>(b.csum);
         int *targ = b.infer ? nullptr : b.targ, *carg = b.infer ? nullptr : b.carg;
         float *xo = (b.infer && (xbf || last)) ? nullptr : b.x[l];
         __nv_bfloat16 *xbo = (xbf && !last) ? reinterpret_cast<__nv_bfloat16 *>(b.x[l]) : nullptr;
         if (xbf && l == 0) {
             k_norm_relu_pool_tile<H, 2><<<NT, kBlock, 0, s>>>(b.tstart, b.tgraph, b.y[l], b.mu[l], b.rstd[l],
-                                                              th + pl.inG[l], th + pl.inB[l], xo, xbo, b.tsum,
+                                                              th + pl.inG[l], th + pl.inB[l], xo, xbo, tsum,
                                                               b.tmax, targ, b.h1, th + pl.convW[0],
                                                               th + pl.convB[0]); AMG_COUNT();
         } else if (xbf) {
             k_norm_relu_pool_tile<H, 1><<<NT, kBlock, 0, s>>>(b.tstart, b.tgraph, b.y[l], b.mu[l], b.rstd[l],
-                                                              th + pl.inG[l], th + pl.inB[l], xo, xbo, b.tsum,
+                                                              th + pl.inG[l], th + pl.inB[l], xo, xbo, tsum,
                                                               b.tmax, targ); AMG_COUNT();
         } else {
             k_norm_relu_pool_tile<H><<<NT, kBlock, 0, s>>>(b.tstart, b.tgraph, b.y[l], b.mu[l], b.rstd[l],
-                                                           th + pl.inG[l], th + pl.inB[l], xo, xbo, b.tsum, b.tmax,
+                                                           th + pl.inG[l], th + pl.inB[l], xo, xbo, tsum, b.tmax,
                                                            targ); AMG_COUNT();
         }
-        k_pool_combine<H><<<b.NC, CT, 0, s>>>(b.ctile, b.cnode, b.tsum, b.tmax, targ, nullptr, nullptr, l,
-                                              b.csum, b.cmax, carg); AMG_COUNT();
-        k_pool_combine<H><<<G, CT, 0, s>>>(b.gchunk, b.gptr, b.csum, b.cmax, carg, b.pooled, b.argmax, l,
+        k_pool_combine<H><<<b.NC, CT, 0, s>>>(b.ctile, b.cnode, tsum, b.tmax, targ, nullptr, nullptr, l,
+                                              csum, b.cmax, carg); AMG_COUNT();
+        k_pool_combine<H><<<G, CT, 0, s>>>(b.gchunk, b.gptr, csum, b.cmax, carg, b.pooled, b.argmax, l,
                                            nullptr, nullptr, nullptr); AMG_COUNT();
     }
     k_head<H><<<G, kHeadThreads, 0, s>>>(b.pooled, th, b.head, b.c); AMG_COUNT();
@@ -932,12 +954,14 @@ __global__ void __launch_bounds__(128) k_head_bwd(const float *__restrict__ scra
     }
     __syncthreads();
     float da1 = 0.f;
+#pragma unroll 32   // the lane's loads of its weight row in flight together
     for (int k = 0; k < 64; ++k) da1 = fmaf(sdz2[k], th[PL<H>().h2W + t * 64 + k], da1);
     const float dz1 = S[kSa1 + t] > 0.f ? da1 : 0.f;
     sdz1[t] = dz1;
     D[kGdz1 + t] = dz1;
     __syncthreads();
     float ds = 0.f;
+#pragma unroll 32
     for (int k = 0; k < 128; ++k) ds = fmaf(sdz1[k], th[PL<H>().h1W + t * 128 + k], ds);
     const float sg = S[kSsg + t];
     const float dzh = ds * sg * (1.f - sg);
@@ -957,6 +981,7 @@ __global__ void __launch_bounds__(128) k_head_bwd(const float *__restrict__ scra
         const int l = j / (2 * H), m = j % (2 * H);
         const float *W = th + PL<H>().roW[l] + m * kRo;
         float acc = 0.f;
+#pragma unroll
         for (int k = 0; k < kRo; ++k) acc = fmaf(sdz[l * kRo + k], W[k], acc);
         dpooled[static_cast<size_t>(g) * kLayers * 2 * H + j] = acc;
     }
@@ -1063,7 +1088,9 @@ __global__ void __launch_bounds__(kLanes * H) k_bwd_combine(const int *__restric
     __shared__ double red[kLanes][H];
     const int g = blockIdx.x, f = threadIdx.x % H, q = threadIdx.x / H;
     double s1 = 0.0, s2 = 0.0;
-    for (int t = gtile[g] + q; t < gtile[g + 1]; t += kLanes) {
+    const int t1e = gtile[g + 1];
+#pragma unroll 4
+    for (int t = gtile[g] + q; t < t1e; t += kLanes) {
         s1 += tsum[static_cast<size_t>(t) * H + f];
         s2 += tsum2[static_cast<size_t>(t) * H + f];
     }

@@ -89,7 +89,7 @@ struct GcinBatch {
     int NC = 0;
     int *ctile = nullptr, *cnode = nullptr, *gchunk = nullptr;      // chunk -> first tile / node; graph -> first chunk
     float *cmean = nullptr, *cm2 = nullptr, *cmax = nullptr;        // NC x H chunk statistics
-    double *csum = nullptr;                                         // NC x H
+    double *csum = nullptr;                                         // NC x H (holds FP32 pairs)
     int *carg = nullptr;                                            // NC x H
     float *w = nullptr;
     double *w64 = nullptr;
@@ -101,7 +101,7 @@ struct GcinBatch {
     float *x[kLayers] = {};              // N x H      ReLU(IN(y))
     float *mu[kLayers] = {}, *rstd[kLayers] = {};   // G x H
     float *tmean = nullptr, *tm2 = nullptr;          // NT x H tile statistics of y
-    double *tsum = nullptr;                          // NT x H tile sums (pooling / backward)
+    double *tsum = nullptr;                          // NT x H tile sums (pooling: FP32 pairs; backward: FP64)
     double *tsum2 = nullptr;                         // NT x H second tile sums (backward)
     float *tmax = nullptr;                           // NT x H
     int *targ = nullptr;                             // NT x H
