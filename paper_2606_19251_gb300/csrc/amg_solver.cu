@@ -34,6 +34,7 @@
 #include "ctx.cuh"
 #include "wavefront.cuh"
 #include "tail.cuh"
+#include "train_tail.cuh"
 #include "setup_device.h"
 
 using namespace amg;
@@ -3421,28 +3422,6 @@ __global__ void __launch_bounds__(kBlock) k_adj_basis(int n, const int *__restri
     }
 }
 
-__device__ __forceinline__ void adj_add(FloatPair &a, const FloatPair &b) { pair_add(a, b.h, b.l); }
-__device__ __forceinline__ void adj_add(double &a, double b) { a += b; }
-// u r v for the row's own values u, r and a basis value v
-__device__ __forceinline__ FloatPair adj_prod(float u, float r, const FloatPair &v) {
-    const float t = __fmul_rn(u, r), tl = __fmaf_rn(u, r, -t);
-    FloatPair o{__fmul_rn(t, v.h), 0.f};
-    o.l = __fmaf_rn(t, v.l, __fmaf_rn(tl, v.h, __fmaf_rn(t, v.h, -o.h)));
-    return o;
-}
-__device__ __forceinline__ double adj_prod(double u, double r, double v) { return u * r * v; }
-// u v
-__device__ __forceinline__ FloatPair adj_scale(float u, const FloatPair &v) {
-    FloatPair o{__fmul_rn(u, v.h), 0.f};
-    o.l = __fmaf_rn(u, v.l, __fmaf_rn(u, v.h, -o.h));
-    return o;
-}
-__device__ __forceinline__ double adj_scale(double u, double v) { return u * v; }
-__device__ __forceinline__ FloatPair adj_shfl(const FloatPair &v, int o) {
-    return {__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)};
-}
-__device__ __forceinline__ double adj_shfl(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
-
 // One step of the adjoint on a row-group of A's pattern.  The sweep
 // u' = u + M r has rbar = M ubar', dL/dM_ij = ubar'_i r_j; one pass over the
 // pattern forms rbar (stored when rbar != nullptr), adds it to bbar (assigns
@@ -3635,8 +3614,30 @@ struct TrainBufs {
     cudaGraphExec_t exec = nullptr;   // the call's kernels for graph_nvc cycles (from its second call on)
     int graph_nvc = 0, calls = 0;
     long long kernels = 0;
+    int tail = -1;                 // first level of the one-CTA coarse part (train_tail.cuh)
     double *slot(int cyc, int l, int k) const { return ck[(static_cast<size_t>(cyc) * nlev + l) * nsw + k]; }
 };
+
+// Dynamic shared memory of the one-CTA coarse part for `vecs` vectors of
+// `rows` entries of `elem` bytes.
+size_t train_tail_smem(size_t vecs, size_t rows, size_t elem) {
+    return sizeof(double) * 2 * kTtCoarse * kTtLd + vecs * rows * elem;
+}
+
+// First level of the one-CTA coarse part: at most kTrainTailRows rows and at
+// least one smoothed level, its vectors within a CTA's shared memory; -1 if
+// there is none.  Level 0 stays outside (its right-hand side is f itself).
+int train_tail_level(const amg_ctx *c) {
+    const int nlev = static_cast<int>(c->lev.size());
+    size_t rows = c->nL;
+    int best = -1;
+    for (int l = nlev - 2; l >= 1 && nlev - l <= kTailMaxLevels && c->nL <= kTtCoarse; --l) {
+        rows += c->lev[l].n;
+        if (c->lev[l].n > kTrainTailRows || train_tail_smem(4, rows, sizeof(double)) > kTailSmem) break;
+        best = l;
+    }
+    return best;
+}
 
 template <class V>
 void adj_basis(amg_ctx *c, const TrainBufs &tb, int l) {
@@ -3652,6 +3653,7 @@ int train_bufs(amg_ctx *c, TrainBufs &tb, int ncyc) {
     tb.ncyc = ncyc;
     tb.nsw = nsw;
     tb.nlev = nlev;
+    tb.tail = train_tail_level(c);
     auto lay = [&](Planner &pl) {
         tb.ck.assign(static_cast<size_t>(ncyc) * nlev * nsw, nullptr);
         tb.ubar.assign(nlev, nullptr);
@@ -3718,11 +3720,63 @@ T *level_b(amg_ctx *c, const TrainBufs &tb, int cyc, int l) {
     return reinterpret_cast<T *>(c->lev[l].vb);
 }
 
+template <class T, bool ADJ>
+void launch_train_tail(amg_ctx *c, TrainBufs &tb, int cyc, const T *in, T *out, cudaStream_t s) {
+    using V = typename std::conditional<std::is_same<T, float>::value, FloatPair, double>::type;
+    TrainTailArgs<T, V> a{};
+    a.nlev = tb.nlev - tb.tail;
+    a.nu1 = c->opt.nu1;
+    a.nu2 = c->opt.nu2;
+    a.Linv = c->Linv;
+    a.LinvT = c->LinvT;
+    a.in = in;
+    a.out = out;
+    for (int k = 0; k < a.nlev; ++k) {
+        const int l = tb.tail + k;
+        const DevLevel &L = c->lev[l];
+        TrainTailLevel<T, V> &D = a.lev[k];
+        D.n = L.n;
+        D.off = a.rows;
+        a.rows += L.n;
+        if (k == a.nlev - 1) break;
+        auto lg = [](int tpr) {
+            int k = 0;
+            while ((1 << k) < tpr) ++k;
+            return k;
+        };
+        D.la = lg(L.A.tpr);
+        D.lp = lg(L.P.tpr);
+        D.lr = lg(L.R.tpr);
+        D.A = {L.A.rp, L.A.col, mvals<T>(L.A)};
+        D.P = {L.P.rp, L.P.col, mvals<T>(L.P)};
+        D.R = {L.R.rp, L.R.col, mvals<T>(L.R)};
+        D.q = qvals<T>(L);
+        D.o1 = reinterpret_cast<const V *>(tb.o1[l]);
+        D.o2 = reinterpret_cast<const V *>(tb.o2[l]);
+        D.d = reinterpret_cast<const V *>(tb.od[l]);
+        D.ck = reinterpret_cast<T *>(tb.slot(cyc, l, 0));
+        D.stride = tb.nsw > 1 ? reinterpret_cast<T *>(tb.slot(cyc, l, 1)) - D.ck : 0;
+        D.partial = tb.part[l];
+    }
+    const size_t smem = train_tail_smem(ADJ ? 4 : 3, a.rows, sizeof(T));
+    if (ADJ) {
+        cudaFuncSetAttribute(k_train_tail_adj<T, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kTailSmem));
+        launch_pdl(k_train_tail_adj<T, V>, dim3(1), dim3(kTtThreads), smem, s, a);
+    } else {
+        cudaFuncSetAttribute(k_train_tail_fwd<T, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kTailSmem));
+        launch_pdl(k_train_tail_fwd<T, V>, dim3(1), dim3(kTtThreads), smem, s, a);
+    }
+}
+
 template <class T>
 T *fwd_level_ckpt(amg_ctx *c, TrainBufs &tb, int cyc, int l, cudaStream_t s) {
     DevLevel &L = c->lev[l];
     T *b = level_b<T>(c, tb, cyc, l), *u = reinterpret_cast<T *>(L.vu), *r = reinterpret_cast<T *>(L.vr);
     const int nu1 = c->opt.nu1, nsw = nu1 + c->opt.nu2;
+    if (l == tb.tail) {
+        launch_train_tail<T, false>(c, tb, cyc, b, u, s);
+        return u;
+    }
     if (l == tb.nlev - 1) {
         launch_coarse<T>(c, b, u, s);
         return u;
@@ -3774,6 +3828,10 @@ void bwd_level(amg_ctx *c, TrainBufs &tb, int cyc, int l, const T *in, T *other,
     DevLevel &L = c->lev[l];
     const int nu1 = c->opt.nu1, nsw = nu1 + c->opt.nu2;
     T *bb = reinterpret_cast<T *>(tb.bbar[l]);
+    if (l == tb.tail) {
+        launch_train_tail<T, true>(c, tb, cyc, in, bb, s);
+        return;
+    }
     if (l == tb.nlev - 1) {   // u = A_L^-1 b is self-adjoint
         launch_coarse<T>(c, in, bb, s);
         return;
@@ -3867,7 +3925,8 @@ void loss_enqueue(amg_ctx *c, TrainBufs &tb, int nvc, cudaStream_t s) {
 // one graph launch.  12k-row mesh, three cycles: 2341 us a call with five
 // launches per adjoint sweep and a host step for the loss, 1235 us with the
 // fused passes launched singly (a first call), 1011 us as a graph, 749 us
-// with the gradient's sums in FP32 pairs (k_adj_sweep).
+// with the gradient's sums in FP32 pairs (k_adj_sweep), 711 us with the levels
+// of up to 256 rows in one CTA (train_tail.cuh).
 template <class T>
 int loss_grad(amg_ctx *c, TrainBufs &tb, const double *f, int nvc, double *loss, double *dc) {
     cudaStream_t s = c->stream;
