@@ -19,9 +19,10 @@
 
 namespace amg {
 
-// Largest level a tail starts on: at 1024 rows B is 4 MB (FP32), 27 KB an SM,
-// and forming it stays below a tenth of the prediction that precedes it; the
-// next RS level (about 2300 rows) would need nine times the work.
+// Largest level a tail starts on: at 1024 rows B is 4 MB (FP32), 27 KB an SM.
+// Forming it costs n_t times the tail's entries: the next RS level (about 2300
+// rows) would take five times the memory and the work, in every call that has
+// new coefficients.
 constexpr int kTailRows = 1024;
 constexpr int kTailMaxLevels = 16;     // levels of a tail (kernel argument arrays)
 constexpr int kTailCols = 4;           // columns of B a CTA forms at a time
