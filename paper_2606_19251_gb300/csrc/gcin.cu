@@ -804,27 +804,35 @@ constexpr int kSz = 0, kSzh = kEmb, kSsg = 2 * kEmb, kSa1 = 3 * kEmb, kSa2 = 3 *
 // Head gradient layout per graph: dz1[128] | dz2[64] | dzh[128] | dz[128]
 constexpr int kGdz1 = 0, kGdz2 = 128, kGdzh = 192, kGdz = 192 + kEmb;
 
-// Part q of 4 of a dot product of n terms over a column of W (row stride ld),
-// summed over the four lanes 4 k .. 4 k + 3; four lanes per output and an
-// unrolled quarter keep the three dependent layers at a few load round trips
-// each (128 serial terms per lane took 33 us on seven graphs).
-__device__ __forceinline__ float head_dot(const float *v, const float *__restrict__ W, int n, int ld, int q) {
+// Bias plus a dot product of n terms over a column of W (row stride ld).
+// Inference takes four lanes per output, each with an unrolled quarter: the
+// three dependent layers are then a few load round trips each (128 serial
+// terms per lane took 33 us on seven graphs).  Training, whose loss passes the
+// coefficients' last bits on through the V-cycles, adds the terms in one chain.
+template <int LANES>
+__device__ __forceinline__ float head_dot(float bias, const float *v, const float *__restrict__ W, int n, int ld, int q) {
+    if (LANES == 1) {
+#pragma unroll 32
+        for (int m = 0; m < n; ++m) bias = fmaf(v[m], W[m * ld], bias);
+        return bias;
+    }
     float a = 0.f;
 #pragma unroll 32
-    for (int m = q; m < n; m += 4) a = fmaf(v[m], W[m * ld], a);
-    a += __shfl_xor_sync(0xffffffffu, a, 1);
-    return a + __shfl_xor_sync(0xffffffffu, a, 2);
+    for (int m = q; m < n; m += LANES) a = fmaf(v[m], W[m * ld], a);
+#pragma unroll
+    for (int o = 1; o < LANES; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    return bias + a;
 }
 
 // Readout + head for one graph (four threads per element of the 128-vectors).
-constexpr int kHeadThreads = 4 * kEmb;
-template <int H>
-__global__ void __launch_bounds__(kHeadThreads) k_head(const float *__restrict__ pooled, const float *__restrict__ th,
+template <int H, int LANES>
+__global__ void __launch_bounds__(LANES * kEmb) k_head(const float *__restrict__ pooled, const float *__restrict__ th,
                                                        float *__restrict__ scratch, float *__restrict__ c) {
     __shared__ float sp[kLayers * 2 * H];
     __shared__ float sz[kEmb], ss[kEmb], sa1[128], sa2[64];
     __shared__ float red[4];
-    const int g = blockIdx.x, t = threadIdx.x / 4, q = threadIdx.x % 4;
+    constexpr int kHeadThreads = LANES * kEmb;
+    const int g = blockIdx.x, t = threadIdx.x / LANES, q = threadIdx.x % LANES;
     for (int k = threadIdx.x; k < kLayers * 2 * H; k += kHeadThreads)
         sp[k] = pooled[static_cast<size_t>(g) * kLayers * 2 * H + k];
     __syncthreads();
@@ -832,7 +840,7 @@ __global__ void __launch_bounds__(kHeadThreads) k_head(const float *__restrict__
     // readout linears: z[32 l + k] = [mean_l, max_l] . W_l[:, k] + b_l[k]
     {
         const int l = t / kRo, k = t % kRo;
-        const float z = th[PL<H>().roB[l] + k] + head_dot(sp + l * 2 * H, th + PL<H>().roW[l] + k, 2 * H, kRo, q);
+        const float z = head_dot<LANES>(th[PL<H>().roB[l] + k], sp + l * 2 * H, th + PL<H>().roW[l] + k, 2 * H, kRo, q);
         if (q == 0) sz[t] = z;
     }
     __syncthreads();
@@ -856,23 +864,23 @@ __global__ void __launch_bounds__(kHeadThreads) k_head(const float *__restrict__
         ss[i] = sg;
     }
     __syncthreads();
-    const float a1 = fmaxf(th[PL<H>().h1B + t] + head_dot(ss, th + PL<H>().h1W + t, kEmb, 128, q), 0.f);
+    const float a1 = fmaxf(head_dot<LANES>(th[PL<H>().h1B + t], ss, th + PL<H>().h1W + t, kEmb, 128, q), 0.f);
     if (q == 0) {
         sa1[t] = a1;
         S[kSa1 + t] = a1;
     }
     __syncthreads();
     if (t < 64) {
-        const float a2 = fmaxf(th[PL<H>().h2B + t] + head_dot(sa1, th + PL<H>().h2W + t, 128, 64, q), 0.f);
+        const float a2 = fmaxf(head_dot<LANES>(th[PL<H>().h2B + t], sa1, th + PL<H>().h2W + t, 128, 64, q), 0.f);
         if (q == 0) {
             sa2[t] = a2;
             S[kSa2 + t] = a2;
         }
     }
     __syncthreads();
-    if (t < 8) {                                  // one whole warp; five outputs
+    if (threadIdx.x < 32) {                       // one whole warp; five outputs
         const int o = min(t, 4);
-        const float v = th[PL<H>().h3B + o] + head_dot(sa2, th + PL<H>().h3W + o, 64, 5, q);
+        const float v = head_dot<LANES>(th[PL<H>().h3B + o], sa2, th + PL<H>().h3W + o, 64, 5, q);
         if (q == 0 && t < 5) c[g * 5 + t] = v;
     }
 }
@@ -955,7 +963,8 @@ static void forward_impl(GcinBatch &b, const float *th, cudaStream_t s) {
         k_pool_combine<H><<<G, CT, 0, s>>>(b.gchunk, b.gptr, csum, b.cmax, carg, b.pooled, b.argmax, l,
                                            nullptr, nullptr, nullptr); AMG_COUNT();
     }
-    k_head<H><<<G, kHeadThreads, 0, s>>>(b.pooled, th, b.head, b.c); AMG_COUNT();
+    if (b.infer) k_head<H, 4><<<G, 4 * kEmb, 0, s>>>(b.pooled, th, b.head, b.c);
+    else k_head<H, 1><<<G, kEmb, 0, s>>>(b.pooled, th, b.head, b.c); AMG_COUNT();
 }
 
 // The layer 2..4 B tiles of BF16 inference, laid out when the parameters are
