@@ -2166,7 +2166,7 @@ static void layout(amg_ctx *c, Planner &pl) {
     c->partials = pl.take<double>(5 * c->n_partials);  // up to 5 partial sums per block
     c->scal = pl.take<double>(nlev);
     c->wcoef = pl.take<float>(8 * static_cast<size_t>(nlev));
-    c->hist_cap = c->opt.max_iter + 1;
+    c->hist_cap = hist_capacity(c->opt.max_iter);
     char *out = pl.take<char>(kHistOffset + sizeof(double) * c->hist_cap);
     c->state = reinterpret_cast<SolveState *>(out);
     c->hist = out ? reinterpret_cast<double *>(out + kHistOffset) : nullptr;
@@ -2938,7 +2938,7 @@ int amg_spmv_device(amg_ctx *c, int level, const double *d_x, double *d_y, void 
 int amg_judge(amg_ctx *c, const double *b, int n_cycles, double *metric) {
     if (!c) return AMG_ERR_ARG;
     c->err.clear();
-    if (!b || !metric || n_cycles < 1 || n_cycles > 10000) return ctx_fail(c, "bad argument"), AMG_ERR_ARG;
+    if (!b || !metric || n_cycles < 1 || n_cycles > kMaxProbeCycles) return ctx_fail(c, "bad argument"), AMG_ERR_ARG;
     if (c->lev.empty()) return ctx_fail(c, "no hierarchy loaded"), AMG_ERR_STATE;
     if (!c->have_q) return ctx_fail(c, "no pseudo-inverse coefficients set"), AMG_ERR_STATE;
     CK(cudaSetDevice(c->opt.device));
@@ -2974,7 +2974,7 @@ int amg_judge(amg_ctx *c, const double *b, int n_cycles, double *metric) {
 int amg_reroute(amg_ctx *c, const double *b, int n_cycles, double *metric, int *smoother) {
     if (!c) return AMG_ERR_ARG;
     c->err.clear();
-    if (!b || n_cycles < 4 || n_cycles > 10000) return ctx_fail(c, "bad argument (n_cycles >= 4)"), AMG_ERR_ARG;
+    if (!b || n_cycles < 4 || n_cycles > kMaxProbeCycles) return ctx_fail(c, "bad argument (n_cycles >= 4)"), AMG_ERR_ARG;
     if (c->lev.empty()) return ctx_fail(c, "no hierarchy loaded"), AMG_ERR_STATE;
     if (!c->have_q) return ctx_fail(c, "no pseudo-inverse coefficients set"), AMG_ERR_STATE;
     CK(cudaSetDevice(c->opt.device));

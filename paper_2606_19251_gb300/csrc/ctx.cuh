@@ -93,6 +93,11 @@ struct SolveState {
 // solve's host outputs are one copy and one synchronisation.
 constexpr size_t kHistOffset = 256;            // bytes from the state to the history
 constexpr int kHistFirst = 512;                // history entries copied with the state
+// Largest n_cycles of amg_judge and amg_reroute: their probe solves run that
+// many cycles whatever the context's max_iter, into the same history.
+constexpr int kMaxProbeCycles = 10000;
+// History entries of a context (one per cycle and the first residual).
+constexpr int hist_capacity(int max_iter) { return (max_iter > kMaxProbeCycles ? max_iter : kMaxProbeCycles) + 1; }
 static_assert(sizeof(SolveState) <= kHistOffset, "the history follows the state");
 
 // Whole-solve CUDA graph: a kernel node copies the device-side status into
@@ -136,8 +141,8 @@ struct amg_ctx {
     int n_partials = 0;
     double *scal = nullptr;                    // device s_l
     amg::SolveState *state = nullptr;
-    double *hist = nullptr;                    // max_iter + 1, kHistOffset behind the state
-    int hist_cap = 0;
+    double *hist = nullptr;                    // hist_cap entries, kHistOffset behind the state
+    int hist_cap = 0;                          // hist_capacity(max_iter)
     int *dflag = nullptr;
     int *dcol_flag = nullptr;                  // per level: 1 if a column offset does not fit 16 bits
     char *arena = nullptr;
