@@ -561,13 +561,46 @@ __device__ __forceinline__ FloatPair lanes_sum_pair(FloatPair v, FloatPair (*red
 }
 __device__ __forceinline__ double pair_value(const FloatPair &v) { return static_cast<double>(v.h) + static_cast<double>(v.l); }
 
+// A pair sum that leaves FP32's range (or meets an infinity) ends with a
+// non-finite l; it is then taken again in FP64.  Such a total as a pair: h
+// scaled by 2^-64 and l = -inf, which no finite sum has.
+constexpr double kPairWide = 18446744073709551616.0;   // 2^64
+__device__ __forceinline__ FloatPair pair_of(double d) {
+    const float h = static_cast<float>(d);
+    if (isfinite(h)) return {h, static_cast<float>(d - static_cast<double>(h))};
+    return {static_cast<float>(d / kPairWide), -INFINITY};
+}
+__device__ __forceinline__ double pair_decode(const FloatPair &v) {
+    return v.l == -INFINITY ? static_cast<double>(v.h) * kPairWide : pair_value(v);
+}
+
+// Sum of term(t) over the parts a .. e - 1; the total in the threads with
+// tid < H.  Those alone convert it and take a sum past FP32's range again: the
+// conversion in every lane cost 0.9 us a launch (prediction on 50k rows 253 ->
+// 267 us).
+template <int H, class F>
+__device__ __forceinline__ double lanes_total(int a, int e, FloatPair (*red)[H], const F &term) {
+    const int q = threadIdx.x / H;
+    FloatPair s{0.f, 0.f};
+#pragma unroll 8
+    for (int t = a + q; t < e; t += kLanes) pair_add(s, term(t));
+    s = lanes_sum_pair<H>(s, red);
+    double d = 0.0;
+    if (q != 0) return d;
+    if (isfinite(s.l)) return pair_value(s);
+#pragma unroll 1
+    for (int t = a; t < e; ++t) d += static_cast<double>(term(t));
+    return d;
+}
+
 // Group statistics from part statistics (biased variance):
 // mean = sum_t n_t mean_t / n, M2 = sum_t [M2_t + n_t (mean_t - mean)^2].
 // Parts t of group g are gtile[g] .. gtile[g+1] with node ranges
 // tstart[t] .. tstart[t+1].  Run twice: tiles -> chunks (final = 0: writes
 // the chunk mean and M2 into mu / rstd) and chunks -> graphs (final = 1:
 // writes the instance-norm mean and 1/sqrt(var + eps)).  16 lanes of parts
-// per feature, summed as FP32 pairs; FP64 only for the totals' divisions.
+// per feature, summed as FP32 pairs; FP64 for the totals' divisions and for
+// sums past FP32's range (features of matrices with entries of 1e9 and more).
 // In FP64 each part cost two instructions of 64 cycles on a sub-partition's
 // FP64 unit (7 of a stage's 12 us on a 50k-node mesh); the part loops are
 // unrolled so that a thread's loads are in flight together.  With the
@@ -583,25 +616,19 @@ __global__ void __launch_bounds__(kLanes * H) k_stats_combine(const int *__restr
     __shared__ FloatPair red[kLanes][H];
     __shared__ float smean[H];
     const int g = blockIdx.x, f = threadIdx.x % H, q = threadIdx.x / H;
-    const int t0 = gtile[g] + q, t1 = gtile[g + 1];
-    FloatPair s{0.f, 0.f};
-#pragma unroll 8
-    for (int t = t0; t < t1; t += kLanes)
-        pair_add(s, static_cast<float>(tstart[t + 1] - tstart[t]) * tmean[static_cast<size_t>(t) * H + f]);
-    s = lanes_sum_pair<H>(s, red);
+    const int t0 = gtile[g], t1 = gtile[g + 1];
+    const double s = lanes_total<H>(t0, t1, red, [&](int t) {
+        return static_cast<float>(tstart[t + 1] - tstart[t]) * tmean[static_cast<size_t>(t) * H + f];
+    });
     const int n = gptr[g + 1] - gptr[g];
-    if (q == 0) smean[f] = static_cast<float>(pair_value(s) / n);
+    if (q == 0) smean[f] = static_cast<float>(s / n);
     __syncthreads();
     const float mf = smean[f];
-    FloatPair v{0.f, 0.f};
-#pragma unroll 8
-    for (int t = t0; t < t1; t += kLanes) {
+    const double m2 = lanes_total<H>(t0, t1, red, [&](int t) {
         const float d = tmean[static_cast<size_t>(t) * H + f] - mf;
-        pair_add(v, fmaf(static_cast<float>(tstart[t + 1] - tstart[t]) * d, d, tm2[static_cast<size_t>(t) * H + f]));
-    }
-    v = lanes_sum_pair<H>(v, red);
+        return fmaf(static_cast<float>(tstart[t + 1] - tstart[t]) * d, d, tm2[static_cast<size_t>(t) * H + f]);
+    });
     if (q == 0) {
-        const double m2 = pair_value(v);
         mu[static_cast<size_t>(g) * H + f] = mf;
         rstd[static_cast<size_t>(g) * H + f] =
             final ? static_cast<float>(1.0 / sqrt(m2 / n + static_cast<double>(kEps))) : static_cast<float>(m2);
@@ -713,6 +740,12 @@ __global__ void __launch_bounds__(kBlock, 6) k_norm_relu_pool_tile(const int *__
             pair_add(ts, ps[k * H]);
             bm = fmaxf(bm, pm[k * H]);
         }
+        if (!isfinite(ts.l)) {                   // past FP32's range
+            double d = 0.0;
+#pragma unroll 1
+            for (int k = 0; k < Q; ++k) d += static_cast<double>(ps[k * H]);
+            ts = pair_of(d);
+        }
         tsum[static_cast<size_t>(t) * H + ff] = ts;
         tmax[static_cast<size_t>(t) * H + ff] = bm;
         if (targ) {                              // the first node of the maximum
@@ -770,10 +803,16 @@ __global__ void __launch_bounds__(kLanes * H) k_pool_combine(const int *__restri
     }
     rm[q][f] = bm;
     ri[q][f] = bi;
-    const FloatPair total = lanes_sum_pair<H>(s, red);
+    FloatPair total = lanes_sum_pair<H>(s, red);
     if (q == 0) {
         for (int k = 1; k < kLanes; ++k)
             if (rm[k][f] > bm || (rm[k][f] == bm && ri[k][f] < bi)) { bm = rm[k][f]; bi = ri[k][f]; }
+        if (!isfinite(total.l)) {             // past FP32's range: in FP64
+            double d = 0.0;
+#pragma unroll 1
+            for (int t = gtile[g]; t < t1; ++t) d += pair_decode(tsum[static_cast<size_t>(t) * H + f]);
+            total = pair_of(d);
+        }
         if (csum) {
             const size_t o = static_cast<size_t>(g) * H + f;
             csum[o] = total;
@@ -782,7 +821,7 @@ __global__ void __launch_bounds__(kLanes * H) k_pool_combine(const int *__restri
             return;
         }
         float *P = pooled + (static_cast<size_t>(g) * kLayers + layer) * 2 * H;
-        P[f] = static_cast<float>(pair_value(total) / (gptr[g + 1] - gptr[g]));
+        P[f] = static_cast<float>(pair_decode(total) / (gptr[g + 1] - gptr[g]));
         P[H + f] = bm;
         if (targ) argmax[(static_cast<size_t>(g) * kLayers + layer) * H + f] = bi;
     }
