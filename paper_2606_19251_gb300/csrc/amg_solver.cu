@@ -3398,19 +3398,23 @@ namespace {
 
 // What dL/dc needs of the pseudo-inverse basis, in FP32 pairs (FP32 V-cycle)
 // or FP64: per entry x / (a_ii + a_jj) and x^2 / (a_ii + a_jj) with x = a_ij / s
-// (zero on the diagonal), per row (1, x, x^2) / a_ii with x = a_ii / s.  Laid
-// out with the training buffers.
+// (zero on the diagonal), per row (1, x, x^2) / a_ii with x = a_ii / s, all
+// times `scale`, the power of two next below s (adj_scale_log2): the values
+// are then of order one whatever the matrix's units.  Laid out with the
+// training buffers.
+constexpr int kAdjMaxLog2 = 120;   // scale factors stay normal FP32 numbers
 template <class V> struct AdjBasis {
     const V *o1, *o2, *d;
 };
 template <class V>
 __global__ void __launch_bounds__(kBlock) k_adj_basis(int n, const int *__restrict__ rp, const int *__restrict__ col,
                                                       const double *__restrict__ bx, const double *__restrict__ bw,
-                                                      V *__restrict__ o1, V *__restrict__ o2, V *__restrict__ d) {
+                                                      double scale, V *__restrict__ o1, V *__restrict__ o2,
+                                                      V *__restrict__ d) {
     const int i = blockIdx.x * kBlock + threadIdx.x;
     if (i >= n) return;
     for (int p = rp[i]; p < rp[i + 1]; ++p) {
-        const double x = bx[p], w = bw[p];
+        const double x = bx[p], w = bw[p] * scale;
         const bool diag = col[p] == i;
         tail_set(o1[p], diag ? 0.0 : w * x);
         tail_set(o2[p], diag ? 0.0 : w * x * x);
@@ -3434,11 +3438,15 @@ __global__ void __launch_bounds__(kBlock) k_adj_basis(int n, const int *__restri
 // basis entries are loaded ahead of the grid-dependency wait.  With the FP32
 // V-cycle the gradient's sums are FP32 pairs: in FP64 they were about 100
 // instructions a warp of 64 cycles each on a sub-partition's FP64 unit (7 of
-// the pass's 9 us on every level).
+// the pass's 9 us on every level).  A pair has FP32's exponents, so its
+// operands are brought to order one by powers of two, which cancel in the
+// product: r by sc[0] and ubar, which goes as a / ||r||, by sc[1] = 1 / sc[0]
+// (k_loss_seed) and by us = 1 / scale of the basis.
 template <class T, class V, int TPR>
 __global__ void __launch_bounds__(kBlock) k_adj_sweep(int n, const int *__restrict__ rp, const int *__restrict__ col,
                                                       const T *__restrict__ q, AdjBasis<V> basis, const T *ubar,
-                                                      const T *r, T *rbar, T *bbar, int assign, double *partial) {
+                                                      const T *r, T *rbar, T *bbar, int assign, double *partial,
+                                                      const float *sc, T us) {
     constexpr int E = 4;
     const int gid = blockIdx.x * kBlock + threadIdx.x;
     const int row = gid / TPR, lane = gid % TPR;
@@ -3469,6 +3477,7 @@ __global__ void __launch_bounds__(kBlock) k_adj_sweep(int n, const int *__restri
         for (int k = 0; k < 3; ++k) d[k] = basis.d[3 * static_cast<size_t>(row) + k];
     }
     pdl_wait_and_release();
+    const T sr = sc[0], su = sc[1];
     const T ui = row < n ? load_now(ubar + row) : T(0), ri = own ? load_now(r + row) : T(0);
     const T bi = own && !assign ? load_now(bbar + row) : T(0);
     T acc = T(0);
@@ -3484,19 +3493,20 @@ __global__ void __launch_bounds__(kBlock) k_adj_sweep(int n, const int *__restri
 #pragma unroll
         for (int j = 0; j < E; ++j) {
             acc += m[j] * uj[j];
-            tail_fma(g[3], rj[j], o1[j]);
-            tail_fma(g[4], rj[j], o2[j]);
+            tail_fma(g[3], rj[j] * sr, o1[j]);
+            tail_fma(g[4], rj[j] * sr, o2[j]);
         }
         if (base + E * TPR < end) fetch(base + E * TPR);
     }
     acc = group_sum<TPR>(acc);
-    g[3] = adj_scale(ui, g[3]);
-    g[4] = adj_scale(ui, g[4]);
+    const T uv = ui * (su * us);   // the factors first: ui alone may be near FP32's lowest normal number
+    g[3] = adj_scale(uv, g[3]);
+    g[4] = adj_scale(uv, g[4]);
     if (own) {
         if (rbar) rbar[row] = acc;
         bbar[row] = assign ? acc : bi + acc;
 #pragma unroll
-        for (int k = 0; k < 3; ++k) g[k] = adj_prod(ui, ri, d[k]);
+        for (int k = 0; k < 3; ++k) g[k] = adj_prod(uv, ri * sr, d[k]);
     }
     __shared__ V red[5][kBlock / 32];
 #pragma unroll
@@ -3580,8 +3590,10 @@ __global__ void __launch_bounds__(kBlock) k_loss_dots(int n, const T *r, const T
     block_partial2(a, b, prr, pff);
 }
 
-// scal[0] = r.r, scal[1] = f.f and seed = r / (ln 10 r.r): every block sums
-// the partials (in the same order), so no launch stands between
+// scal[0] = r.r, scal[1] = f.f, after them two floats, the power of two that
+// brings r to order one and its inverse (for the gradient's sums), and seed =
+// r / (ln 10 r.r): every block sums the partials (in the same order), so no
+// launch stands between
 template <class T>
 __global__ void __launch_bounds__(kBlock) k_loss_seed(int n, const T *r, T *seed, const double *prr, const double *pff,
                                                       int np, double *scal) {
@@ -3592,10 +3604,20 @@ __global__ void __launch_bounds__(kBlock) k_loss_seed(int n, const T *r, T *seed
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         scal[0] = rr;
         scal[1] = ff;
+        const int e = (rr > 0.0 && isfinite(rr)) ? max(-kAdjMaxLog2, min(kAdjMaxLog2, ilogb(sqrt(rr / n)))) : 0;
+        float *sc = reinterpret_cast<float *>(scal + 2);
+        sc[0] = ldexpf(1.0f, -e);
+        sc[1] = ldexpf(1.0f, e);
     }
     const double a = 1.0 / (2.302585092994045684 * rr);
     for (int i = blockIdx.x * kBlock + threadIdx.x; i < n; i += gridDim.x * kBlock)
         seed[i] = static_cast<T>(a * static_cast<double>(r[i]));
+}
+
+// Exponent of the power of two next below a level's largest coupling.
+int adj_scale_log2(const amg_ctx *c, int l) {
+    const double s = c->scales[l];
+    return (s > 0.0 && std::isfinite(s)) ? std::max(-kAdjMaxLog2, std::min(kAdjMaxLog2, std::ilogb(s))) : 0;
 }
 
 struct TrainBufs {
@@ -3607,8 +3629,9 @@ struct TrainBufs {
     std::vector<int> nblk;
     double *f = nullptr, *zero = nullptr;   // level 0: right-hand side, zeros
     double *xu = nullptr;          // level-0 iterate of the multi-cycle loss
-    double *dcoef = nullptr;       // n_levels x 5, then r.r and f.f
-    double *h_out = nullptr;       // pinned copy of dcoef
+    double *dcoef = nullptr;       // n_levels x 5, then r.r, f.f and the gradient sums' scale (two floats)
+    double *h_out = nullptr;       // pinned copy of dcoef up to f.f
+    const float *scale() const { return reinterpret_cast<const float *>(dcoef + 5 * nlev + 2); }
     size_t part_bytes = 0;
     char *arena = nullptr;
     cudaGraphExec_t exec = nullptr;   // the call's kernels for graph_nvc cycles (from its second call on)
@@ -3643,6 +3666,7 @@ template <class V>
 void adj_basis(amg_ctx *c, const TrainBufs &tb, int l) {
     const DevLevel &L = c->lev[l];
     k_adj_basis<V><<<grid_for(L.n), kBlock, 0, c->stream>>>(L.n, L.A.rp, L.A.col, L.bx, L.bw,
+                                                            std::ldexp(1.0, adj_scale_log2(c, l)),
                                                             reinterpret_cast<V *>(tb.o1[l]), reinterpret_cast<V *>(tb.o2[l]),
                                                             reinterpret_cast<V *>(tb.od[l])); AMG_COUNT();
 }
@@ -3691,7 +3715,7 @@ int train_bufs(amg_ctx *c, TrainBufs &tb, int ncyc) {
             tb.part[l] = p;
             if (p) p += 5 * static_cast<size_t>(tb.nblk[l]);
         }
-        tb.dcoef = pl.take<double>(static_cast<size_t>(nlev) * 5 + 2);
+        tb.dcoef = pl.take<double>(static_cast<size_t>(nlev) * 5 + 3);
     };
     Planner pl;
     lay(pl);
@@ -3731,6 +3755,7 @@ void launch_train_tail(amg_ctx *c, TrainBufs &tb, int cyc, const T *in, T *out, 
     a.LinvT = c->LinvT;
     a.in = in;
     a.out = out;
+    a.scale = tb.scale();
     for (int k = 0; k < a.nlev; ++k) {
         const int l = tb.tail + k;
         const DevLevel &L = c->lev[l];
@@ -3757,6 +3782,7 @@ void launch_train_tail(amg_ctx *c, TrainBufs &tb, int cyc, const T *in, T *out, 
         D.ck = reinterpret_cast<T *>(tb.slot(cyc, l, 0));
         D.stride = tb.nsw > 1 ? reinterpret_cast<T *>(tb.slot(cyc, l, 1)) - D.ck : 0;
         D.partial = tb.part[l];
+        D.us = static_cast<T>(std::ldexp(1.0, -adj_scale_log2(c, l)));
     }
     const size_t smem = train_tail_smem(ADJ ? 4 : 3, a.rows, sizeof(T));
     if (ADJ) {
@@ -3805,13 +3831,13 @@ T *fwd_level_ckpt(amg_ctx *c, TrainBufs &tb, int cyc, int l, cudaStream_t s) {
 template <class T> struct AdjLaunch {
     template <int TPR>
     static void sweep(const DevLevel &L, const TrainBufs &tb, int l, const T *ubar, const T *r, T *rbar, T *bbar,
-                      int assign, cudaStream_t s) {
+                      int assign, T us, cudaStream_t s) {
         using V = typename std::conditional<std::is_same<T, float>::value, FloatPair, double>::type;
         const AdjBasis<V> basis{reinterpret_cast<const V *>(tb.o1[l]), reinterpret_cast<const V *>(tb.o2[l]),
                                 reinterpret_cast<const V *>(tb.od[l])};
         launch_pdl(k_adj_sweep<T, V, TPR>, dim3(grid_for(static_cast<long long>(L.n) * TPR)), dim3(kBlock), 0, s, L.n,
                    L.A.rp, static_cast<const int *>(L.A.col), qvals<T>(L), basis, ubar, r, rbar, bbar, assign,
-                   tb.part[l]);
+                   tb.part[l], tb.scale(), us);
     }
     template <int TPR>
     static void restrict_(const DevMat &P, const T *x, T *rhobar, T *bbar, int assign, cudaStream_t s) {
@@ -3840,13 +3866,14 @@ void bwd_level(amg_ctx *c, TrainBufs &tb, int cyc, int l, const T *in, T *other,
     T *out = reinterpret_cast<T *>(tb.tmp[l]), *spare = other;
     T *rbar = reinterpret_cast<T *>(L.vt);            // free during the backward pass
     int assign = 1;                                   // bbar's first contribution replaces the last call's
+    const T us = static_cast<T>(std::ldexp(1.0, -adj_scale_log2(c, l)));
     auto advance = [&]() {
         ub = out;
         std::swap(out, spare);
     };
     auto sweep = [&](int k) {                         // ubar <- ubar - A (M ubar), bbar += M ubar
         TPR_DISPATCH(L.A.tpr, AdjLaunch<T>::template sweep, L, tb, l, ub,
-                     reinterpret_cast<const T *>(tb.slot(cyc, l, k)), rbar, bb, assign, s);
+                     reinterpret_cast<const T *>(tb.slot(cyc, l, k)), rbar, bb, assign, us, s);
         assign = 0;
         L_resid<T>(L.A, ub, rbar, out, s);
         advance();
@@ -3865,7 +3892,7 @@ void bwd_level(amg_ctx *c, TrainBufs &tb, int cyc, int l, const T *in, T *other,
     for (int k = nu1 - 1; k >= 1; --k) sweep(k);
     if (nu1 >= 1) {        // first sweep from zero: u = M b
         TPR_DISPATCH(L.A.tpr, AdjLaunch<T>::template sweep, L, tb, l, ub,
-                     static_cast<const T *>(level_b<T>(c, tb, cyc, l)), static_cast<T *>(nullptr), bb, 0, s);
+                     static_cast<const T *>(level_b<T>(c, tb, cyc, l)), static_cast<T *>(nullptr), bb, 0, us, s);
     }
 }
 

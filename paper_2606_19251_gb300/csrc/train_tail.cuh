@@ -54,6 +54,7 @@ template <class T, class V> struct TrainTailLevel {
     T *ck;                              // this cycle's checkpoints
     long long stride;                   // elements between them
     double *partial;                    // five sums of dL/dc
+    T us;                               // the basis's scale (k_adj_sweep), inverted
 };
 template <class T, class V> struct TrainTailArgs {
     int nlev, nu1, nu2, rows;           // rows: all levels together
@@ -61,6 +62,7 @@ template <class T, class V> struct TrainTailArgs {
     const double *Linv, *LinvT;
     const T *in;                        // b (forward) or dL/d(output) (adjoint) of the first level
     T *out;                             // u (forward) or dL/db (adjoint) of the first level
+    const float *scale;                 // r's and ubar's scale in the gradient sums (adjoint)
 };
 
 // One row's sum over `tpr` lanes, in the order of row_dot and group_sum.
@@ -235,11 +237,12 @@ __global__ void __launch_bounds__(kTtThreads) k_train_tail_adj(const __grid_cons
         }
         __syncthreads();
     };
+    T sr = T(1), su = T(1);
     // rbar = M ubar, bbar (+)= rbar, and the sweep's share of dL/dc with the checkpoint ck
     auto sweep = [&](const TrainTailLevel<T, V> &L, const T *ck, bool assign) {
         const T *ub = sub + L.off;
         T *bb = sbb + L.off, *rb = srb + L.off, *r = sk + L.off;
-        for (int i = threadIdx.x; i < L.n; i += kTtThreads) r[i] = ck[i];
+        for (int i = threadIdx.x; i < L.n; i += kTtThreads) r[i] = ck[i] * sr;
         __syncthreads();
         const int tpr = 1 << L.la, lane = threadIdx.x & (tpr - 1);
         for (int base = 0; base < L.n; base += kTtThreads >> L.la) {
@@ -254,7 +257,7 @@ __global__ void __launch_bounds__(kTtThreads) k_train_tail_adj(const __grid_cons
                     tail_fma(s3, r[j], L.o1[p]);
                     tail_fma(s4, r[j], L.o2[p]);
                 }
-                const T ui = ub[row];
+                const T ui = ub[row] * (su * L.us);
                 adj_add(g[3], adj_scale(ui, s3));
                 adj_add(g[4], adj_scale(ui, s4));
                 if (lane == 0) {
@@ -276,6 +279,8 @@ __global__ void __launch_bounds__(kTtThreads) k_train_tail_adj(const __grid_cons
     };
     tt_stage(A.lev[last].n, A.Linv, A.LinvT, sL);
     pdl_wait_and_release();
+    sr = A.scale[0];
+    su = A.scale[1];
     for (int i = threadIdx.x; i < A.lev[0].n; i += kTtThreads) sub[i] = A.in[i];
     __syncthreads();
     for (int l = 0; l < last; ++l) {
