@@ -4021,13 +4021,19 @@ extern "C" int amg_loss_grad(amg_ctx *c, const double *coef, const double *f, in
             if (tb->arena) cudaFree(tb->arena);
             if (tb->h_out) cudaFreeHost(tb->h_out);
             delete tb;
-            return rc;
+        } else {
+            c->train = tb;
         }
-        c->train = tb;
     }
-    TrainBufs &tb = *static_cast<TrainBufs *>(c->train);
-    if (c->opt.precision == AMG_FP64) return loss_grad<double>(c, tb, f, n_vc, loss, dc);
-    return loss_grad<float>(c, tb, f, n_vc, loss, dc);
+    if (!rc) {
+        TrainBufs &tb = *static_cast<TrainBufs *>(c->train);
+        rc = c->opt.precision == AMG_FP64 ? loss_grad<double>(c, tb, f, n_vc, loss, dc)
+                                          : loss_grad<float>(c, tb, f, n_vc, loss, dc);
+    }
+    // the new coefficients are in force: after an error, too, their assembly has
+    // ended when the call returns (the next call may run on another stream)
+    if (rc) cudaStreamSynchronize(c->stream);
+    return rc;
 }
 
 namespace amg {
