@@ -1463,8 +1463,19 @@ static T *wf_smooth(amg_ctx *c, int l, cudaStream_t s, const T *b, T *u_in, int 
 // ---------------------------------------------------------------------------
 // V-cycle driver
 // ---------------------------------------------------------------------------
+// Two Jacobi sweeps from zero in one pass on a two-pass level: in FP32 only
+// (1025^2 grid: V-cycle 176.0 -> 169.5 us).  The pass forms omega / a_jj b_j at
+// every entry, which in FP64 doubles the work of GB300's narrow FP64 unit (FP64
+// V-cycles in two passes / in one: 5-point grid of 0.9M rows 297 / 324 us, 1.5M
+// rows 457 / 502; 7-point grid of 1M rows 971 / 1095; 900k unstructured rows
+// 350 / 382).
+template <class T> static bool first_two_in_one(bool gnn, bool zero_init, int nsweeps) {
+    return std::is_same<T, float>::value && !gnn && zero_init && nsweeps >= 2;
+}
+
 // Smoothing sweeps on level l; returns the buffer holding the result (Jacobi
 // alternates between cur and alt).
+
 template <class T>
 static T *smooth(amg_ctx *c, int l, cudaStream_t s, const T *b, T *cur, T *alt, T *r, int nsweeps,
                  bool zero_init) {
@@ -1473,8 +1484,7 @@ static T *smooth(amg_ctx *c, int l, cudaStream_t s, const T *b, T *cur, T *alt, 
     if (nsweeps == 0 && zero_init) cudaMemsetAsync(cur, 0, sizeof(T) * L.n, s);
     if (c->smoother == AMG_SMOOTHER_CHEB) return cheb_smooth<T>(c, L, s, b, cur, alt, nsweeps, zero_init);
     int k = 0;
-    // two Jacobi sweeps from zero in one pass (1025^2 grid: V-cycle 176.0 -> 169.5 us)
-    if (!gnn && zero_init && nsweeps >= 2) {
+    if (first_two_in_one<T>(gnn, zero_init, nsweeps)) {
         TPR_DISPATCH(L.A.tpr, Launch<T>::template jacobi_first2, L.A, jvals<T>(L), b, cur, s);
         k = 2;
     }
@@ -3069,7 +3079,7 @@ double smooth_bytes(const amg_ctx *c, const DevLevel &L, int tb, int nsweeps, bo
     const bool gnn = (c->smoother == AMG_SMOOTHER_GNN);
     double b = 0.0;
     int k = 0;
-    if (!gnn && zero_init && nsweeps >= 2) {
+    if (tb == 4 ? first_two_in_one<float>(gnn, zero_init, nsweeps) : first_two_in_one<double>(gnn, zero_init, nsweeps)) {
         b += pass_bytes(L.A, tb, 2.0 * L.n, 1);                                // two Jacobi sweeps
         k = 2;
     }
