@@ -1636,7 +1636,7 @@ static int build_tail(amg_ctx *c, int sm, cudaStream_t s) {
         D.R = {L.R.rp, L.R.col, mvals<T>(L.R)};
         D.m = sm ? qvals<T>(L) : jvals<T>(L);
     }
-    using V = typename std::conditional<std::is_same<T, float>::value, FloatPair, double>::type;
+    using V = typename TailValue<T>::type;
     const size_t smem = static_cast<size_t>(off) * sizeof(V);
     CK(cudaFuncSetAttribute(k_tail_build<T, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kTailSmem)));
     k_tail_build<T, V><<<(c->lev[t.level].n + kTailCols - 1) / kTailCols, kTailThreads, smem, s>>>(a); AMG_COUNT();
@@ -1661,10 +1661,11 @@ static void launch_tail(const DevTail &t, int n, const T *b, T *e, cudaStream_t 
     const T *B = static_cast<const T *>(t.B);
     const dim3 g((n + kBlock / 32 - 1) / (kBlock / 32));
     const int loads = (t.ld * static_cast<int>(sizeof(T)) + 511) / 512;   // 16-byte loads per lane and row
+    static_assert(kTailRows * sizeof(T) <= 512 * (sizeof(T) == 8 ? 16 : 8), "the largest instantiation holds a row");
     if (loads <= 2) launch_pdl(k_tail_apply<T, 2>, g, dim3(kBlock), 0, s, n, t.ld, B, b, e);
     else if (loads <= 4) launch_pdl(k_tail_apply<T, 4>, g, dim3(kBlock), 0, s, n, t.ld, B, b, e);
     else if (loads <= 8) launch_pdl(k_tail_apply<T, 8>, g, dim3(kBlock), 0, s, n, t.ld, B, b, e);
-    else launch_pdl(k_tail_apply<T, 16>, g, dim3(kBlock), 0, s, n, t.ld, B, b, e);
+    else if constexpr (sizeof(T) == 8) launch_pdl(k_tail_apply<T, 16>, g, dim3(kBlock), 0, s, n, t.ld, B, b, e);
 }
 
 // Smoothing on a latency-optimised level: every pseudo-inverse sweep is one
@@ -2162,7 +2163,7 @@ static void layout(amg_ctx *c, Planner &pl) {
         const size_t tb = c->opt.precision == AMG_FP64 ? sizeof(double) : sizeof(float);
         t.level = tl;
         t.ld = static_cast<int>((n * tb + 511) / 512 * 512 / tb);
-        t.B = pl.take<char>(tb * n * t.ld);
+        t.B = pl.take<char>(sizeof(double) * n * t.ld);   // FP64, or FP32 pairs
     }
     const int n0 = c->host[0].A.n_rows;
     c->ell_ptr = pl.take<int>(c->h_ell_ptr.size());
@@ -3119,7 +3120,7 @@ double vcycle_bytes_level(const amg_ctx *c, int l, int tb) {
     const int nlev = static_cast<int>(c->lev.size());
     if (l == nlev - 1) return 8.0 * c->nL * c->nL + 2.0 * tb * c->nL;
     if (tail_of(const_cast<amg_ctx *>(c)) && tail_of(const_cast<amg_ctx *>(c))->level == l)
-        return 1.0 * tb * L.n * L.n + 2.0 * tb * L.n;   // the coarse tail's dense operator
+        return 8.0 * L.n * L.n + 2.0 * tb * L.n;   // the coarse tail's dense operator (FP64 or FP32 pairs)
     const bool cheb = (c->smoother == AMG_SMOOTHER_CHEB);
     const int nu1 = cheb ? (c->opt.nu1 > 0 ? 1 : 0) : c->opt.nu1;
     const int nu2 = cheb ? (c->opt.nu2 > 0 ? 1 : 0) : c->opt.nu2;
@@ -3522,14 +3523,14 @@ __global__ void __launch_bounds__(kBlock) k_adj_sweep(int n, const int *__restri
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) adj_add(g[k], adj_shfl(g[k], o));
+        for (int o = 16; o > 0; o >>= 1) tail_add(g[k], tail_shfl(g[k], o));
         if (threadIdx.x % 32 == 0) red[k][threadIdx.x / 32] = g[k];
     }
     __syncthreads();
     if (threadIdx.x < 5) {
         V t = red[threadIdx.x][0];
 #pragma unroll
-        for (int k = 1; k < kBlock / 32; ++k) adj_add(t, red[threadIdx.x][k]);
+        for (int k = 1; k < kBlock / 32; ++k) tail_add(t, red[threadIdx.x][k]);
         partial[blockIdx.x * 5 + threadIdx.x] += tail_get(t);
     }
 }
@@ -3756,7 +3757,7 @@ T *level_b(amg_ctx *c, const TrainBufs &tb, int cyc, int l) {
 
 template <class T, bool ADJ>
 void launch_train_tail(amg_ctx *c, TrainBufs &tb, int cyc, const T *in, T *out, cudaStream_t s) {
-    using V = typename std::conditional<std::is_same<T, float>::value, FloatPair, double>::type;
+    using V = typename TailValue<T>::type;
     TrainTailArgs<T, V> a{};
     a.nlev = tb.nlev - tb.tail;
     a.nu1 = c->opt.nu1;
@@ -3842,7 +3843,7 @@ template <class T> struct AdjLaunch {
     template <int TPR>
     static void sweep(const DevLevel &L, const TrainBufs &tb, int l, const T *ubar, const T *r, T *rbar, T *bbar,
                       int assign, T us, cudaStream_t s) {
-        using V = typename std::conditional<std::is_same<T, float>::value, FloatPair, double>::type;
+        using V = typename TailValue<T>::type;
         const AdjBasis<V> basis{reinterpret_cast<const V *>(tb.o1[l]), reinterpret_cast<const V *>(tb.o2[l]),
                                 reinterpret_cast<const V *>(tb.od[l])};
         launch_pdl(k_adj_sweep<T, V, TPR>, dim3(grid_for(static_cast<long long>(L.n) * TPR)), dim3(kBlock), 0, s, L.n,

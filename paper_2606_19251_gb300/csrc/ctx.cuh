@@ -65,7 +65,7 @@ struct WfPlan {
 struct DevTail {
     int level = -1;                            // first level of the tail, or -1
     int ld = 0;                                // row stride of B (entries)
-    void *B = nullptr;                         // in the V-cycle precision
+    void *B = nullptr;                         // FP64, or high and low words of FP32 pairs (FP32 V-cycle)
     bool ok = false;                           // B belongs to the smoother's current values
 };
 

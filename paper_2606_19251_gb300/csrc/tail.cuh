@@ -10,8 +10,9 @@
 // unstructured rows 71 -> 52 / 173 -> 138 us, on a 1025^2 grid (Jacobi)
 // 209 -> 186 us; a whole FP64 solve on a 64^2 grid 926 -> 681 us; prediction
 // and solve on the 50k mesh 4.43 -> 3.60 ms with B re-formed in every pass.
-// The error of a V-cycle against 64 bits stays where it was (1.2e-7 to
-// 2.6e-7 on those meshes on both sides).
+//
+// The coarsest solve of an FP32 V-cycle is FP64, so B is held and applied in
+// FP32 pairs (about 48 bits) and e is rounded once: PRECISION_FIGURES
 #pragma once
 #include <cuda_runtime.h>
 
@@ -30,9 +31,9 @@ constexpr int kTailThreads = 512;
 constexpr size_t kTailSmem = 220 * 1024;         // shared memory a tail's level vectors may take
 constexpr double kTailCoarseWork = 134217728.0;  // n_t n_L^2 bound: the FP64 coarsest solves of the n_t columns
 
-// The FP32 V-cycle's B is formed in FP32 pairs (FloatPair) and rounded once
-// to FP32: GB300 runs 64 FP32 FMAs for each FP64 one, so the ten FP32
-// operations of a pair FMA are ~6x cheaper than a DFMA.
+// The FP32 V-cycle's B is formed in FP32 pairs (FloatPair): GB300 runs 64
+// FP32 FMAs for each FP64 one, so the ten FP32 operations of a pair FMA are
+// ~6x cheaper than a DFMA.
 // acc += a x (Dekker / Knuth error-free product and sum)
 __device__ __forceinline__ void tail_fma(FloatPair &acc, float a, const FloatPair &x) {
     const float p = __fmul_rn(a, x.h);
@@ -54,8 +55,28 @@ __device__ __forceinline__ void tail_set(FloatPair &v, double x) {
 __device__ __forceinline__ void tail_set(double &v, double x) { v = x; }
 __device__ __forceinline__ double tail_get(const FloatPair &v) { return static_cast<double>(v.h) + static_cast<double>(v.l); }
 __device__ __forceinline__ double tail_get(double v) { return v; }
-__device__ __forceinline__ void tail_round(float &o, const FloatPair &v) { o = __fadd_rn(v.h, v.l); }
-__device__ __forceinline__ void tail_round(double &o, double v) { o = v; }
+__device__ __forceinline__ float tail_round(const FloatPair &v) { return __fadd_rn(v.h, v.l); }
+__device__ __forceinline__ double tail_round(double v) { return v; }
+// B's entry k (and, `lo` entries behind it, a pair's low word)
+__device__ __forceinline__ void tail_store(float *B, size_t lo, size_t k, const FloatPair &v) {
+    B[k] = v.h;
+    B[lo + k] = v.l;
+}
+__device__ __forceinline__ void tail_store(double *B, size_t, size_t k, double v) { B[k] = v; }
+__device__ __forceinline__ void tail_add(FloatPair &a, const FloatPair &b) { pair_add(a, b.h, b.l); }
+__device__ __forceinline__ void tail_add(double &a, double b) { a += b; }
+__device__ __forceinline__ FloatPair tail_shfl(const FloatPair &v, int o) {
+    return {__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)};
+}
+__device__ __forceinline__ double tail_shfl(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+
+// What T's values are held in while B is formed and applied.
+template <class T> struct TailValue {
+    using type = double;
+};
+template <> struct TailValue<float> {
+    using type = FloatPair;
+};
 
 template <class T> struct TailCsr {
     const int *rp, *col;
@@ -72,7 +93,7 @@ template <class T> struct TailArgs {
     int nlev, nu1, nu2, pinv, ld;
     TailLevel<T> lev[kTailMaxLevels];
     const double *Linv, *LinvT;
-    T *B;                       // n_t rows of ld entries
+    T *B;                       // n_t rows of ld entries (FP32: the low words n_t ld entries behind)
 };
 
 // acc[c] = (NEG ? -1 : 1) sum_k m_ik x_kc of one CSR row and kTailCols columns
@@ -224,53 +245,65 @@ __global__ void __launch_bounds__(kTailThreads) k_tail_build(const __grid_consta
     const V *u = sm + A.lev[0].off + nt * kTailCols;
     for (int e = threadIdx.x; e < nt * kTailCols; e += kTailThreads) {
         const int i = e / kTailCols, j = j0 + e % kTailCols;
-        if (j < nt) tail_round(A.B[static_cast<size_t>(i) * A.ld + j], u[e]);
+        if (j < nt) tail_store(A.B, static_cast<size_t>(nt) * A.ld, static_cast<size_t>(i) * A.ld + j, u[e]);
     }
 }
 
-// e = B b: a warp per row, its whole row of B (at most 4 J entries of 16
-// bytes per lane group) in registers before the grid-dependency wait (B is
+// e = B b: a warp per row, its whole row of B (J 16-byte loads per lane, and
+// as many of the low words) in registers before the grid-dependency wait (B is
 // constant during a solve), so only the loads of b follow the previous
 // kernel.  ld is n rounded up to 512 bytes; the padding of B is zero.
 template <class T, int J>
 __global__ void __launch_bounds__(kBlock) k_tail_apply(int n, int ld, const T *__restrict__ B,
                                                        const T *__restrict__ b, T *__restrict__ e) {
+    constexpr bool kPair = sizeof(T) == 4;
     constexpr int W = 16 / sizeof(T);          // entries per 16-byte load
+    using V = typename TailValue<T>::type;
     struct alignas(16) Vec { T v[W]; };
     const int row = blockIdx.x * (kBlock / 32) + static_cast<int>(threadIdx.x >> 5), lane = threadIdx.x & 31;
-    Vec m[J];
+    Vec m[J], ml[kPair ? J : 1];
+    const T *Br = B + static_cast<size_t>(row) * ld, *Bl = Br + static_cast<size_t>(n) * ld;
 #pragma unroll
     for (int j = 0; j < J; ++j) {
         const int k = (j * 32 + lane) * W;
-        if (row < n && k < ld) {
-            m[j] = *reinterpret_cast<const Vec *>(B + static_cast<size_t>(row) * ld + k);
-        } else {
+        const bool in = row < n && k < ld;
 #pragma unroll
-            for (int q = 0; q < W; ++q) m[j].v[q] = T(0);
+        for (int q = 0; q < W; ++q) m[j].v[q] = T(0);
+        if (in) m[j] = *reinterpret_cast<const Vec *>(Br + k);
+        if constexpr (kPair) {
+#pragma unroll
+            for (int q = 0; q < W; ++q) ml[j].v[q] = T(0);
+            if (in) ml[j] = *reinterpret_cast<const Vec *>(Bl + k);
         }
     }
     pdl_wait_and_release();
     if (row >= n) return;
-    T acc[W];
+    V acc[W];
 #pragma unroll
-    for (int q = 0; q < W; ++q) acc[q] = T(0);
+    for (int q = 0; q < W; ++q) tail_set(acc[q], 0.0);
+    auto add = [&](int j, int q, T x) {
+        if constexpr (kPair) tail_fma(acc[q], x, FloatPair{m[j].v[q], ml[j].v[q]});
+        else tail_fma(acc[q], x, m[j].v[q]);
+    };
 #pragma unroll
     for (int j = 0; j < J; ++j) {
         const int k = (j * 32 + lane) * W;
         if (k + W <= n) {
             const Vec x = *reinterpret_cast<const Vec *>(b + k);
 #pragma unroll
-            for (int q = 0; q < W; ++q) acc[q] += m[j].v[q] * x.v[q];
+            for (int q = 0; q < W; ++q) add(j, q, x.v[q]);
         } else {
 #pragma unroll
             for (int q = 0; q < W; ++q)
-                if (k + q < n) acc[q] += m[j].v[q] * b[k + q];
+                if (k + q < n) add(j, q, b[k + q]);
         }
     }
-    T s = acc[0] + acc[1];
-    if constexpr (W == 4) s += acc[2] + acc[3];
-    s = warp_sum(s);
-    if (lane == 0) e[row] = s;
+    V s = acc[0];
+#pragma unroll
+    for (int q = 1; q < W; ++q) tail_add(s, acc[q]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) tail_add(s, tail_shfl(s, o));
+    if (lane == 0) e[row] = tail_round(s);
 }
 
 }  // namespace amg

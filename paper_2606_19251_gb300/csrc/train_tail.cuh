@@ -23,8 +23,6 @@ constexpr int kTtThreads = 1024;
 constexpr int kTtCoarse = 64;           // largest coarsest level
 constexpr int kTtLd = kTtCoarse + 1;    // row stride of its factors in shared memory
 
-__device__ __forceinline__ void adj_add(FloatPair &a, const FloatPair &b) { pair_add(a, b.h, b.l); }
-__device__ __forceinline__ void adj_add(double &a, double b) { a += b; }
 // u r v for the row's own values u, r and a basis value v
 __device__ __forceinline__ FloatPair adj_prod(float u, float r, const FloatPair &v) {
     const float t = __fmul_rn(u, r), tl = __fmaf_rn(u, r, -t);
@@ -40,10 +38,6 @@ __device__ __forceinline__ FloatPair adj_scale(float u, const FloatPair &v) {
     return o;
 }
 __device__ __forceinline__ double adj_scale(double u, double v) { return u * v; }
-__device__ __forceinline__ FloatPair adj_shfl(const FloatPair &v, int o) {
-    return {__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)};
-}
-__device__ __forceinline__ double adj_shfl(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 
 template <class T, class V> struct TrainTailLevel {
     int n, off;                         // rows; first row in the concatenated level vectors
@@ -226,13 +220,13 @@ __global__ void __launch_bounds__(kTtThreads) k_train_tail_adj(const __grid_cons
 #pragma unroll
         for (int k = 0; k < 5; ++k) {
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) adj_add(g[k], adj_shfl(g[k], o));
+            for (int o = 16; o > 0; o >>= 1) tail_add(g[k], tail_shfl(g[k], o));
             if (threadIdx.x % 32 == 0) red[k][threadIdx.x / 32] = g[k];
         }
         __syncthreads();
         if (threadIdx.x < 5) {
             V t = red[threadIdx.x][0];
-            for (int k = 1; k < kTtThreads / 32; ++k) adj_add(t, red[threadIdx.x][k]);
+            for (int k = 1; k < kTtThreads / 32; ++k) tail_add(t, red[threadIdx.x][k]);
             L.partial[threadIdx.x] += tail_get(t);
         }
         __syncthreads();
@@ -258,11 +252,11 @@ __global__ void __launch_bounds__(kTtThreads) k_train_tail_adj(const __grid_cons
                     tail_fma(s4, r[j], L.o2[p]);
                 }
                 const T ui = ub[row] * (su * L.us);
-                adj_add(g[3], adj_scale(ui, s3));
-                adj_add(g[4], adj_scale(ui, s4));
+                tail_add(g[3], adj_scale(ui, s3));
+                tail_add(g[4], adj_scale(ui, s4));
                 if (lane == 0) {
 #pragma unroll
-                    for (int k = 0; k < 3; ++k) adj_add(g[k], adj_prod(ui, r[row], L.d[3 * static_cast<size_t>(row) + k]));
+                    for (int k = 0; k < 3; ++k) tail_add(g[k], adj_prod(ui, r[row], L.d[3 * static_cast<size_t>(row) + k]));
                 }
             }
             acc = tt_group_sum(acc, tpr);
