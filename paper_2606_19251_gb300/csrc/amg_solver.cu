@@ -1593,21 +1593,34 @@ static DevTail *tail_of(amg_ctx *c) {
     return t->level >= 0 ? t : nullptr;
 }
 
-// First level of the tail: at most kTailRows rows, at least one smoothed
-// level in it, its level vectors within a CTA's shared memory and the
-// coarsest solves of its columns affordable; -1 if there is none.
-static int tail_level(const amg_ctx *c) {
+// First level of a tail: at most kTailRows rows, at least one smoothed level
+// in it, its level vectors within a CTA's shared memory, the coarsest solves
+// of its columns affordable and n_t x its levels' entries (the work of forming
+// B) at most `work`; -1 if there is none.
+static int tail_level(const amg_ctx *c, double work) {
     const int nlev = static_cast<int>(c->host.size());
     const double nL = c->host.back().A.n_rows;
     size_t rows = nL;
+    double entries = static_cast<double>(c->host.back().A.nnz());
     int best = -1;
     for (int l = nlev - 2; l >= 0 && nlev - l <= kTailMaxLevels; --l) {
         const int n = c->host[l].A.n_rows;
         rows += n;
-        if (n > kTailRows || 3 * rows * kTailCols * sizeof(double) > kTailSmem || n * nL * nL > kTailCoarseWork) break;
+        entries += static_cast<double>(c->host[l].A.nnz());
+        if (n > kTailRows || 3 * rows * kTailCols * sizeof(double) > kTailSmem || n * nL * nL > kTailCoarseWork ||
+            n * entries > work)
+            break;
         best = l;
     }
     return best;
+}
+
+static void set_tail_level(const amg_ctx *c, DevTail &t, int level) {
+    t.level = level;
+    t.ok = false;
+    if (level < 0) return;
+    const size_t tb = c->opt.precision == AMG_FP64 ? sizeof(double) : sizeof(float);
+    t.ld = static_cast<int>((c->host[level].A.n_rows * tb + 511) / 512 * 512 / tb);
 }
 
 template <class T>
@@ -1638,16 +1651,22 @@ static int build_tail(amg_ctx *c, int sm, cudaStream_t s) {
     }
     using V = typename TailValue<T>::type;
     const size_t smem = static_cast<size_t>(off) * sizeof(V);
-    CK(cudaFuncSetAttribute(k_tail_build<T, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kTailSmem)));
-    k_tail_build<T, V><<<(c->lev[t.level].n + kTailCols - 1) / kTailCols, kTailThreads, smem, s>>>(a); AMG_COUNT();
+    const DevLevel &L0 = c->lev[t.level];
+    auto kernel = k_tail_build<T, V, 4>;
+    if constexpr (sizeof(T) == 8)
+        if (L0.A.nnz < kTailLongRows * L0.n) kernel = k_tail_build<T, V, 1>;
+    CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kTailSmem)));
+    kernel<<<(L0.n + kTailCols - 1) / kTailCols, kTailThreads, smem, s>>>(a); AMG_COUNT();
     CKL("V-cycle tail");
     t.ok = true;
     return AMG_OK;
 }
 
 // Make the tail of the smoother in use current before V-cycles on s.  The
-// smoother's values change with the coefficients; B is re-formed at the next
-// V-cycle that needs it (or with host-given coefficients, in that call).
+// smoother's values change with the coefficients or omega; B is re-formed by
+// the next V-cycle or solve (Jacobi's first one with the hierarchy), so that a
+// call that only sets values pays for none (amg_set_coeffs on 9k rows 337 us
+// with B and its wait in it, 35 without; amg_set_jacobi 222 and 34).
 static int ensure_tail(amg_ctx *c, cudaStream_t s) {
     c->use_tail = true;
     DevTail *t = tail_of(c);
@@ -2155,15 +2174,17 @@ static void layout(amg_ctx *c, Planner &pl) {
     // stretched meshes bring smoothers to the edge of convergence, where a
     // stationary iteration amplifies any change of rounding, so there the
     // cycle keeps its level-by-level rounding.
-    const int tl = c->lev[0].A.stream ? -1 : tail_level(c);
-    for (DevTail &t : c->tail) {
+    // Jacobi's B is formed once, with the hierarchy, the pseudo-inverse's with
+    // every coefficient set.
+    const bool tail = !c->lev[0].A.stream;
+    const int small = tail ? tail_level(c, c->opt.precision == AMG_FP64 ? kTailWork64 : kTailWork) : -1;
+    for (int sm = 0; sm < 2; ++sm) {
+        DevTail &t = c->tail[sm];
         t = DevTail{};
-        if (tl < 0) continue;
-        const int n = c->host[tl].A.n_rows;
-        const size_t tb = c->opt.precision == AMG_FP64 ? sizeof(double) : sizeof(float);
-        t.level = tl;
-        t.ld = static_cast<int>((n * tb + 511) / 512 * 512 / tb);
-        t.B = pl.take<char>(sizeof(double) * n * t.ld);   // FP64, or FP32 pairs
+        t.small = small;
+        set_tail_level(c, t, sm == 0 && tail ? tail_level(c, INFINITY) : small);
+        if (t.level >= 0)   // FP64, or FP32 pairs
+            t.B = pl.take<char>(sizeof(double) * c->host[t.level].A.n_rows * t.ld);
     }
     const int n0 = c->host[0].A.n_rows;
     c->ell_ptr = pl.take<int>(c->h_ell_ptr.size());
@@ -2551,16 +2572,21 @@ int amg_set_jacobi(amg_ctx *c, double omega) {
     if (!std::isfinite(omega)) return ctx_fail(c, "omega not finite"), AMG_ERR_ARG;
     CK(cudaSetDevice(c->opt.device));
     if (omega != c->jac_omega) {
+        c->tail[0].ok = false;
         for (auto &L : c->lev) {
             k_jacobi_vals<<<grid_for(L.n), kBlock, 0, c->stream>>>(L.n, L.diag, omega, L.j64, L.j32); AMG_COUNT();
         }
         CKL("jacobi values");
-        c->tail[0].ok = false;
-        c->jac_omega = omega;
-        c->smoother = AMG_SMOOTHER_JACOBI;
-        const int rc = ensure_tail(c, c->stream);
-        if (rc) return rc;
         CK(cudaStreamSynchronize(c->stream));
+        // re-formed by the next V-cycle, within the work that new values may
+        // cost: an omega that was changed once may be changed again
+        DevTail &t = c->tail[0];
+        if (t.level != t.small) {                  // the captured graphs hold the tail's level
+            for (int o = 0; o < 2; ++o) free_graph(c->sgraph[AMG_SMOOTHER_JACOBI + 3 * o]);
+            free_vgraph(c->vgraph[AMG_SMOOTHER_JACOBI]);
+        }
+        set_tail_level(c, t, t.small);
+        c->jac_omega = omega;
     }
     c->smoother = AMG_SMOOTHER_JACOBI;
     return AMG_OK;
@@ -2689,7 +2715,7 @@ int set_coeffs_device(amg_ctx *c, const double *coef, cudaStream_t s, bool sync)
     }
     c->q_nodes = false;
     c->q64_stale = false;
-    c->tail[1].ok = false;
+    c->tail[1].ok = false;                         // re-formed by the next V-cycle
     CKL("assemble pseudo-inverse");
     // the solve kernels fetch matrix values ahead of their grid-dependency
     // wait: finish writing them before any of those kernels is launched (a
@@ -2710,11 +2736,7 @@ int amg_set_coeffs(amg_ctx *c, const double *coef, int n_rows) {
     if (!coef || n_rows < static_cast<int>(c->lev.size()) - 1)
         return ctx_fail(c, "need one coefficient row per smoothed level"), AMG_ERR_ARG;
     CK(cudaSetDevice(c->opt.device));
-    int rc = set_coeffs_device(c, coef, c->stream, true);
-    if (!rc) rc = ensure_tail(c, c->stream);
-    if (rc) return rc;
-    CK(cudaStreamSynchronize(c->stream));
-    return AMG_OK;
+    return set_coeffs_device(c, coef, c->stream, true);
 }
 
 int amg_set_node_coeffs(amg_ctx *c, const double *coef, long long n_values) {
@@ -2738,6 +2760,7 @@ int amg_set_node_coeffs(amg_ctx *c, const double *coef, long long n_values) {
     }
     double *d_c = nullptr;
     CK(cudaMalloc(&d_c, sizeof(double) * need));
+    c->tail[1].ok = false;                         // re-formed by the next V-cycle
     cudaError_t e = cudaMemcpyAsync(d_c, coef, sizeof(double) * need, cudaMemcpyHostToDevice, s);
     long long off = 0;
     for (int l = 0; l < nlev - 1 && e == cudaSuccess; ++l) {
@@ -2759,11 +2782,7 @@ int amg_set_node_coeffs(amg_ctx *c, const double *coef, long long n_values) {
     c->have_q = true;
     c->q_nodes = true;   // the wavefront chains read the stored values
     c->q64_stale = false;
-    c->tail[1].ok = false;
     c->smoother = AMG_SMOOTHER_GNN;
-    const int rc = ensure_tail(c, s);
-    if (rc) return rc;
-    CK(cudaStreamSynchronize(s));
     return AMG_OK;
 }
 

@@ -64,6 +64,7 @@ struct WfPlan {
 // Dense operator of the V-cycle's coarse tail (tail.cuh) for one smoother.
 struct DevTail {
     int level = -1;                            // first level of the tail, or -1
+    int small = -1;                            // the same within the work that new values may cost (kTailWork)
     int ld = 0;                                // row stride of B (entries)
     void *B = nullptr;                         // FP64, or high and low words of FP32 pairs (FP32 V-cycle)
     bool ok = false;                           // B belongs to the smoother's current values

@@ -6,13 +6,18 @@
 // of that chain is one launch of a few microseconds whose only cost is its
 // dependent load chain, so B (n_t x n_t) is formed once per smoother and
 // applied as one matrix-vector product instead of 7 launches per level.
-// Measured on GB300 (per pass, before -> after): one V-cycle on 9k / 280k
-// unstructured rows 71 -> 52 / 173 -> 138 us, on a 1025^2 grid (Jacobi)
-// 209 -> 186 us; a whole FP64 solve on a 64^2 grid 926 -> 681 us; prediction
-// and solve on the 50k mesh 4.43 -> 3.60 ms with B re-formed in every pass.
+// Measured on GB300 (per pass, levels one by one -> with the tail): one V-cycle
+// launched kernel by kernel on 9k / 280k unstructured rows 71 -> 52 / 173 ->
+// 138 us, on a 1025^2 grid (Jacobi) 209 -> 186 us; a whole FP64 solve on a 64^2
+// grid 926 -> 681 us; prediction and solve on the 50k mesh 4.43 -> 3.60 ms with
+// B re-formed in every pass.  What forming B costs, and where the tail of a
+// pseudo-inverse may start for it: kTailWork.
 //
 // The coarsest solve of an FP32 V-cycle is FP64, so B is held and applied in
-// FP32 pairs (about 48 bits) and e is rounded once: PRECISION_FIGURES
+// FP32 pairs (about 48 bits) and e is rounded once.  V-cycle error against
+// 64 bits, geometric mean of nine meshes, both smoothers and four or eight
+// seeds each, relative to the levels one by one: 1.01, with B in FP32 and FP32
+// sums 1.04.  The pairs cost 0 to 1.5 us a V-cycle (280k rows 136.2 -> 137.7).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -20,15 +25,30 @@
 
 namespace amg {
 
-// Largest level a tail starts on: at 1024 rows B is 4 MB (FP32), 27 KB an SM.
-// Forming it costs n_t times the tail's entries: the next RS level (about 2300
-// rows) would take five times the memory and the work, in every call that has
-// new coefficients.
+// Largest level a tail starts on: at 1024 rows B is 8 MB, 54 KB an SM.  The
+// next RS level (about 2300 rows) would take five times the memory and the
+// work.
 constexpr int kTailRows = 1024;
 constexpr int kTailMaxLevels = 16;     // levels of a tail (kernel argument arrays)
 constexpr int kTailCols = 4;           // columns of B a CTA forms at a time
-constexpr int kTailThreads = 512;
+constexpr int kTailThreads = 1024;
 constexpr size_t kTailSmem = 220 * 1024;         // shared memory a tail's level vectors may take
+// Bound of n_t x (entries of the tail's levels) where B is formed again with
+// new values, in the first V-cycle or solve after them: always for the
+// pseudo-inverse, for Jacobi after a change of omega.  The work is 8 passes
+// over those entries for n_t columns (4 with Jacobi).  Measured, the
+// pseudo-inverse's B: 280 rows, n_t x entries 1.3e6, 42 us; 513 rows, 3.0e6, 67
+// us; 978 rows, 15.6e6, 220 us (FP64 409); 525 rows of a 3-D mesh, 18.7e6, 182 us
+// (463).  Against that stand 5 to 10 us a V-cycle for a level of 500 to 1000
+// rows more in the tail: it pays after 25 to 35 V-cycles, more than a solve with
+// conjugate gradients takes.  Within the bounds amg_set_coeffs and a prediction
+// with 0, 1, 2, ... V-cycles after them take no longer than with the levels one
+// by one (9k rows, amg_set_coeffs and one V-cycle: 139 us one by one, 381 with
+// the tail from 978 rows, 126 from 231 rows; FP64 168, 525, 167).  Jacobi's B
+// is formed with the hierarchy, where 0.1 to 0.3 ms stand beside 5 to 50 ms of
+// setup, and is not bounded there.
+constexpr double kTailWork = 4e6, kTailWork64 = 1.5e6;
+constexpr int kTailLongRows = 32;      // FP64: four lanes a row from this mean length on
 constexpr double kTailCoarseWork = 134217728.0;  // n_t n_L^2 bound: the FP64 coarsest solves of the n_t columns
 
 // The FP32 V-cycle's B is formed in FP32 pairs (FloatPair): GB300 runs 64
@@ -96,53 +116,95 @@ template <class T> struct TailArgs {
     T *B;                       // n_t rows of ld entries (FP32: the low words n_t ld entries behind)
 };
 
-// acc[c] = (NEG ? -1 : 1) sum_k m_ik x_kc of one CSR row and kTailCols columns
-template <bool NEG, class T, class V>
-__device__ __forceinline__ void tail_row(const TailCsr<T> &M, int row, const V *__restrict__ x, V (&acc)[kTailCols]) {
-    const int e = __ldg(M.rp + row + 1);
-    for (int p = __ldg(M.rp + row); p < e; p += 4) {
-        int c[4];
-        T v[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            c[j] = p + j < e ? __ldg(M.col + p + j) : 0;
-            v[j] = p + j < e ? __ldg(M.val + p + j) : T(0);
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            if (p + j >= e) break;
-            const T a = NEG ? -v[j] : v[j];
-#pragma unroll
-            for (int k = 0; k < kTailCols; ++k) tail_fma(acc[k], a, x[c[j] * kTailCols + k]);
-        }
-    }
+// Column g = tid % 4 of the sum over the row's four lanes (each holds its
+// share of every column).
+template <class V>
+__device__ __forceinline__ V tail_scatter(const V (&acc)[kTailCols], int g) {
+    static_assert(kTailCols == 4, "two exchange steps");
+    const bool hi = g & 2;
+    V a = hi ? acc[2] : acc[0], b = hi ? acc[3] : acc[1];
+    tail_add(a, tail_shfl(hi ? acc[0] : acc[2], 2));
+    tail_add(b, tail_shfl(hi ? acc[1] : acc[3], 2));
+    const bool odd = g & 1;
+    V s = odd ? b : a;
+    tail_add(s, tail_shfl(odd ? a : b, 1));
+    return s;
 }
 
-// One smoothing sweep u += M (b - A u) on a level's columns (all threads).
-template <class T, class V>
-__device__ void tail_sweep(const TailLevel<T> &L, int pinv, const V *b, V *u, V *r) {
-    for (int i = threadIdx.x; i < L.n; i += kTailThreads) {
+// f(k, M x at k) for every entry k = row kTailCols + column: LANES (1 or 4)
+// lanes share a row's entries; of four, each then takes one column.
+template <int LANES, class T, class V, class F>
+__device__ __forceinline__ void tail_rows(int n, const TailCsr<T> &M, const V *x, const F &f) {
+    struct alignas(16) Two { V a, b; };      // 16-byte loads: a level's vectors start at multiples of kTailCols
+    const int g = threadIdx.x % LANES;
+    for (int base = 0; base < n; base += kTailThreads / LANES) {
+        const int row = base + static_cast<int>(threadIdx.x) / LANES;
         V acc[kTailCols];
 #pragma unroll
-        for (int k = 0; k < kTailCols; ++k) acc[k] = b[i * kTailCols + k];
-        tail_row<true>(L.A, i, u, acc);
+        for (int k = 0; k < kTailCols; ++k) tail_set(acc[k], 0.0);
+        if (row < n) {
+            const int e = __ldg(M.rp + row + 1);
+            for (int p0 = __ldg(M.rp + row) + g; p0 < e; p0 += 4 * LANES) {
+                int c[4];
+                T v[4];
 #pragma unroll
-        for (int k = 0; k < kTailCols; ++k) r[i * kTailCols + k] = tail_norm(acc[k]);
+                for (int j = 0; j < 4; ++j) {
+                    const int p = p0 + j * LANES;
+                    c[j] = p < e ? __ldg(M.col + p) : 0;
+                    v[j] = p < e ? __ldg(M.val + p) : T(0);
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (p0 + j * LANES >= e) break;
+                    const Two *xr = reinterpret_cast<const Two *>(x + c[j] * kTailCols);
+                    const Two lo = xr[0], hi = xr[1];
+                    tail_fma(acc[0], v[j], lo.a);
+                    tail_fma(acc[1], v[j], lo.b);
+                    tail_fma(acc[2], v[j], hi.a);
+                    tail_fma(acc[3], v[j], hi.b);
+                }
+            }
+        }
+        if constexpr (LANES == 1) {
+            if (row < n) {
+#pragma unroll
+                for (int k = 0; k < kTailCols; ++k) f(row * kTailCols + k, acc[k]);
+            }
+        } else {
+            const V s = tail_scatter(acc, g);
+            if (row < n) f(row * kTailCols + g, s);
+        }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < L.n; i += kTailThreads) {
-        V acc[kTailCols];
-#pragma unroll
-        for (int k = 0; k < kTailCols; ++k) acc[k] = u[i * kTailCols + k];
-        if (pinv) {
-            tail_row<false>(TailCsr<T>{L.A.rp, L.A.col, L.m}, i, r, acc);
-        } else {
-            const T j = L.m[i];
-#pragma unroll
-            for (int k = 0; k < kTailCols; ++k) tail_fma(acc[k], j, r[i * kTailCols + k]);
-        }
-#pragma unroll
-        for (int k = 0; k < kTailCols; ++k) u[i * kTailCols + k] = tail_norm(acc[k]);
+}
+
+// y = y + s with s negated on demand, renormalised
+__device__ __forceinline__ FloatPair tail_sum(FloatPair y, const FloatPair &s, bool neg = false) {
+    if (neg) pair_add(y, -s.h, -s.l);
+    else pair_add(y, s.h, s.l);
+    return tail_norm(y);
+}
+__device__ __forceinline__ double tail_sum(double y, double s, bool neg = false) { return neg ? y - s : y + s; }
+
+// r = b - A u
+template <int LANES, class T, class V>
+__device__ __forceinline__ void tail_resid(const TailLevel<T> &L, const V *b, const V *u, V *r) {
+    tail_rows<LANES>(L.n, L.A, u, [&](int k, const V &s) { r[k] = tail_sum(b[k], s, true); });
+}
+
+// u = (add ? u : 0) + M r
+template <int LANES, class T, class V>
+__device__ __forceinline__ void tail_smooth(const TailLevel<T> &L, int pinv, const V *r, V *u, bool add) {
+    V zero;
+    tail_set(zero, 0.0);
+    if (pinv) {
+        tail_rows<LANES>(L.n, TailCsr<T>{L.A.rp, L.A.col, L.m}, r, [&](int k, const V &s) { u[k] = tail_sum(add ? u[k] : zero, s); });
+        return;
+    }
+    for (int k = threadIdx.x; k < L.n * kTailCols; k += kTailThreads) {
+        V acc = add ? u[k] : zero;
+        tail_fma(acc, __ldg(L.m + k / kTailCols), r[k]);
+        u[k] = tail_norm(acc);
     }
     __syncthreads();
 }
@@ -151,7 +213,13 @@ __device__ void tail_sweep(const TailLevel<T> &L, int pinv, const V *b, V *u, V 
 // vectors, every level's b, u, r for those columns in shared memory, so one
 // launch forms B without grid-wide steps (each CTA re-reads the levels'
 // matrices from L2).  Dynamic shared memory: 3 sum_l n_l kTailCols values.
-template <class T, class V>
+// A step's time is its longest row's (coarse rows have 10 to 100 entries), so
+// with FP32 pairs four lanes share a row and exchange their columns' sums at
+// its end (one thread a row: 978 rows 285 -> 220 us, 525 rows of 60 entries 431
+// -> 182, 280 rows 56 -> 42).  In FP64 the exchange costs as much of the narrow
+// FP64 unit as a short row (978 rows of 13 entries 409 -> 509 us), so there four
+// lanes take rows of kTailLongRows entries on average (525 rows 637 -> 463).
+template <class T, class V, int LANES>
 __global__ void __launch_bounds__(kTailThreads) k_tail_build(const __grid_constant__ TailArgs<T> A) {
     extern __shared__ __align__(16) unsigned char tail_smem[];
     V *sm = reinterpret_cast<V *>(tail_smem);
@@ -169,42 +237,19 @@ __global__ void __launch_bounds__(kTailThreads) k_tail_build(const __grid_consta
     for (int l = 0; l < last; ++l) {
         const TailLevel<T> &L = A.lev[l];
         V *b = sm + L.off, *u = b + L.n * kTailCols, *r = u + L.n * kTailCols;
-        for (int i = threadIdx.x; i < L.n; i += kTailThreads) {   // first sweep from zero: u = M b
-            V acc[kTailCols];
-#pragma unroll
-            for (int k = 0; k < kTailCols; ++k) acc[k] = zero;
-            if (A.nu1 > 0 && A.pinv) {
-                tail_row<false>(TailCsr<T>{L.A.rp, L.A.col, L.m}, i, b, acc);
-            } else if (A.nu1 > 0) {
-                const T j = L.m[i];
-#pragma unroll
-                for (int k = 0; k < kTailCols; ++k) tail_fma(acc[k], j, b[i * kTailCols + k]);
-            }
-#pragma unroll
-            for (int k = 0; k < kTailCols; ++k) u[i * kTailCols + k] = tail_norm(acc[k]);
+        if (A.nu1 > 0) {
+            tail_smooth<LANES>(L, A.pinv, b, u, false);                      // first sweep from zero: u = M b
+        } else {
+            for (int k = threadIdx.x; k < L.n * kTailCols; k += kTailThreads) u[k] = zero;
+            __syncthreads();
         }
-        __syncthreads();
-        for (int s = 1; s < A.nu1; ++s) tail_sweep<T, V>(L, A.pinv, b, u, r);
-        for (int i = threadIdx.x; i < L.n; i += kTailThreads) {   // r = b - A u
-            V acc[kTailCols];
-#pragma unroll
-            for (int k = 0; k < kTailCols; ++k) acc[k] = b[i * kTailCols + k];
-            tail_row<true>(L.A, i, u, acc);
-#pragma unroll
-            for (int k = 0; k < kTailCols; ++k) r[i * kTailCols + k] = tail_norm(acc[k]);
+        for (int s = 1; s < A.nu1; ++s) {
+            tail_resid<LANES>(L, b, u, r);
+            tail_smooth<LANES>(L, A.pinv, r, u, true);
         }
-        __syncthreads();
-        const TailLevel<T> &C = A.lev[l + 1];
-        V *bc = sm + C.off;
-        for (int i = threadIdx.x; i < C.n; i += kTailThreads) {   // b_{l+1} = R r
-            V acc[kTailCols];
-#pragma unroll
-            for (int k = 0; k < kTailCols; ++k) acc[k] = zero;
-            tail_row<false>(L.R, i, r, acc);
-#pragma unroll
-            for (int k = 0; k < kTailCols; ++k) bc[i * kTailCols + k] = tail_norm(acc[k]);
-        }
-        __syncthreads();
+        tail_resid<LANES>(L, b, u, r);
+        V *bc = sm + A.lev[l + 1].off;
+        tail_rows<LANES>(A.lev[l + 1].n, L.R, r, [&](int k, const V &s) { bc[k] = tail_norm(s); });
     }
     {   // coarsest level: u = L^-T (L^-1 b) in FP64; y is kept in r as doubles
         const int n = A.lev[last].n;
@@ -212,18 +257,28 @@ __global__ void __launch_bounds__(kTailThreads) k_tail_build(const __grid_consta
         V *u = sm + A.lev[last].off + n * kTailCols;
         static_assert(sizeof(V) == sizeof(double), "y shares r's storage");
         double *y = reinterpret_cast<double *>(u + n * kTailCols);
-        for (int e = threadIdx.x; e < n * kTailCols; e += kTailThreads) {
-            const int i = e / kTailCols, k = e % kTailCols;
+        // a warp's lanes take 32 / kTailCols terms of a row and its columns
+        constexpr int kParts = 32 / kTailCols;
+        const int k = threadIdx.x % kTailCols, part = threadIdx.x % 32 / kTailCols;
+        auto total = [&](double v) {
+#pragma unroll
+            for (int o = kTailCols; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            return v;
+        };
+        for (int i = threadIdx.x / 32; i < n; i += kTailThreads / 32) {
+            const double *row = A.Linv + static_cast<size_t>(i) * n;
             double acc = 0.0;
-            for (int q = 0; q <= i; ++q) acc = fma(A.Linv[static_cast<size_t>(i) * n + q], tail_get(b[q * kTailCols + k]), acc);
-            y[e] = acc;
+            for (int q = part; q <= i; q += kParts) acc = fma(row[q], tail_get(b[q * kTailCols + k]), acc);
+            acc = total(acc);
+            if (part == 0) y[i * kTailCols + k] = acc;
         }
         __syncthreads();
-        for (int e = threadIdx.x; e < n * kTailCols; e += kTailThreads) {
-            const int i = e / kTailCols, k = e % kTailCols;
+        for (int i = threadIdx.x / 32; i < n; i += kTailThreads / 32) {
+            const double *row = A.LinvT + static_cast<size_t>(i) * n;
             double acc = 0.0;
-            for (int q = i; q < n; ++q) acc = fma(A.LinvT[static_cast<size_t>(i) * n + q], y[q * kTailCols + k], acc);
-            tail_set(u[e], acc);
+            for (int q = i + part; q < n; q += kParts) acc = fma(row[q], y[q * kTailCols + k], acc);
+            acc = total(acc);
+            if (part == 0) tail_set(u[i * kTailCols + k], acc);
         }
         __syncthreads();
     }
@@ -231,16 +286,11 @@ __global__ void __launch_bounds__(kTailThreads) k_tail_build(const __grid_consta
         const TailLevel<T> &L = A.lev[l];
         V *b = sm + L.off, *u = b + L.n * kTailCols, *r = u + L.n * kTailCols;
         const V *e = sm + A.lev[l + 1].off + A.lev[l + 1].n * kTailCols;
-        for (int i = threadIdx.x; i < L.n; i += kTailThreads) {   // u += P e
-            V acc[kTailCols];
-#pragma unroll
-            for (int k = 0; k < kTailCols; ++k) acc[k] = u[i * kTailCols + k];
-            tail_row<false>(L.P, i, e, acc);
-#pragma unroll
-            for (int k = 0; k < kTailCols; ++k) u[i * kTailCols + k] = tail_norm(acc[k]);
+        tail_rows<LANES>(L.n, L.P, e, [&](int k, const V &s) { u[k] = tail_sum(u[k], s); });
+        for (int s = 0; s < A.nu2; ++s) {
+            tail_resid<LANES>(L, b, u, r);
+            tail_smooth<LANES>(L, A.pinv, r, u, true);
         }
-        __syncthreads();
-        for (int s = 0; s < A.nu2; ++s) tail_sweep<T, V>(L, A.pinv, b, u, r);
     }
     const V *u = sm + A.lev[0].off + nt * kTailCols;
     for (int e = threadIdx.x; e < nt * kTailCols; e += kTailThreads) {
