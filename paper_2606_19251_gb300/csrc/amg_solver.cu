@@ -1882,13 +1882,21 @@ static void free_vgraph(VcycleGraph &G) {
 }
 
 // One V-cycle on lev[0].vb for amg_vcycle_device; returns the result's
-// buffer.  A caller's Krylov loop repeats it, and as single launches it is
-// bound by the host (1.35 us each on a Grace core, against 0.6 to 0.9 us per
-// dependent kernel of a graph and 1 us for launching one): from the second
-// call on it is one graph launch (9k rows: 50.6 -> 34.4 us a call; 280k rows,
-// bound by the device, 137.4 -> 135.3).  The first call launches the kernels, so a
-// V-cycle that is not repeated pays for no capture; so does a caller's own
-// capture (use_tail is off), and a capture that fails leaves the kernels.
+// buffer.  A caller's Krylov loop repeats it, and as single launches back to
+// back it is bound by the host (1.35 us each on a Grace core, against 0.6 to
+// 0.9 us per dependent kernel of a graph and 1 us for launching one), so after
+// a while it becomes one graph launch (9k rows, before the pseudo-inverse's
+// tail was bounded: 50.6 -> 34.4 us a call; 280k rows, bound by the device,
+// 137.4 -> 135.3).  A caller that waits for each call gains less (45 -> 43 and
+// 99 -> 91 us) and capturing and instantiating cost 85 (4k rows) to 190 us
+// (1M rows) once per hierarchy and smoother.  By the twelfth call the V-cycles
+// before it have saved that against the levels one by one on every mesh
+// measured (4k to 1M rows), so that no number of calls takes longer than it did
+// there; captured at the second call, two to eight calls did (50k rows, two
+// calls: 211 us one by one, 362 with the capture in the second, 214 without).
+// A caller's own capture takes none (use_tail is off), and a capture that
+// fails leaves the kernels.
+constexpr int kVcycleCaptureCall = 12;
 template <class T>
 static T *vcycle_repeat(amg_ctx *c, cudaStream_t s) {
     VcycleGraph &G = c->vgraph[c->smoother];
@@ -1899,7 +1907,7 @@ static T *vcycle_repeat(amg_ctx *c, cudaStream_t s) {
     }
     if (!c->use_tail || c->opt.fused_sweeps) return vcycle_level<T>(c, 0, s);
     if (!G.exec) {
-        if (++G.calls != 2) return vcycle_level<T>(c, 0, s);
+        if (++G.calls != kVcycleCaptureCall) return vcycle_level<T>(c, 0, s);
         // another stream of this thread may be under capture: ours must not disturb it
         cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
         cudaThreadExchangeStreamCaptureMode(&mode);
@@ -3978,12 +3986,15 @@ void loss_enqueue(amg_ctx *c, TrainBufs &tb, int nvc, cudaStream_t s) {
 }
 
 // Training calls a problem once per epoch with new coefficients: from the
-// second call with the same number of cycles on, its 300 to 400 kernels are
-// one graph launch.  12k-row mesh, three cycles: 2341 us a call with five
-// launches per adjoint sweep and a host step for the loss, 1235 us with the
-// fused passes launched singly (a first call), 1011 us as a graph, 749 us
-// with the gradient's sums in FP32 pairs (k_adj_sweep), 711 us with the levels
-// of up to 256 rows in one CTA (train_tail.cuh).
+// second call with the same number of cycles on, its kernels (about 230 on a
+// 12k-row mesh with three cycles) are one graph launch.  That mesh: 2341 us a
+// call with five launches per adjoint sweep and a host step for the loss, 1235
+// us with the fused passes launched singly, 1011 us as a graph, 749 us with the
+// gradient's sums in FP32 pairs (k_adj_sweep), 711 us with the levels of up to
+// 256 rows in one CTA (train_tail.cuh).  The first three calls of a context
+// take 1050 us (buffers and single launches), 1640 (capture) and 640.  The
+// graph holds one number of cycles: a caller that alternates between two stays
+// with single launches.
 template <class T>
 int loss_grad(amg_ctx *c, TrainBufs &tb, const double *f, int nvc, double *loss, double *dc) {
     cudaStream_t s = c->stream;

@@ -113,8 +113,8 @@ struct SolveGraph {
     int q_nodes = -1;    // the pseudo-inverse source the captured chains use
 };
 
-// One V-cycle of amg_vcycle_device as a CUDA graph, captured at the second
-// call with the same hierarchy and smoother.
+// One V-cycle of amg_vcycle_device as a CUDA graph, captured once the calls
+// with the same hierarchy and smoother have paid for it (vcycle_repeat).
 struct VcycleGraph {
     cudaGraphExec_t exec = nullptr;
     long long version = -1;
