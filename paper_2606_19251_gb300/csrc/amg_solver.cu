@@ -2070,13 +2070,26 @@ static void layout_mat(Planner &pl, DevMat &m, const HostCSR &h) {
 }
 
 // A level streams from HBM when the values of A and Q^-1, their columns and
-// four vectors are a quarter more than the 129 MB of L2.  Measured (evict-first
-// values on / off): 2.5M rows (210 MB) residual 27.9 / 32.9 us, Q^-1 pass 26.0
-// / 32.7; 1.1M rows (138 MB) 19.8 / 20.1 and 20.2 / 19.0; 1M rows of a 5-point
-// grid (68 MB) 9.0 / 7.5, so below the line the values are left to L2.  With
-// the row's own values loaded early (load_now) and the policy made once the
-// 2.5M-row passes take 24.4 and 23.7 us, a V-cycle there 604 instead of 682.
+// four vectors pass the 129 MB of L2.  V-cycles with evict-first values and
+// alternating row order on every two-pass level / on none, by these bytes of
+// the finest level: 99 to 111 MB 1.05 to 1.13 times slower (Jacobi and the
+// pseudo-inverse), 128 MB 1.10, 132 MB 0.96 to 0.985, 144 MB 0.95 to 0.985, 170
+// MB 0.91 to 0.97, 213 MB 0.94 to 0.965, and 0.99 to 1.00 with an FP64 V-cycle
+// past the line.  Jacobi and Chebyshev read A alone, but their line lies at the
+// same bytes (5-point grid of 2M rows, 132 MB with Q^-1 and 92 without: Jacobi
+// 286 / 291 us, Chebyshev 402 / 424).  2.5M rows: residual pass 24.4 / 32.9 us,
+// Q^-1 pass 23.7 / 32.7.
 constexpr double kStreamBytes = 129e6;
+
+// Largest finest level (bytes of A and Q^-1 in FP32, as above) with an FP32
+// tail.  The rule is on accuracy alone and size stands in for it: the learned
+// smoother stagnates on the largest stretched meshes (four of twelve 2.5M-row
+// meshes with cells of 1000:1), a stationary iteration that does not converge
+// carries every change of FP32 rounding into its iterates (1e-6 there, 1e-12
+// where it converges), and these cycles keep the rounding of the levels one by
+// one.  They give up 7 % of a V-cycle for it (2.5M rows, a tail from 1024 rows:
+// 633 -> 591 us).  An FP64 V-cycle's rounding is far below that: no bound.
+constexpr double kTailFinest = 129e6;
 
 // Warp slices of the finest level's FP64 operator (see Ell64): rows sorted
 // by length, longest first, within windows of kEllWindow rows (stable, so
@@ -2177,15 +2190,11 @@ static void layout(amg_ctx *c, Planner &pl) {
     c->Ldense = pl.take<double>(static_cast<size_t>(nL) * nL);
     c->Linv = pl.take<double>(static_cast<size_t>(nL) * nL);
     c->LinvT = pl.take<double>(static_cast<size_t>(nL) * nL);
-    // Not where the finest level streams from HBM: the tail is worth 7 % of
-    // such a cycle (2.5M rows: 633 us without, 591 us with), but the largest
-    // stretched meshes bring smoothers to the edge of convergence, where a
-    // stationary iteration amplifies any change of rounding, so there the
-    // cycle keeps its level-by-level rounding.
     // Jacobi's B is formed once, with the hierarchy, the pseudo-inverse's with
     // every coefficient set.
-    const bool tail = !c->lev[0].A.stream;
-    const int small = tail ? tail_level(c, c->opt.precision == AMG_FP64 ? kTailWork64 : kTailWork) : -1;
+    const bool fp64 = c->opt.precision == AMG_FP64;
+    const bool tail = fp64 || 10.0 * c->lev[0].A.nnz + 16.0 * c->lev[0].n <= kTailFinest;
+    const int small = tail ? tail_level(c, fp64 ? kTailWork64 : kTailWork) : -1;
     for (int sm = 0; sm < 2; ++sm) {
         DevTail &t = c->tail[sm];
         t = DevTail{};

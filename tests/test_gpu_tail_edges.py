@@ -97,6 +97,20 @@ def test_large_coarsest_level(rows, max_coarse, tail, prec, tol):
         P.amg_destroy(ctx)
 
 
+def test_fp64_tail_on_a_finest_level_past_l2():
+    """The bound on the finest level is one of FP32 rounding: an FP64 V-cycle has its tail there too."""
+    ctx = P.amg_create(precision=P.AMG_FP64)
+    try:
+        A = W.poisson5(1040)
+        P.amg_setup_device(ctx, A, 0, P.AMG_SPLIT_RS_BLOCKS)
+        P.amg_set_coeffs(ctx, np.tile(COEFFS, (P.amg_num_levels(ctx), 1)))
+        b = W.rhs_uniform(1, A.n_rows)
+        (e, first), (e2, n) = _v(ctx, b), _v(ctx, b)
+        assert first == n + 1 and np.array_equal(e, e2)
+    finally:
+        P.amg_destroy(ctx)
+
+
 def test_calls_that_set_values_form_no_operator():
     """amg_set_coeffs and amg_set_jacobi launch the assembly alone."""
     levels = OS.build_hierarchy(W.fv_mesh("graded", 3000, 3)[0], max_coarse=40)
