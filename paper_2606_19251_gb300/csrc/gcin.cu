@@ -427,56 +427,6 @@ __device__ __forceinline__ float4 agg_rows(int p0, int p1, const int *__restrict
     return h;
 }
 
-// The same sum with U gathers in flight a lane, whole batches predicated, and
-// the next chunk's (col, w) pairs loaded while this one is added: for the FP32
-// layer kernel, which has the registers (78 of 80) and is bound by the latency
-// of its gathers (110k-node 3-D graph, H = 32: prediction 519 -> 509 us).  The
-// tensor-core layer and the backward aggregation gain nothing from it.
-template <int H, int U>
-__device__ __forceinline__ float4 agg_rows_deep(int p0, int p1, const int *__restrict__ col, const float *__restrict__ w,
-                                                const float4 *__restrict__ x4, int hl) {
-    constexpr int L = H / 4;
-    static_assert(L % U == 0, "whole batches per chunk");
-    float4 h = make_float4(0.f, 0.f, 0.f, 0.f);
-    const int deg = p1 - p0;
-    int maxdeg = deg;
-#pragma unroll
-    for (int o = L; o < 32; o <<= 1) maxdeg = max(maxdeg, __shfl_xor_sync(0xffffffffu, maxdeg, o));
-    int cn = hl < deg ? col[p0 + hl] : 0;
-    float wn = hl < deg ? w[p0 + hl] : 0.f;
-    for (int base = 0; base < maxdeg; base += L) {
-        const int cj = cn;
-        const float wj = wn;
-        const int nx = base + L + hl;
-        if (nx < deg) {
-            cn = col[p0 + nx];
-            wn = w[p0 + nx];
-        }
-        const int cnt = deg - base;                  // entries of this row in the chunk (may be <= 0)
-        const int cmax = min(L, maxdeg - base);
-        for (int k = 0; k < cmax; k += U) {
-            float wk[U];
-            float4 v[U];
-#pragma unroll
-            for (int j = 0; j < U; ++j) {
-                const int c = __shfl_sync(0xffffffffu, cj, k + j, L);
-                wk[j] = __shfl_sync(0xffffffffu, wj, k + j, L);
-                v[j] = (k + j < cnt) ? x4[static_cast<size_t>(c) * L + hl] : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-#pragma unroll
-            for (int j = 0; j < U; ++j) {
-                if (k + j < cnt) {
-                    h.x = fmaf(wk[j], v[j].x, h.x);
-                    h.y = fmaf(wk[j], v[j].y, h.y);
-                    h.z = fmaf(wk[j], v[j].z, h.z);
-                    h.w = fmaf(wk[j], v[j].w, h.w);
-                }
-            }
-        }
-    }
-    return h;
-}
-
 // Layers 2..4: h = A_hat x (H features), y = h W + b; tile stats.
 template <int H>
 __global__ void __launch_bounds__(kBlock) k_agg_lin_tile(const int *__restrict__ rp, const int *__restrict__ col,
@@ -499,7 +449,7 @@ __global__ void __launch_bounds__(kBlock) k_agg_lin_tile(const int *__restrict__
         const bool live = k < nn;                    // the last rows of the last group may be absent
         const int i = a + (live ? k : k0);
         const int p0 = rp[i], p1 = live ? rp[i + 1] : p0;
-        const float4 hv = agg_rows_deep<H, 8>(p0, p1, col, w, x4, hl);
+        const float4 hv = agg_rows<H>(p0, p1, col, w, x4, hl);
         if (live && hout) reinterpret_cast<float4 *>(hout)[static_cast<size_t>(i) * L + hl] = hv;
         float4 yv = b4;
 #pragma unroll 4
