@@ -17,6 +17,10 @@
 // Sweep of relaxed Jacobi (Sec. 2.3): u' = u + omega D^-1 (b - A u).
 // Coarsest level: FP64 dense Cholesky factor L (setup), applied as
 // u = L^-T (L^-1 b) with L^-1 formed once at setup.
+// Coarse tail: on small levels the whole V-cycle from some level t down, with
+// that solve in it, is one dense operator, e = B b (tail.cuh); the Chebyshev
+// smoother, a caller's capture and very large FP32 hierarchies step through
+// the levels instead.
 // Outer loop (FP64): r = b - A x, ||r|| / ||b||, x += V(r).
 #include <cuda_runtime.h>
 
@@ -632,8 +636,8 @@ __global__ void __launch_bounds__(kBlock) k_solve_init(int n, const double *__re
 // ---------------------------------------------------------------------------
 // kernels: conjugate gradients preconditioned by one V-cycle (FP64)
 // ---------------------------------------------------------------------------
-// Fixed-order sum of np partials, computed identically by every block (so
-// each block derives the same alpha / beta without a separate launch).
+// Fixed-order sum of np partials, computed identically by every block (the
+// loss's seed: no launch stands between the partials and their use).
 __device__ __forceinline__ double sum_partials(const double *__restrict__ part, int np, double *red) {
     double v = 0.0;
     for (int i = threadIdx.x; i < np; i += kBlock) v += part[i];

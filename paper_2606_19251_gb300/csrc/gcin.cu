@@ -267,7 +267,8 @@ __device__ __forceinline__ uint2 bf16x4(float a, float b, float c, float d) {
 // sums with one addition each.  A thread owns one feature and keeps its column
 // of W, so y needs no shared memory; its two accumulators per statistic are
 // the groups of tile_stats.  1.95M nodes: 228 us with four lanes, y staged in
-// shared memory and W read per node (L1 pipe 84 %).
+// shared memory and W read per node (L1 pipe 84 %).  Twelve CTAs an SM leave
+// 40 registers, at which it spills 16 bytes a thread (28 read back).
 constexpr int kL1Threads = 2 * kTile;
 template <int H, bool YB = false>
 __global__ void __launch_bounds__(kL1Threads, 12) k_layer1_tile(const int *__restrict__ rp, const int *__restrict__ col,
@@ -556,7 +557,8 @@ __device__ __forceinline__ double lanes_total(int a, int e, FloatPair (*red)[H],
 // unrolled so that a thread's loads are in flight together.  With the
 // normalisation pass's and the head's reductions: prediction on 50k rows 363
 // -> 314 us and, with pairs here and in the pooling, 301 -> 263 us; on 1.2M rows
-// 2698 -> 2487 and 2235 -> 2114 us.
+// 2698 -> 2487 and 2235 -> 2114 us (the checks for sums past FP32's range: 4 us
+// on 50k, 11 on 1.2M rows).
 template <int H>
 __global__ void __launch_bounds__(kLanes * H) k_stats_combine(const int *__restrict__ gtile, const int *__restrict__ gptr,
                                                             const int *__restrict__ tstart,
@@ -597,7 +599,8 @@ __global__ void __launch_bounds__(kLanes * H) k_stats_combine(const int *__restr
 // 16-byte vectors (four features of a thread; as 8-byte FP64 values at a
 // stride of four they kept the L1 pipe at 85 to 94 %), and a feature's 16
 // sums are added as an FP32 pair (the 32 FP64 operations per feature and tile
-// were 100 us of a 1.95M-node pass).
+// were 100 us of a 1.95M-node pass).  Six CTAs an SM leave 40 registers: at
+// width 64 it spills 92 to 152 bytes a thread (184 to 244 read back).
 template <int H, int YM = 0>
 __global__ void __launch_bounds__(kBlock, 6) k_norm_relu_pool_tile(const int *__restrict__ tstart,
                                                                 const int *__restrict__ tgraph,
@@ -1569,7 +1572,7 @@ int gnn_predict_coeffs(amg_ctx *c, double *c_out) {
     g->batch.hidden = g->hidden;
     g->batch.wtile = g->wtile;
     // forward + smoother assembly (straight from the device coefficients) run
-    // as one CUDA graph, captured once per batch and arithmetic: ~40 small
+    // as one CUDA graph, captured once per batch and arithmetic: 28 small
     // kernels whose host launch cost would otherwise exceed their run time
     const int key = g->batch.bf16 + 2 * c->opt.precision + 4 * (g->hidden == kHidden32 ? 1 : 0);
     if (!g->exec || g->exec_version != g->batch_version || g->exec_key != key) {

@@ -222,7 +222,8 @@ __global__ void __launch_bounds__(kBlock) k_pack_wtile(const float *__restrict__
 }
 
 // XB (inference): x rows are bfloat16 (8 features per lane), the B tile comes
-// pre-packed from wt, and no h is kept.
+// pre-packed from wt, and no h is kept.  Four CTAs an SM leave 64 registers,
+// at which width 64 spills 16 bytes a thread.
 template <int H, bool XB = false>
 __global__ void __launch_bounds__(kBlock, 4) k_agg_lin_tc(const int *__restrict__ rp, const int *__restrict__ col,
                                                        const float *__restrict__ w, const void *__restrict__ xin,

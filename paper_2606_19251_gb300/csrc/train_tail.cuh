@@ -7,8 +7,11 @@
 // launch and dependent loads on levels of a few hundred rows.  Here one CTA
 // keeps the levels' vectors in shared memory and steps with __syncthreads, the
 // matrices in its L1.  Every row is summed by as many lanes and in the same
-// order as in the launched passes, so both routes give the same bits (the loss
-// is one FP32-rounded number: another order would move it by its rounding).
+// order as in the launched passes, so the V-cycle, its adjoint and with them
+// the loss (one FP32-rounded number: another order would move it by its
+// rounding) keep their bits.  The sums of dL/dc run over this one CTA's threads
+// and over a level's sweeps before they are reduced, another order than the
+// launched passes'; in FP32 pairs or FP64 they agree to about 1e-14.
 // 12k-row mesh, three cycles: 739 -> 711 us a call; five-mesh training batch
 // 5104 -> 4966.  The line: with levels up to 512 rows in the one CTA 725 -> 738
 // us, up to 1024 rows 734 -> 745 (batch 5076 -> 5357): there the SMs that the
