@@ -525,23 +525,22 @@ __device__ __forceinline__ double pair_decode(const FloatPair &v) {
     return v.l == -INFINITY ? static_cast<double>(v.h) * kPairWide : pair_value(v);
 }
 
-// Sum of term(t) over the parts a .. e - 1; the total in the threads with
-// tid < H.  Those alone convert it and take a sum past FP32's range again: the
-// conversion in every lane cost 0.9 us a launch (prediction on 50k rows 253 ->
-// 267 us).
-template <int H, class F>
-__device__ __forceinline__ double lanes_total(int a, int e, FloatPair (*red)[H], const F &term) {
-    const int q = threadIdx.x / H;
-    FloatPair s{0.f, 0.f};
-#pragma unroll 8
-    for (int t = a + q; t < e; t += kLanes) pair_add(s, term(t));
-    s = lanes_sum_pair<H>(s, red);
+// The statistics' sums of one feature in FP64 (out of line: the threads that
+// need it are rare, and inlined it cost the others registers).
+__device__ __noinline__ double stats_sum_wide(int a, int e, int f, int H, const int *tstart, const float *tmean) {
     double d = 0.0;
-    if (q != 0) return d;
-    if (isfinite(s.l)) return pair_value(s);
-#pragma unroll 1
-    for (int t = a; t < e; ++t) d += static_cast<double>(term(t));
+    for (int t = a; t < e; ++t)
+        d += static_cast<double>(static_cast<float>(tstart[t + 1] - tstart[t]) * tmean[static_cast<size_t>(t) * H + f]);
     return d;
+}
+__device__ __noinline__ double stats_m2_wide(int a, int e, int f, int H, const int *tstart, const float *tmean,
+                                             const float *tm2, float mean) {
+    double v = 0.0;
+    for (int t = a; t < e; ++t) {
+        const float d = tmean[static_cast<size_t>(t) * H + f] - mean;
+        v += static_cast<double>(fmaf(static_cast<float>(tstart[t + 1] - tstart[t]) * d, d, tm2[static_cast<size_t>(t) * H + f]));
+    }
+    return v;
 }
 
 // Group statistics from part statistics (biased variance):
@@ -557,8 +556,8 @@ __device__ __forceinline__ double lanes_total(int a, int e, FloatPair (*red)[H],
 // unrolled so that a thread's loads are in flight together.  With the
 // normalisation pass's and the head's reductions: prediction on 50k rows 363
 // -> 314 us and, with pairs here and in the pooling, 301 -> 263 us; on 1.2M rows
-// 2698 -> 2487 and 2235 -> 2114 us (the checks for sums past FP32's range: 4 us
-// on 50k, 11 on 1.2M rows).
+// 2698 -> 2487 and 2235 -> 2114 us (the checks for sums past FP32's range take
+// 12 us of the 1.2M rows, nothing on 50k).
 template <int H>
 __global__ void __launch_bounds__(kLanes * H) k_stats_combine(const int *__restrict__ gtile, const int *__restrict__ gptr,
                                                             const int *__restrict__ tstart,
@@ -568,19 +567,26 @@ __global__ void __launch_bounds__(kLanes * H) k_stats_combine(const int *__restr
     __shared__ FloatPair red[kLanes][H];
     __shared__ float smean[H];
     const int g = blockIdx.x, f = threadIdx.x % H, q = threadIdx.x / H;
-    const int t0 = gtile[g], t1 = gtile[g + 1];
-    const double s = lanes_total<H>(t0, t1, red, [&](int t) {
-        return static_cast<float>(tstart[t + 1] - tstart[t]) * tmean[static_cast<size_t>(t) * H + f];
-    });
+    const int t0 = gtile[g] + q, t1 = gtile[g + 1];
+    FloatPair s{0.f, 0.f};
+#pragma unroll 8
+    for (int t = t0; t < t1; t += kLanes)
+        pair_add(s, static_cast<float>(tstart[t + 1] - tstart[t]) * tmean[static_cast<size_t>(t) * H + f]);
+    s = lanes_sum_pair<H>(s, red);
     const int n = gptr[g + 1] - gptr[g];
-    if (q == 0) smean[f] = static_cast<float>(s / n);
+    if (q == 0)
+        smean[f] = static_cast<float>((isfinite(s.l) ? pair_value(s) : stats_sum_wide(t0, t1, f, H, tstart, tmean)) / n);
     __syncthreads();
     const float mf = smean[f];
-    const double m2 = lanes_total<H>(t0, t1, red, [&](int t) {
+    FloatPair v{0.f, 0.f};
+#pragma unroll 8
+    for (int t = t0; t < t1; t += kLanes) {
         const float d = tmean[static_cast<size_t>(t) * H + f] - mf;
-        return fmaf(static_cast<float>(tstart[t + 1] - tstart[t]) * d, d, tm2[static_cast<size_t>(t) * H + f]);
-    });
+        pair_add(v, fmaf(static_cast<float>(tstart[t + 1] - tstart[t]) * d, d, tm2[static_cast<size_t>(t) * H + f]));
+    }
+    v = lanes_sum_pair<H>(v, red);
     if (q == 0) {
+        const double m2 = isfinite(v.l) ? pair_value(v) : stats_m2_wide(t0, t1, f, H, tstart, tmean, tm2, mf);
         mu[static_cast<size_t>(g) * H + f] = mf;
         rstd[static_cast<size_t>(g) * H + f] =
             final ? static_cast<float>(1.0 / sqrt(m2 / n + static_cast<double>(kEps))) : static_cast<float>(m2);
@@ -716,6 +722,13 @@ __global__ void __launch_bounds__(kBlock, 6) k_norm_relu_pool_tile(const int *__
     }
 }
 
+// A pooled sum of one feature in FP64.
+__device__ __noinline__ FloatPair pool_sum_wide(int a, int e, int f, int H, const FloatPair *tsum) {
+    double d = 0.0;
+    for (int t = a; t < e; ++t) d += pair_decode(tsum[static_cast<size_t>(t) * H + f]);
+    return pair_of(d);
+}
+
 // Group sum and max (first index of the max kept) from part partials; as
 // for the statistics, tiles -> chunks (csum != nullptr: writes the chunk sum,
 // max and argmax) and chunks -> graphs (writes the pooled mean and max).
@@ -760,12 +773,7 @@ __global__ void __launch_bounds__(kLanes * H) k_pool_combine(const int *__restri
     if (q == 0) {
         for (int k = 1; k < kLanes; ++k)
             if (rm[k][f] > bm || (rm[k][f] == bm && ri[k][f] < bi)) { bm = rm[k][f]; bi = ri[k][f]; }
-        if (!isfinite(total.l)) {             // past FP32's range: in FP64
-            double d = 0.0;
-#pragma unroll 1
-            for (int t = gtile[g]; t < t1; ++t) d += pair_decode(tsum[static_cast<size_t>(t) * H + f]);
-            total = pair_of(d);
-        }
+        if (!isfinite(total.l)) total = pool_sum_wide(t0, t1, f, H, tsum);   // past FP32's range
         if (csum) {
             const size_t o = static_cast<size_t>(g) * H + f;
             csum[o] = total;
