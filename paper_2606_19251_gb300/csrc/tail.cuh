@@ -47,8 +47,9 @@ constexpr size_t kTailSmem = 220 * 1024;         // shared memory a tail's level
 // with 0, 1, 2, ... V-cycles after them take no longer than with the levels one
 // by one (9k rows, amg_set_coeffs and one V-cycle: 139 us one by one, 381 with
 // the tail from 978 rows, 126 from 231 rows; FP64 168, 525, 167).  Jacobi's B
-// is formed with the hierarchy, where 0.1 to 0.3 ms stand beside 5 to 50 ms of
-// setup, and is not bounded there.
+// is formed with the hierarchy, where 0.1 to 0.5 ms stand beside 5 to 50 ms of
+// setup (1025^2 grid 45.5 -> 45.8 ms, 262k rows of a 3-D grid 28.2 -> 28.6), and
+// is not bounded there.
 constexpr double kTailWork = 4e6, kTailWork64 = 1.5e6;
 constexpr int kTailLongRows = 32;      // FP64: four lanes a row from this mean length on
 constexpr double kTailCoarseWork = 134217728.0;  // n_t n_L^2 bound: the FP64 coarsest solves of the n_t columns
