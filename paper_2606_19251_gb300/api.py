@@ -304,8 +304,8 @@ def amg_solve(ctx, b, x0=None, rtol=1e-8, max_iter=None):
     """Returns (status, x, history)."""
     b = np.ascontiguousarray(b, dtype=np.float64)
     x = np.zeros_like(b) if x0 is None else np.array(x0, dtype=np.float64, copy=True)
-    cap = (max_iter if max_iter is not None else 100000) + 1
-    hist = np.zeros(cap)
+    # the context's own max_iter (up to 100000) decides how many entries are written
+    hist = np.zeros(max(100000, max_iter or 0) + 1)
     nvc = C.c_int()
     rc = _check(ctx, lib().amg_solve(ctx, _dptr(b), _dptr(x), float(rtol), C.byref(nvc), _dptr(hist)),
                 SOLVE_STATUSES)
@@ -314,7 +314,7 @@ def amg_solve(ctx, b, x0=None, rtol=1e-8, max_iter=None):
 
 def amg_solve_device(ctx, d_b, d_x, rtol=1e-8, stream=None, hist_cap=100001):
     """Solve in place on device tensors; returns (status, history)."""
-    hist = np.zeros(hist_cap)
+    hist = np.zeros(max(100001, hist_cap))   # as in amg_solve
     nvc = C.c_int()
     rc = _check(ctx, lib().amg_solve_device(ctx, _dev(d_b), _dev(d_x), float(rtol), _stream(stream),
                                             C.byref(nvc), _dptr(hist)), SOLVE_STATUSES)

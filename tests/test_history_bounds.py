@@ -49,3 +49,24 @@ def test_probes_longer_than_max_iter(max_iter):
         finally:
             P.amg_destroy(ctx)
     assert out[0] == out[1]
+
+
+@pytest.mark.parametrize("call,kw", [("amg_solve", dict(max_iter=3)), ("amg_solve_device", dict(hist_cap=4)),
+                                     ("amg_solve", {}), ("amg_solve_device", {})])
+def test_binding_gives_room_for_any_history(monkeypatch, call, kw):
+    """The library writes one entry per cycle of the context's max_iter (at most
+    100000), whatever the caller expects: the buffer it gets holds them all."""
+    from paper_2606_19251_gb300 import api
+    sizes = []
+
+    class Lib:
+        def __getattr__(self, name):
+            return lambda *a: 0
+
+    monkeypatch.setattr(api, "lib", lambda: Lib())
+    monkeypatch.setattr(api, "_dev", lambda t: None)
+    monkeypatch.setattr(api, "_stream", lambda s: None)
+    monkeypatch.setattr(api, "_dptr", lambda a: sizes.append(a.size))
+    b = np.zeros(7)
+    api.amg_solve(None, b, **kw) if call == "amg_solve" else api.amg_solve_device(None, b, b, **kw)
+    assert max(sizes) == 100001
